@@ -101,6 +101,41 @@ struct PairClass {
 
 struct pcm_ctx_impl;
 
+// PCM_FP64 integrals (integrals64.cu): the points in tiles, the kept pairs of
+// all classes in sorted order, and the ESP pairs
+struct __align__(16) F64Pt {
+    double x, y, z, w;
+};
+struct F64Box {
+    double lo[3], inv;                     // lower corner, 1 / side of the cube around the cavity
+};
+struct F64Src {                            // kept pairs of the classes; first sorted position of each
+    const double *Px[6], *Py[6], *Pz[6], *p[6];
+    int off[7];
+};
+struct F64Int {
+    DBuf<double> tab;                      // Boys table (f64.cuh)
+    int ntile = 0;                         // tiles of 32 points
+    DBuf<int> pt_idx, pt_cls;              // per slot: point, exponent class
+    DBuf<F64Pt> pt_xyz;                    // per slot: coordinates, charge of the current call
+    DBuf<float4> pt_sph;                   // per tile: bounding sphere
+    int off[7] = {0, 0, 0, 0, 0, 0, 0};    // first sorted position of each class
+    DBuf<int> ord;                         // sorted position -> kept pair of its class
+    DBuf<double> P;                        // 4 x pairs: centre, exponent
+    DBuf<float4> info;                     // the same in FP32
+    bool use_rc = false;
+    DBuf<double2> rc;                      // exponent classes x pairs: rho, cn
+    DBuf<unsigned> key;
+    DBuf<int> val;
+    // ESP pairs of the last density test
+    DBuf<unsigned char> flag;
+    DBuf<int> list, pos;                   // sorted positions of the ESP pairs; pairs kept before each position
+    int eoff[7] = {0, 0, 0, 0, 0, 0, 0};   // first ESP pair of each class in list
+    size_t roff[6] = {0, 0, 0, 0, 0, 0};   // first record of each class in rec
+    DBuf<double> rec;
+    DBuf<double> S;                        // Fock accumulators per term
+};
+
 // Work of one thread block of the packed integral kernels, so that the blocks
 // of many molecules can run in one launch (batches).
 struct EspJob {
@@ -142,6 +177,10 @@ struct pcm_ctx {
     // Boys tables
     pcm::DBuf<double> boys64;
     pcm::DBuf<float> boys32;
+    // PCM_FP64 Fock and gradient integrals
+    pcm::F64Int f64;
+    pcm::DBuf<unsigned> sort_key;          // scratch of sort_pairs
+    pcm::DBuf<int> sort_val, sort_cnt;
 
     // molecule
     int natom = 0;
@@ -285,7 +324,17 @@ struct pcm_ctx {
 
 namespace pcm {
 // launchers implemented in the .cu files ------------------------------------
+void gauss_legendre(int n, std::vector<double> &x, std::vector<double> &w);
 int boys_build_tables(pcm_ctx *c);
+// stable radix sort of (key, value) pairs on the context's stream (sort.cu)
+int sort_pairs(pcm_ctx *c, int n, int bits, DBuf<unsigned> &key, DBuf<int> &val);
+// PCM_FP64 integrals (integrals64.cu)
+int f64_build_tables(pcm_ctx *c);
+int f64_prepare(pcm_ctx *c);
+int f64_esp_prepare(pcm_ctx *c, const double *dP);
+int f64_grad_point(pcm_ctx *c, const double *dq, double *gk);
+int f64_charges(pcm_ctx *c, const double *dq);
+int f64_w(pcm_ctx *c, int k, bool esp, double *W);
 int surface_build(pcm_ctx *c, int natom, const double *xyz, const double *Z, const double *radius, int n);
 int basis_build(pcm_ctx *c, int nshell, const int *shell_atom, const int *shell_l, const int *shell_nprim,
                 const double *exps, const double *coefs);

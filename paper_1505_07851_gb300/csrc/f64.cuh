@@ -1,0 +1,159 @@
+// FP64 pair-point interactions in few FP64 instructions.
+//
+// The FP64 pipe of this GPU issues 1.67 lanes per clock and SM (measured; 77
+// cycles per warp instruction and scheduler), so an FP64 integral kernel costs
+// its FP64 instructions and nothing else: loads, integer work and FP32 tests
+// hide behind them, and FP64 comparisons and conversions cost as much as an
+// FMA.  An interaction of a pair (exponent p, centre P) with a point (zeta, C)
+// is written in the form of farfield.cuh,
+//   sum_n b_n Q_n(X, Y, Z),  (X, Y, Z) = P - C,
+// with per-pair polynomials Q_n and
+//   far  (T = rho R^2 >= f64_far_T): b_n = R^-(2n+1),
+//   near:                            b_n = cn (2 rho)^n F_n(T) / (2n-1)!!,  cn = 2 sqrt(rho / pi)
+// (U / (sqrt(pi) / (2 sqrt(p))) = 2 sqrt(rho / pi)), so both forms share the
+// polynomials.  Beyond f64_far_T the two agree to below 1e-16 relative.
+#pragma once
+#include "common.cuh"
+#include "farfield.cuh"
+
+namespace pcm {
+
+// smallest T at which F_0..F_m equal their asymptotic forms to 1e-16 relative
+// (the neglected part of F_m is about e^-T 2^m T^(m-1/2) / ((2m-1)!! sqrt(pi)) of it)
+__host__ __device__ constexpr double f64_far_T(int m)
+{
+    return m == 0 ? 35.0 : (m == 1 ? 39.5 : (m == 2 ? 43.0 : (m == 3 ? 46.5 : (m == 4 ? 49.5 : 52.5))));
+}
+
+// Table of F_m(T) / (2m-1)!!, m = 0..5, at T_i = i / 256 as Taylor coefficients
+// in d = T - T_i (five terms: |d| <= 1/512, the next one is below 2^-55 of F_m):
+// per row and m six doubles, c0..c4 and a pad, so that a row is read in 16-byte
+// words.  1/256 instead of 1/32 costs 4 MB (resident in L2) and saves two FMAs
+// and the d / k scalings per F_m.
+constexpr int F64_MTOP = 5;
+constexpr int F64_INV_DT = 256;
+constexpr int F64_NROW = 54 * F64_INV_DT + 2;
+constexpr int F64_STRIDE = 6 * (F64_MTOP + 1);
+// adding 1.5 * 2^44 leaves round(256 T) in the low word of the sum
+constexpr double F64_MAGIC = 26388279066624.0;
+
+// b_n of the far form; 1/R from the hardware estimate (2^-20) and one
+// third-order step: r0 (1 + e/2 + 3 e^2/8), e = 1 - R^2 r0^2, error 5 e^3 / 16 < 2^-58
+template <int L>
+__device__ __forceinline__ void f64_far(double R2, double (&b)[L + 1])
+{
+    double r0;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r0) : "d"(R2));
+    const double e = fma(-R2 * r0, r0, 1.0);
+    const double rs = fma(r0 * e, fma(e, 0.375, 0.5), r0);
+    b[0] = rs;
+    if constexpr (L > 0) {
+        const double rs2 = rs * rs;
+#pragma unroll
+        for (int n = 1; n <= L; ++n) b[n] = b[n - 1] * rs2;
+    }
+}
+
+// b_n of the near form; lanes without `use` read row 0 and return garbage
+template <int L>
+__device__ __forceinline__ void f64_near(double R2, double rho, double cn, bool use, const double *__restrict__ tab,
+                                         double (&b)[L + 1])
+{
+    const double t = fma(rho, R2, F64_MAGIC);
+    const int i = use ? __double2loint(t) : 0;
+    const double d = fma(rho, R2, F64_MAGIC - t);
+    const double2 *row = reinterpret_cast<const double2 *>(tab + (size_t)i * F64_STRIDE);
+    double f = cn;
+#pragma unroll
+    for (int n = 0; n <= L; ++n) {
+        const double2 c01 = __ldg(row + 3 * n), c23 = __ldg(row + 3 * n + 1);
+        const double c4 = __ldg(reinterpret_cast<const double *>(row + 3 * n + 2));
+        const double F = fma(fma(fma(fma(c4, d, c23.y), d, c23.x), d, c01.y), d, c01.x);
+        if (n > 0) f *= rho + rho;
+        b[n] = f * F;
+    }
+}
+
+// monomials X^a Y^b Z^c of degree 1..L in Hermite index order (mono[0] unused)
+template <int L>
+__device__ __forceinline__ void f64_monomials(double X, double Y, double Z, double (&mono)[nherm(L)])
+{
+    constexpr MonoTab MT = mono_tab(L);
+    if constexpr (L > 0) {
+        mono[1] = X;
+        mono[2] = Y;
+        mono[3] = Z;
+#pragma unroll
+        for (int i = 4; i < nherm(L); ++i) {
+            const int a = MT.a[i], b = MT.b[i], c = MT.c[i];
+            if (a > 0)
+                mono[i] = mono[hidx(a - 1, b, c)] * X;
+            else if (b > 0)
+                mono[i] = mono[hidx(a, b - 1, c)] * Y;
+            else
+                mono[i] = mono[hidx(a, b, c - 1)] * Z;
+        }
+    }
+}
+
+// acc[d] += d/dP_d of sum_n b_n Q_n (coefficients G: the terms of farfield.cuh),
+// with b_0..b_{L+1}: both forms have d b_n / dX = -(2n + 1) X b_{n+1}
+template <int L>
+__device__ __forceinline__ void f64_dot_grad(double X, double Y, double Z, const double (&b)[L + 2],
+                                             const double (&G)[far_nterms(L)], double (&acc)[3])
+{
+    constexpr FarTerms FT = far_terms(L);
+    double S = b[1] * G[0];
+    if constexpr (L > 0) {
+        double mono[nherm(L)];
+        f64_monomials<L>(X, Y, Z, mono);
+        mono[0] = 1.0;
+#pragma unroll
+        for (int n = 1; n <= L; ++n) {
+            double Q = 0.0, D[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+            for (int k = 1; k < far_nterms(L); ++k) {
+                if (FT.n[k] != n) continue;
+                const int e[3] = {FT.a[k], FT.b[k], FT.c[k]};
+                if (e[0] + e[1] + e[2] == 0) {
+                    Q += G[k];
+                    continue;
+                }
+                Q = fma(G[k], mono[hidx(e[0], e[1], e[2])], Q);
+#pragma unroll
+                for (int d = 0; d < 3; ++d)
+                    if (e[d] > 0) {
+                        const double g = e[d] > 1 ? (double)e[d] * G[k] : G[k];
+                        const int h = hidx(e[0] - (d == 0), e[1] - (d == 1), e[2] - (d == 2));
+                        D[d] = h == 0 ? D[d] + g : fma(g, mono[h], D[d]);
+                    }
+            }
+            S = fma((double)(2 * n + 1) * b[n + 1], Q, S);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) acc[d] = fma(b[n], D[d], acc[d]);
+        }
+    }
+    acc[0] = fma(-X, S, acc[0]);
+    acc[1] = fma(-Y, S, acc[1]);
+    acc[2] = fma(-Z, S, acc[2]);
+}
+
+// S[k] += b_n X^a Y^b Z^c for every term k = (n; a, b, c)
+template <int L>
+__device__ __forceinline__ void f64_accumulate(double X, double Y, double Z, const double (&b)[L + 1],
+                                               double (&S)[far_nterms(L)])
+{
+    constexpr FarTerms FT = far_terms(L);
+    S[0] += b[0];
+    if constexpr (L > 0) {
+        double mono[nherm(L)];
+        f64_monomials<L>(X, Y, Z, mono);
+#pragma unroll
+        for (int k = 1; k < far_nterms(L); ++k) {
+            const int h = hidx(FT.a[k], FT.b[k], FT.c[k]);
+            S[k] = h == 0 ? S[k] + b[FT.n[k]] : fma(b[FT.n[k]], mono[h], S[k]);
+        }
+    }
+}
+
+}  // namespace pcm

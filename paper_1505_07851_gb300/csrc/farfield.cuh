@@ -40,7 +40,7 @@ __host__ __device__ constexpr int far_nterms(int L)
 }
 
 struct FarTerms {
-    int n[64], a[64], b[64], c[64];
+    int n[80], a[80], b[80], c[80];
     int count;
 };
 

@@ -246,85 +246,6 @@ __global__ void esp_reduce_kernel(int M, int nseg, const double *__restrict__ pa
     c[k] = s;
 }
 
-// ---------------------------------------------------------------------------
-// Fock main kernel: one thread per primitive pair, looping over the points of
-// its split in exponent-class order, staged in shared memory tiles of TQ.
-// W[split][h][pair] = sum_k q_k U_k R_h(rho_k, P - C_k)
-// ---------------------------------------------------------------------------
-constexpr int FOCK_NT = 128;
-constexpr int FOCK_TQ = 128;
-
-template <int L>
-__global__ void __launch_bounds__(FOCK_NT) fock_kernel_f64(int npair, const double *__restrict__ gPx,
-                                                           const double *__restrict__ gPy,
-                                                           const double *__restrict__ gPz,
-                                                           const double *__restrict__ gp, int ksplit,
-                                                           const double *__restrict__ px, const double *__restrict__ py,
-                                                           const double *__restrict__ pz, const double *__restrict__ q,
-                                                           int M, int ncls, const int *__restrict__ cls_off,
-                                                           const double *__restrict__ cls_zeta,
-                                                           const double *__restrict__ boys, double *__restrict__ W)
-{
-    constexpr int NH = nherm(L);
-    __shared__ double sx[FOCK_TQ], sy[FOCK_TQ], sz[FOCK_TQ], sq[FOCK_TQ];
-    const int r = blockIdx.x * FOCK_NT + threadIdx.x;
-    const bool active = r < npair;
-    const int rr = active ? r : 0;
-    const double Px = gPx[rr], Py = gPy[rr], Pz = gPz[rr], p = gp[rr];
-    const int ka = blockIdx.y * ksplit;
-    const int kb = min(M, ka + ksplit);
-    double w[NH];
-#pragma unroll
-    for (int h = 0; h < NH; ++h) w[h] = 0.0;
-    for (int ec = 0; ec < ncls; ++ec) {
-        const int a = max(ka, cls_off[ec]), b = min(kb, cls_off[ec + 1]);
-        if (a >= b) continue;
-        const double zz = cls_zeta[ec];
-        const double z2 = zz * zz;
-        const double inv = 1.0 / (p + z2);
-        const double rho = p * z2 * inv;
-        const double U = sqrt(z2 * inv);
-        const double m2r = -2.0 * rho;
-        for (int t0 = a; t0 < b; t0 += FOCK_TQ) {
-            const int nt = min(FOCK_TQ, b - t0);
-            __syncthreads();
-            for (int t = threadIdx.x; t < nt; t += FOCK_NT) {
-                sx[t] = px[t0 + t];
-                sy[t] = py[t0 + t];
-                sz[t] = pz[t0 + t];
-                sq[t] = q[t0 + t];
-            }
-            __syncthreads();
-            for (int kk = 0; kk < nt; ++kk) {
-                const double X = Px - sx[kk], Y = Py - sy[kk], Z = Pz - sz[kk];
-                const double T = rho * (X * X + Y * Y + Z * Z);
-                double F[L + 1];
-                boys_eval<L>(T, boys, F);
-                const double sc = sq[kk] * U;
-                if constexpr (L == 0) {
-                    w[0] = fma(sc, F[0], w[0]);
-                } else {
-                    double Rn[L + 1];
-                    double f = sc;
-#pragma unroll
-                    for (int n = 0; n <= L; ++n) {
-                        Rn[n] = f * F[n];
-                        f *= m2r;
-                    }
-                    double R[NH];
-                    hermite_R<L, double>(X, Y, Z, Rn, R);
-#pragma unroll
-                    for (int h = 0; h < NH; ++h) w[h] += R[h];
-                }
-            }
-        }
-    }
-    if (active) {
-#pragma unroll
-        for (int h = 0; h < NH; ++h) W[((size_t)blockIdx.y * NH + h) * npair + r] = w[h];
-    }
-}
-
 // Fock epilogue: one thread per shell pair.  For each kept primitive pair of
 // the shell pair, L_ab = -(2 pi/p) K sum_tuv E^{ab}_tuv W_tuv is contracted
 // with c_a c_b (Eq. 16) and summed in pair order (Eq. 17).  A diagonal shell
@@ -405,121 +326,10 @@ __global__ void fock_epilogue_kernel(int nsp, int npair, int nsplit, const int *
 // Each integral [a|J_k|b] depends on the centre of a, the centre of b and the
 // point r_k, which moves with its atom.
 //
-// Point part (gc of Eq. 22): d/dC R_tuv(P - C) = -R_{t+1,u,v} (and y, z), so
-//   d c_k / dC_k = -sum_pairs U sum_tuv eD_tuv R_{tuv + 1_d}
-// with the ESP pairs' density coefficients eD (t+u+v <= L) and R up to L+1.
-// One thread per point as in the ESP kernel; three sums per point.
-// ---------------------------------------------------------------------------
-template <int L>
-__global__ void __launch_bounds__(ESP_NT) esp_grad_kernel(int nesp, int seglen, const double *__restrict__ eP,
-                                                          const double *__restrict__ eD,
-                                                          const int *__restrict__ blk_off,
-                                                          const double *__restrict__ px, const double *__restrict__ py,
-                                                          const double *__restrict__ pz, const int *__restrict__ pcls,
-                                                          const double *__restrict__ cls_zeta,
-                                                          const double *__restrict__ boys, int M,
-                                                          double *__restrict__ part)
-{
-    constexpr int NH = nherm(L);
-    constexpr int L1 = L + 1;
-    constexpr int NH1 = nherm(L1);
-    __shared__ double sP[4][ESP_TP];
-    __shared__ double sD[NH][ESP_TP];
-    __shared__ double sRho[ESP_MAXCB][ESP_TP];
-    __shared__ double sU[ESP_MAXCB][ESP_TP];
-
-    const int k0 = blk_off[blockIdx.x], k1 = blk_off[blockIdx.x + 1];
-    const int cmin = pcls[k0];
-    const int ncb = pcls[k1 - 1] - cmin + 1;
-    const int j0 = blockIdx.y * seglen;
-    const int j1 = min(nesp, j0 + seglen);
-
-    double x[ESP_PPT], y[ESP_PPT], z[ESP_PPT], gx[ESP_PPT], gy[ESP_PPT], gz[ESP_PPT];
-    int e[ESP_PPT];
-    bool on[ESP_PPT];
-#pragma unroll
-    for (int q = 0; q < ESP_PPT; ++q) {
-        const int k = k0 + threadIdx.x + q * ESP_NT;
-        on[q] = k < k1;
-        const int kk = on[q] ? k : k0;
-        x[q] = px[kk];
-        y[q] = py[kk];
-        z[q] = pz[kk];
-        e[q] = pcls[kk] - cmin;
-        gx[q] = gy[q] = gz[q] = 0.0;
-    }
-
-    for (int jt = j0; jt < j1; jt += ESP_TP) {
-        const int nt = min(ESP_TP, j1 - jt);
-        __syncthreads();
-        for (int t = threadIdx.x; t < 4 * ESP_TP; t += ESP_NT) {
-            const int f = t / ESP_TP, jj = t % ESP_TP;
-            sP[f][jj] = jj < nt ? eP[(size_t)f * nesp + jt + jj] : 1.0;
-        }
-        for (int t = threadIdx.x; t < NH * ESP_TP; t += ESP_NT) {
-            const int h = t / ESP_TP, jj = t % ESP_TP;
-            sD[h][jj] = jj < nt ? eD[(size_t)h * nesp + jt + jj] : 0.0;
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < ncb * ESP_TP; t += ESP_NT) {
-            const int ec = t / ESP_TP, jj = t % ESP_TP;
-            const double zz = cls_zeta[cmin + ec];
-            const double z2 = zz * zz;
-            const double p = sP[3][jj];
-            const double inv = 1.0 / (p + z2);
-            sRho[ec][jj] = p * z2 * inv;
-            sU[ec][jj] = sqrt(z2 * inv);
-        }
-        __syncthreads();
-        for (int jj = 0; jj < nt; ++jj) {
-            const double Px = sP[0][jj], Py = sP[1][jj], Pz = sP[2][jj];
-#pragma unroll
-            for (int q = 0; q < ESP_PPT; ++q) {
-                const double rho = sRho[e[q]][jj];
-                const double X = Px - x[q], Y = Py - y[q], Z = Pz - z[q];
-                const double T = rho * (X * X + Y * Y + Z * Z);
-                double F[L1 + 1];
-                boys_eval<L1>(T, boys, F);
-                double Rn[L1 + 1];
-                double m2r = -2.0 * rho, f = 1.0;
-#pragma unroll
-                for (int n = 0; n <= L1; ++n) {
-                    Rn[n] = f * F[n];
-                    f *= m2r;
-                }
-                double R[NH1];
-                hermite_R<L1, double>(X, Y, Z, Rn, R);
-                double sx = 0.0, sy = 0.0, sz = 0.0;
-#pragma unroll
-                for (int t = 0; t <= L; ++t)
-#pragma unroll
-                    for (int u = 0; u <= L - t; ++u)
-#pragma unroll
-                        for (int v = 0; v <= L - t - u; ++v) {
-                            const double d = sD[hidx(t, u, v)][jj];
-                            sx = fma(d, R[hidx(t + 1, u, v)], sx);
-                            sy = fma(d, R[hidx(t, u + 1, v)], sy);
-                            sz = fma(d, R[hidx(t, u, v + 1)], sz);
-                        }
-                const double U = sU[e[q]][jj];
-                gx[q] = fma(U, sx, gx[q]);
-                gy[q] = fma(U, sy, gy[q]);
-                gz[q] = fma(U, sz, gz[q]);
-            }
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < ESP_PPT; ++q) {
-        const int k = k0 + threadIdx.x + q * ESP_NT;
-        if (on[q]) {
-            part[((size_t)blockIdx.y * 3 + 0) * M + k] = gx[q];
-            part[((size_t)blockIdx.y * 3 + 1) * M + k] = gy[q];
-            part[((size_t)blockIdx.y * 3 + 2) * M + k] = gz[q];
-        }
-    }
-}
-
-// g[d][k] += -q_k sum over segments of the point-part sums, in segment order
+// The point part's kernels (gc of Eq. 22: d/dC R_tuv(P - C) = -R_{t+1,u,v} and
+// y, z) are in integrals64.cu and integrals_mixed.cu; here its reduction for
+// PCM_MIXED: g[d][k] += -q_k sum over segments of the point-part sums, in
+// segment order
 __global__ void grad_point_reduce_kernel(int M, int nseg, const double *__restrict__ part,
                                          const double *__restrict__ q, double *__restrict__ g)
 {
@@ -834,6 +644,10 @@ int esp_compute(pcm_ctx *c, const double *dP, double *dc)
     return esp_class_stats(c);
 }
 
+// the FP32 Fock kernels' threads per block and points per tile
+constexpr int FOCK_NT = 128;
+constexpr int FOCK_TQ = 128;
+
 // points of each split and the number of splits for a Fock launch of nb
 // pair blocks: enough CTAs to fill the GPU, splits on whole point tiles
 static void fock_split(pcm_ctx *c, int nb, int *nsplit, int *ks)
@@ -936,10 +750,11 @@ static int fock_class(pcm_ctx *c, PairClass &pc, const double *dq, double *ddF)
         const bool mixed = c->opt.precision == PCM_MIXED;
         const int k = kk;
         if (mixed && c->opt.autotune) PCM_TRY(fock_tune(c, k, L, dq));
-        const int npt = mixed ? fock_mixed_pairs_per_thread(c, L, pc.npair) : 1;
-        const int nb = (pc.npair + FOCK_NT * npt - 1) / (FOCK_NT * npt);
-        int ks;
-        fock_split(c, nb, &nsplit, &ks);
+        int npt = 1, ks = 0;
+        if (mixed) {
+            npt = fock_mixed_pairs_per_thread(c, L, pc.npair);
+            fock_split(c, (pc.npair + FOCK_NT * npt - 1) / (FOCK_NT * npt), &nsplit, &ks);
+        }
         if (defer) {
             PCM_TRY(c->fock_Wk[k].alloc((size_t)nsplit * NH * pc.npair));
             PCM_TRY(fock_mixed_class(c, k, dq, nsplit, ks, c->fock_Wk[k].p, npt));
@@ -949,17 +764,11 @@ static int fock_class(pcm_ctx *c, PairClass &pc, const double *dq, double *ddF)
             return PCM_OK;
         }
         PCM_TRY(c->fock_W.alloc((size_t)nsplit * NH * pc.npair));
-        dim3 grid(nb, nsplit);
         if (c->have_events) PCM_CUDA(cudaEventRecord(c->ev_a[6 + k], c->stream));
-        if (mixed) {
+        if (mixed)
             PCM_TRY(fock_mixed_class(c, k, dq, nsplit, ks, c->fock_W.p, npt));
-        } else {
-            fock_kernel_f64<L><<<grid, FOCK_NT, 0, c->stream>>>(pc.npair, pc.Px.p, pc.Py.p, pc.Pz.p, pc.p.p, ks,
-                                                                 c->px.p, c->py.p, c->pz.p, dq, c->M, c->ncls,
-                                                                 c->cls_off.p, c->cls_zeta.p, c->boys64.p,
-                                                                 c->fock_W.p);
-            PCM_LAUNCHED(c);
-        }
+        else
+            PCM_TRY(f64_w(c, k, false, c->fock_W.p));
         if (c->have_events) PCM_CUDA(cudaEventRecord(c->ev_b[6 + k], c->stream));
     }
     if (defer) {
@@ -978,6 +787,7 @@ static int fock_class(pcm_ctx *c, PairClass &pc, const double *dq, double *ddF)
 int fock_compute(pcm_ctx *c, const double *dq, double *ddF)
 {
     c->stats.integrals_fock = 0.0;
+    if (c->opt.precision == PCM_FP64) PCM_TRY(f64_charges(c, dq));
     PCM_TRY((fock_class<0, 0>(c, c->cls[0], dq, ddF)));
     PCM_TRY((fock_class<1, 0>(c, c->cls[1], dq, ddF)));
     PCM_TRY((fock_class<1, 1>(c, c->cls[2], dq, ddF)));
@@ -1029,16 +839,6 @@ static int pair_csr(pcm_ctx *c, PairClass &pc)
     return PCM_OK;
 }
 
-template <int L>
-static void launch_esp_grad(pcm_ctx *c, PairClass &pc, const int *blk, int nblk, int seg_base, int nseg_cls,
-                            int seglen)
-{
-    dim3 grid(nblk, nseg_cls);
-    esp_grad_kernel<L><<<grid, ESP_NT, 0, c->stream>>>(pc.nesp, seglen, pc.eP.p, pc.eD.p, blk, c->px.p, c->py.p,
-                                                        c->pz.p, c->pcls.p, c->cls_zeta.p, c->boys64.p, c->M,
-                                                        c->esp_part.p + (size_t)seg_base * 3 * c->M);
-}
-
 template <int LA, int LB>
 static int grad_pair_class(pcm_ctx *c, PairClass &pc, const double *dP, const double *dq, double *gpair)
 {
@@ -1046,20 +846,17 @@ static int grad_pair_class(pcm_ctx *c, PairClass &pc, const double *dP, const do
     constexpr int NH1 = nherm(L1);
     if (pc.nesp == 0) return PCM_OK;
     const int n = pc.nesp;
-    const int npt = c->opt.precision == PCM_MIXED ? fock_mixed_pairs_per_thread(c, L1, n) : 1;
-    const int nb = (n + FOCK_NT * npt - 1) / (FOCK_NT * npt);
-    int nsplit, ks;
-    fock_split(c, nb, &nsplit, &ks);
-    PCM_TRY(c->fock_W.alloc((size_t)nsplit * NH1 * n));
+    const int k = (int)(&pc - c->cls);
+    int nsplit = 1;
     if (c->opt.precision == PCM_MIXED) {
-        PCM_TRY(grad_w_mixed(c, (int)(&pc - c->cls), dq, nsplit, ks, c->fock_W.p, npt));
+        const int npt = fock_mixed_pairs_per_thread(c, L1, n);
+        int ks;
+        fock_split(c, (n + FOCK_NT * npt - 1) / (FOCK_NT * npt), &nsplit, &ks);
+        PCM_TRY(c->fock_W.alloc((size_t)nsplit * NH1 * n));
+        PCM_TRY(grad_w_mixed(c, k, dq, nsplit, ks, c->fock_W.p, npt));
     } else {
-        dim3 grid(nb, nsplit);
-        fock_kernel_f64<L1><<<grid, FOCK_NT, 0, c->stream>>>(n, pc.eP.p, pc.eP.p + n, pc.eP.p + 2 * (size_t)n,
-                                                              pc.eP.p + 3 * (size_t)n, ks, c->px.p, c->py.p, c->pz.p,
-                                                              dq, c->M, c->ncls, c->cls_off.p, c->cls_zeta.p,
-                                                              c->boys64.p, c->fock_W.p);
-        PCM_LAUNCHED(c);
+        PCM_TRY(c->fock_W.alloc((size_t)NH1 * n));
+        PCM_TRY(f64_w(c, k, true, c->fock_W.p));
     }
     PCM_TRY(c->g_full.alloc(6 * (size_t)pc.npair));
     PCM_CUDA(cudaMemsetAsync(c->g_full.p, 0, 6 * (size_t)pc.npair * sizeof(double), c->stream));
@@ -1092,12 +889,13 @@ static int grad_pair_all(pcm_ctx *c, const double *dP, const double *dq, double 
 // the per-pair contraction and every reduction in FP64.
 int grad_integrals(pcm_ctx *c, const double *dP, const double *dq, double *gk, double *gpair)
 {
-    PCM_TRY(esp_prepare_all(c, dP));
-    if (c->opt.precision == PCM_MIXED) {
-        double ints = 0.0;
-        for (int k = 0; k < 6; ++k)
-            ints += (double)c->cls[k].nesp * ncart(c->cls[k].la) * ncart(c->cls[k].lb) * c->M;
-        c->stats.integrals_grad = 2.0 * ints;
+    const bool mixed = c->opt.precision == PCM_MIXED;
+    PCM_TRY(mixed ? esp_prepare_all(c, dP) : f64_esp_prepare(c, dP));
+    double ints = 0.0;
+    for (int k = 0; k < 6; ++k)
+        ints += (double)c->cls[k].nesp * ncart(c->cls[k].la) * ncart(c->cls[k].lb) * c->M;
+    c->stats.integrals_grad = 2.0 * ints;
+    if (mixed) {
         int total = 0;
         PCM_TRY(grad_point_mixed(c, &total));
         if (total > 0) {
@@ -1105,49 +903,9 @@ int grad_integrals(pcm_ctx *c, const double *dP, const double *dq, double *gk, d
                                                                                   gk);
             PCM_LAUNCHED(c);
         }
-        return grad_pair_all(c, dP, dq, gpair);
-    }
-    std::vector<int> off;
-    esp_blocks(c, off);
-    const int nblk = (int)off.size() - 1;
-    DBuf<int> &blk = c->si[5];
-    PCM_TRY(blk.alloc(off.size()));
-    PCM_CUDA(cudaMemcpyAsync(blk.p, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-    int nseg[6], seglen[6], total = 0;
-    double ints = 0.0;
-    for (int k = 0; k < 6; ++k) {
-        PairClass &pc = c->cls[k];
-        nseg[k] = seglen[k] = 0;
-        if (pc.nesp == 0) continue;
-        ints += (double)pc.nesp * ncart(pc.la) * ncart(pc.lb) * c->M;
-        const int maxseg = (pc.nesp + ESP_TP - 1) / ESP_TP;
-        int ns = std::max(1, std::min(maxseg, (target_ctas(c) + nblk - 1) / nblk));
-        int sl = (pc.nesp + ns - 1) / ns;
-        sl = (sl + ESP_TP - 1) / ESP_TP * ESP_TP;
-        nseg[k] = (pc.nesp + sl - 1) / sl;
-        seglen[k] = sl;
-        total += nseg[k];
-    }
-    c->stats.integrals_grad = 2.0 * ints;
-    if (total > 0) {
-        PCM_TRY(c->esp_part.alloc((size_t)total * 3 * c->M));
-        int base = 0;
-        static const int LSUM[6] = {0, 1, 2, 2, 3, 4};
-        for (int k = 0; k < 6; ++k) {
-            PairClass &pc = c->cls[k];
-            if (nseg[k] == 0) continue;
-            switch (LSUM[k]) {
-            case 0: launch_esp_grad<0>(c, pc, blk.p, nblk, base, nseg[k], seglen[k]); break;
-            case 1: launch_esp_grad<1>(c, pc, blk.p, nblk, base, nseg[k], seglen[k]); break;
-            case 2: launch_esp_grad<2>(c, pc, blk.p, nblk, base, nseg[k], seglen[k]); break;
-            case 3: launch_esp_grad<3>(c, pc, blk.p, nblk, base, nseg[k], seglen[k]); break;
-            case 4: launch_esp_grad<4>(c, pc, blk.p, nblk, base, nseg[k], seglen[k]); break;
-            }
-            PCM_LAUNCHED(c);
-            base += nseg[k];
-        }
-        grad_point_reduce_kernel<<<(c->M + 255) / 256, 256, 0, c->stream>>>(c->M, total, c->esp_part.p, dq, gk);
-        PCM_LAUNCHED(c);
+    } else {
+        PCM_TRY(f64_grad_point(c, dq, gk));
+        PCM_TRY(f64_charges(c, dq));
     }
     return grad_pair_all(c, dP, dq, gpair);
 }

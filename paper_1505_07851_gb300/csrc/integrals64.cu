@@ -1,0 +1,866 @@
+// PCM_FP64 Fock correction and gradient integrals (the interactions are those of
+// f64.cuh; the potentials, which feed the linear solve, are in integrals.cu).
+//
+// Work is laid out for warps, because the FP64 pipe bounds every kernel here
+// and a warp instruction that serves few lanes costs as much as a full one:
+//   - the points in tiles of 32 that lie together (consecutive along a Hilbert
+//     curve, ordered by exponent class within a tile);
+//   - the primitive pairs of a class sorted by cell (the same curve) and, within
+//     a cell, by exponent, so that a warp's pairs have the same reach.
+// A tile's bounding sphere then tells, in a few FP32 instructions, whether a
+// pair is beyond f64_far_T for all of the tile's points.  The gradient's point
+// part runs a warp per point tile (a lane per point) over the pairs, the Fock
+// accumulation a warp per 32 pairs (a lane per pair) over the point tiles.
+// Against kernels with a seven-term Taylor step, the Hermite recurrence and FP64
+// branches per interaction (25 / 41 FP64 instructions for ss / ps pairs; here 12 /
+// 19 far and 16 / 27 near): Fock correction of a 150-atom s/sp cluster (6566 points)
+// 72.1 -> 42.2 ms, gradient of a 100-atom s/p/d cluster 109.9 -> 68.3 ms.
+#include <math.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "common.cuh"
+#include "context.h"
+#include "f64.cuh"
+
+namespace pcm {
+
+constexpr int F64_LSUM[6] = {0, 1, 2, 2, 3, 4};
+constexpr int F64_HBITS = 5;              // cells per side of the pairs' grid: 2^5
+constexpr int F64_PBITS = 4;              // exponent bins within a cell
+constexpr int F64_PTBITS = 6;             // cells per side of the points' grid
+constexpr int F64_SORT_MIN = 4096;        // fewer pairs than this stay in kept order, fewer points than a quarter too
+constexpr int F64_RC_CLASSES = 16;        // up to this many exponent classes rho and cn are tabulated per (class, pair)
+// thread blocks that a launch aims at: two waves of 8 per SM, so that unequal blocks even out
+constexpr int F64_CTAS = 152 * 16;
+
+__device__ inline double f64_comp_factor(int l, int c)
+{
+    return l == 2 && (c == 1 || c == 2 || c == 4) ? 1.7320508075688772935 : 1.0;
+}
+
+// ESP pair record: P, then the coefficients of f64_dot, padded to 16 bytes
+__host__ __device__ constexpr int f64_rec(int L) { return (3 + far_nterms(L) + 1) / 2 * 2; }
+
+// ---------------------------------------------------------------------------
+// table of F_m / (2m-1)!! (f64.cuh): one warp per row, F_9 by quadrature (the
+// lanes share the nodes), the others by downward recursion
+// ---------------------------------------------------------------------------
+constexpr int F64_GL = 24;
+constexpr int F64_PANELS = 16;
+
+__global__ void f64_table_kernel(const double *__restrict__ gx, const double *__restrict__ gw,
+                                 double *__restrict__ tab)
+{
+    const int row = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (row >= F64_NROW) return;
+    constexpr int TOP = F64_MTOP + 4;
+    const double T = (double)row / F64_INV_DT;
+    double s = 0.0;
+    for (int k = lane; k < F64_GL * F64_PANELS; k += 32) {
+        const double u = ((double)(k / F64_GL) + 0.5 * (gx[k % F64_GL] + 1.0)) / F64_PANELS;
+        const double u2 = u * u;
+        double w = 0.5 * gw[k % F64_GL] / F64_PANELS;
+        for (int j = 0; j < TOP; ++j) w *= u2;
+        s = fma(w, exp(-T * u2), s);
+    }
+    s = warp_sum(s);
+    double F[TOP + 1];
+    F[TOP] = s;
+    const double eT = exp(-T);
+#pragma unroll
+    for (int m = TOP; m > 0; --m) F[m - 1] = fma(2.0 * T, F[m], eT) / (double)(2 * m - 1);
+    if (lane != 0) return;
+    double df = 1.0;
+#pragma unroll
+    for (int m = 0; m <= F64_MTOP; ++m) {
+        if (m > 1) df *= (double)(2 * m - 1);
+        double *c = tab + (size_t)row * F64_STRIDE + 6 * m;
+        c[0] = F[m] / df;
+        c[1] = -F[m + 1] / df;
+        c[2] = F[m + 2] / (2.0 * df);
+        c[3] = -F[m + 3] / (6.0 * df);
+        c[4] = F[m + 4] / (24.0 * df);
+        c[5] = 0.0;
+    }
+}
+
+int f64_build_tables(pcm_ctx *c)
+{
+    std::vector<double> x, w;
+    gauss_legendre(F64_GL, x, w);
+    DBuf<double> g;
+    PCM_TRY(g.alloc(2 * F64_GL));
+    PCM_CUDA(cudaMemcpyAsync(g.p, x.data(), F64_GL * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+    PCM_CUDA(cudaMemcpyAsync(g.p + F64_GL, w.data(), F64_GL * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+    PCM_TRY(c->f64.tab.alloc((size_t)F64_NROW * F64_STRIDE));
+    f64_table_kernel<<<(F64_NROW + 3) / 4, 128, 0, c->stream>>>(g.p, g.p + F64_GL, c->f64.tab.p);
+    PCM_LAUNCHED(c);
+    PCM_CUDA(cudaStreamSynchronize(c->stream));  // g is freed on return
+    return PCM_OK;
+}
+
+// ---------------------------------------------------------------------------
+// orders: a Hilbert curve over a cubic grid (Skilling, AIP Conf. Proc. 707, 381
+// (2004): axes to transposed index by Gray decoding of the exchanged bits)
+// ---------------------------------------------------------------------------
+template <int BITS>
+__device__ __forceinline__ unsigned hilbert3(unsigned x, unsigned y, unsigned z)
+{
+    unsigned X[3] = {x, y, z};
+    for (unsigned q = 1u << (BITS - 1); q > 1; q >>= 1) {
+        const unsigned p = q - 1;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            if (X[i] & q) {
+                X[0] ^= p;
+            } else {
+                const unsigned t = (X[0] ^ X[i]) & p;
+                X[0] ^= t;
+                X[i] ^= t;
+            }
+        }
+    }
+    X[1] ^= X[0];
+    X[2] ^= X[1];
+    unsigned t = 0;
+    for (unsigned q = 1u << (BITS - 1); q > 1; q >>= 1)
+        if (X[2] & q) t ^= q - 1;
+    unsigned h = 0;
+    for (int b = BITS - 1; b >= 0; --b)
+        for (int i = 0; i < 3; ++i) h = (h << 1) | (((X[i] ^ t) >> b) & 1u);
+    return h;
+}
+
+template <int BITS>
+__device__ __forceinline__ unsigned curve_key(double x, double y, double z, const F64Box &b)
+{
+    const int top = (1 << BITS) - 1;
+    const double s = (double)(1 << BITS) * b.inv;
+    const int i = min(max((int)((x - b.lo[0]) * s), 0), top);
+    const int j = min(max((int)((y - b.lo[1]) * s), 0), top);
+    const int k = min(max((int)((z - b.lo[2]) * s), 0), top);
+    return hilbert3<BITS>(i, j, k);
+}
+
+__global__ void f64_point_key_kernel(int M, const double *__restrict__ px, const double *__restrict__ py,
+                                     const double *__restrict__ pz, F64Box box, unsigned *__restrict__ key,
+                                     int *__restrict__ val)
+{
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= M) return;
+    key[k] = curve_key<F64_PTBITS>(px[k], py[k], pz[k], box);
+    val[k] = k;
+}
+
+// one warp per tile of 32 points: order by class, gather, bounding sphere
+__global__ void f64_point_tile_kernel(int M, const int *__restrict__ val, const double *__restrict__ px,
+                                      const double *__restrict__ py, const double *__restrict__ pz,
+                                      const int *__restrict__ pcls, int *__restrict__ idx, int *__restrict__ cls,
+                                      F64Pt *__restrict__ xyz, float4 *__restrict__ sph)
+{
+    const int tile = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (tile * 32 >= M) return;
+    const int nt = min(32, M - tile * 32);
+    const int at = tile * 32 + min(lane, nt - 1);
+    const int k = val ? val[at] : at;
+    const int e = pcls[k];
+    int rank = 0;
+    for (int o = 0; o < nt; ++o) {
+        const int eo = __shfl_sync(0xffffffffu, e, o);
+        rank += (eo < e || (eo == e && o < lane)) ? 1 : 0;
+    }
+    const double x = px[k], y = py[k], z = pz[k];
+    if (lane < nt) {
+        idx[tile * 32 + rank] = k;
+        cls[tile * 32 + rank] = e;
+        xyz[tile * 32 + rank] = F64Pt{x, y, z, 0.0};
+    }
+    float lo[3] = {(float)x, (float)y, (float)z}, hi[3] = {(float)x, (float)y, (float)z};
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
+            hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
+        }
+    const float cx = 0.5f * (lo[0] + hi[0]), cy = 0.5f * (lo[1] + hi[1]), cz = 0.5f * (lo[2] + hi[2]);
+    const float dx = (float)x - cx, dy = (float)y - cy, dz = (float)z - cz;
+    float r2 = dx * dx + dy * dy + dz * dz;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) r2 = fmaxf(r2, __shfl_xor_sync(0xffffffffu, r2, o));
+    // the margin covers the FP32 rounding of the coordinates and distances
+    if (lane == 0) sph[tile] = make_float4(cx, cy, cz, sqrtf(r2) * 1.0001f + 1e-4f);
+}
+
+__device__ __forceinline__ int f64_class_of(const F64Src &s, int g)
+{
+    int k = 0;
+#pragma unroll
+    for (int i = 1; i < 6; ++i) k += g >= s.off[i] ? 1 : 0;
+    return k;
+}
+
+// class, cell along the curve, exponent bin (half octaves from 0.2, ascending)
+__global__ void f64_pair_key_kernel(int n, F64Src src, F64Box box, unsigned *__restrict__ key, int *__restrict__ val)
+{
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= n) return;
+    const int k = f64_class_of(src, g), r = g - src.off[k];
+    const unsigned h = curve_key<F64_HBITS>(src.Px[k][r], src.Py[k][r], src.Pz[k][r], box);
+    const int pb = min(max((int)floorf(2.f * log2f(5.f * (float)src.p[k][r])), 0), (1 << F64_PBITS) - 1);
+    key[g] = ((unsigned)k << (3 * F64_HBITS + F64_PBITS)) | (h << F64_PBITS) | (unsigned)pb;
+    val[g] = g;
+}
+
+// rho and cn of f64.cuh for exponent z2 = zeta^2
+__device__ __forceinline__ double2 f64_rho_cn(double p, double z2)
+{
+    const double rho = p * z2 / (p + z2);
+    return make_double2(rho, 2.0 * sqrt(rho / PCM_PI));
+}
+
+// sorted pair data: kept index, centre and exponent, FP32 copies for the tests,
+// and (for few exponent classes) rho and cn per class
+__global__ void f64_pair_gather_kernel(int n, F64Src src, const int *__restrict__ val, int ncls,
+                                       const double *__restrict__ cls_zeta, int *__restrict__ ord,
+                                       double *__restrict__ P, float4 *__restrict__ info, double2 *__restrict__ rc)
+{
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= n) return;
+    const int k = f64_class_of(src, g), r = (val ? val[g] : g) - src.off[k];
+    const double x = src.Px[k][r], y = src.Py[k][r], z = src.Pz[k][r], p = src.p[k][r];
+    ord[g] = r;
+    P[g] = x;
+    P[(size_t)n + g] = y;
+    P[2 * (size_t)n + g] = z;
+    P[3 * (size_t)n + g] = p;
+    info[g] = make_float4((float)x, (float)y, (float)z, (float)p);
+    if (rc)
+        for (int e = 0; e < ncls; ++e) rc[(size_t)e * n + g] = f64_rho_cn(p, cls_zeta[e] * cls_zeta[e]);
+}
+
+// point tiles and sorted pairs of the current geometry and basis
+int f64_prepare(pcm_ctx *c)
+{
+    F64Int &f = c->f64;
+    const int M = c->M;
+    F64Box box;
+    double ext = 1e-3;
+    for (int d = 0; d < 3; ++d) {
+        double lo = 1e300, hi = -1e300;
+        for (int I = 0; I < c->natom; ++I) {
+            lo = std::min(lo, c->h_xyz[3 * I + d] - c->h_radius[I]);
+            hi = std::max(hi, c->h_xyz[3 * I + d] + c->h_radius[I]);
+        }
+        box.lo[d] = lo;
+        ext = std::max(ext, hi - lo);
+    }
+    box.inv = 1.0 / (ext * (1.0 + 1e-9));
+    F64Src src;
+    int n = 0;
+    for (int k = 0; k < 6; ++k) {
+        src.off[k] = f.off[k] = n;
+        src.Px[k] = c->cls[k].Px.p;
+        src.Py[k] = c->cls[k].Py.p;
+        src.Pz[k] = c->cls[k].Pz.p;
+        src.p[k] = c->cls[k].p.p;
+        n += c->cls[k].npair;
+    }
+    src.off[6] = f.off[6] = n;
+    f.ntile = (M + 31) / 32;
+    PCM_TRY(f.pt_idx.alloc(M));
+    PCM_TRY(f.pt_cls.alloc(M));
+    PCM_TRY(f.pt_xyz.alloc(M));
+    PCM_TRY(f.pt_sph.alloc(f.ntile));
+    const bool sort_pts = M >= F64_SORT_MIN / 4;
+    if (sort_pts) {
+        PCM_TRY(f.key.alloc(M));
+        PCM_TRY(f.val.alloc(M));
+        f64_point_key_kernel<<<(M + 127) / 128, 128, 0, c->stream>>>(M, c->px.p, c->py.p, c->pz.p, box, f.key.p,
+                                                                    f.val.p);
+        PCM_LAUNCHED(c);
+        PCM_TRY(sort_pairs(c, M, 3 * F64_PTBITS, f.key, f.val));
+    }
+    f64_point_tile_kernel<<<(f.ntile + 3) / 4, 128, 0, c->stream>>>(M, sort_pts ? f.val.p : nullptr, c->px.p, c->py.p,
+                                                                   c->pz.p, c->pcls.p, f.pt_idx.p, f.pt_cls.p,
+                                                                   f.pt_xyz.p, f.pt_sph.p);
+    PCM_LAUNCHED(c);
+    if (n == 0) return PCM_OK;
+    PCM_TRY(f.ord.alloc(n));
+    PCM_TRY(f.P.alloc(4 * (size_t)n));
+    PCM_TRY(f.info.alloc(n));
+    f.use_rc = c->ncls <= F64_RC_CLASSES;
+    if (f.use_rc) PCM_TRY(f.rc.alloc((size_t)c->ncls * n));
+    const bool sort_pr = n >= F64_SORT_MIN;
+    if (sort_pr) {
+        PCM_TRY(f.key.alloc(n));   // the sort may have exchanged these with its scratch
+        PCM_TRY(f.val.alloc(n));
+        f64_pair_key_kernel<<<(n + 127) / 128, 128, 0, c->stream>>>(n, src, box, f.key.p, f.val.p);
+        PCM_LAUNCHED(c);
+        PCM_TRY(sort_pairs(c, n, 3 + 3 * F64_HBITS + F64_PBITS, f.key, f.val));
+    }
+    f64_pair_gather_kernel<<<(n + 127) / 128, 128, 0, c->stream>>>(n, src, sort_pr ? f.val.p : nullptr, c->ncls,
+                                                                  c->cls_zeta.p, f.ord.p, f.P.p, f.info.p,
+                                                                  f.use_rc ? f.rc.p : nullptr);
+    PCM_LAUNCHED(c);
+    return PCM_OK;
+}
+
+// ---------------------------------------------------------------------------
+// ESP preparation: density test of Eq. 18 over the sorted pairs of every class,
+// one compaction, then the coefficients of f64_dot per kept pair
+// ---------------------------------------------------------------------------
+template <int LA, int LB>
+__global__ void f64_flag_kernel(int off, int npair, const int *__restrict__ ord, const int *__restrict__ sp,
+                                const int *__restrict__ ia, const int *__restrict__ ib, const int *__restrict__ spA,
+                                const int *__restrict__ spB, const int *__restrict__ sh_bf,
+                                const double *__restrict__ Q, const double *__restrict__ Pm, int nbf, double thresh,
+                                unsigned char *__restrict__ flag)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= npair) return;
+    const int r = ord[off + j];
+    const int s = sp[r];
+    const int A = spA[s], B = spB[s];
+    const bool mirror = (A != B) || (ia[r] != ib[r]);
+    const int fa = sh_bf[A], fb = sh_bf[B];
+    double wmax = 0.0;
+    for (int a = 0; a < ncart(LA); ++a)
+        for (int b = 0; b < ncart(LB); ++b) {
+            double w = Pm[(size_t)(fa + a) * nbf + fb + b];
+            if (mirror) w += Pm[(size_t)(fb + b) * nbf + fa + a];
+            wmax = fmax(wmax, fabs(w));
+        }
+    flag[off + j] = thresh <= 0.0 || wmax * Q[r] >= thresh ? 1 : 0;
+}
+
+// kept pairs before each class
+__global__ void f64_class_counts_kernel(F64Src src, const int *__restrict__ pos, int *__restrict__ out)
+{
+    if (threadIdx.x < 7) out[threadIdx.x] = pos[src.off[threadIdx.x]];
+}
+
+// record of ESP pair j (list: sorted positions): centre and far-field terms of
+// its Hermite density D_tuv = -(2 pi / p) K sum_ab W_ab c_a c_b E^ab_tuv
+// (W_ab = P_ab + P_ba for a pair that stands for its mirror image too)
+template <int LA, int LB>
+__global__ void f64_coef_kernel(int nesp, int off, const int *__restrict__ list, const int *__restrict__ ord,
+                                const int *__restrict__ sp, const int *__restrict__ ia, const int *__restrict__ ib,
+                                const int *__restrict__ spA, const int *__restrict__ spB,
+                                const int *__restrict__ sh_atom, const int *__restrict__ sh_off,
+                                const int *__restrict__ sh_bf, const double *__restrict__ cnorm,
+                                const double *__restrict__ xyz, const double *__restrict__ Px,
+                                const double *__restrict__ Py, const double *__restrict__ Pz,
+                                const double *__restrict__ pp, const double *__restrict__ pref,
+                                const double *__restrict__ Pm, int nbf, int *__restrict__ elist,
+                                double *__restrict__ rec)
+{
+    constexpr int L = LA + LB;
+    constexpr int NH = nherm(L);
+    constexpr int NC = far_nterms(L);
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= nesp) return;
+    const int r = ord[list[j]];
+    elist[j] = r;
+    const int s = sp[r];
+    const int A = spA[s], B = spB[s];
+    const int i1 = ia[r], i2 = ib[r];
+    const bool mirror = (A != B) || (i1 != i2);
+    const double p = pp[r];
+    const double P[3] = {Px[r], Py[r], Pz[r]};
+    const double *RA = xyz + 3 * sh_atom[A], *RB = xyz + 3 * sh_atom[B];
+    E1T<LA, LB> Ex, Ey, Ez;
+    const double inv2p = 0.5 / p;
+    hermite_E1T<LA, LB>(P[0] - RA[0], P[0] - RB[0], inv2p, Ex);
+    hermite_E1T<LA, LB>(P[1] - RA[1], P[1] - RB[1], inv2p, Ey);
+    hermite_E1T<LA, LB>(P[2] - RA[2], P[2] - RB[2], inv2p, Ez);
+    const double cc = cnorm[sh_off[A] + i1] * cnorm[sh_off[B] + i2];
+    const int fa = sh_bf[A], fb = sh_bf[B];
+    double D[NH];
+#pragma unroll
+    for (int h = 0; h < NH; ++h) D[h] = 0.0;
+#pragma unroll
+    for (int a = 0; a < ncart(LA); ++a) {
+        const int ax = cart_e(LA, a, 0), ay = cart_e(LA, a, 1), az = cart_e(LA, a, 2);
+#pragma unroll
+        for (int b = 0; b < ncart(LB); ++b) {
+            const int bx = cart_e(LB, b, 0), by = cart_e(LB, b, 1), bz = cart_e(LB, b, 2);
+            double w = Pm[(size_t)(fa + a) * nbf + fb + b];
+            if (mirror) w += Pm[(size_t)(fb + b) * nbf + fa + a];
+            w *= cc * f64_comp_factor(LA, a) * f64_comp_factor(LB, b);
+            // E_t vanishes for t > i + j
+#pragma unroll
+            for (int t = 0; t <= ax + bx; ++t)
+#pragma unroll
+                for (int u = 0; u <= ay + by; ++u) {
+                    const double wxy = w * Ex.e[ax][bx][t] * Ey.e[ay][by][u];
+#pragma unroll
+                    for (int v = 0; v <= az + bz; ++v)
+                        D[hidx(t, u, v)] = fma(wxy, Ez.e[az][bz][v], D[hidx(t, u, v)]);
+                }
+        }
+    }
+    constexpr FarContrib FC = far_contrib(L);
+    const double g = -pref[r] * 0.88622692545275801365 / sqrt(p);   // sqrt(pi) / (2 sqrt(p))
+    double G[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) G[k] = 0.0;
+#pragma unroll
+    for (int q = 0; q < FC.count; ++q) G[FC.term[q]] = fma(FC.w[q], D[FC.h[q]], G[FC.term[q]]);
+    double *o = rec + (size_t)j * f64_rec(L);
+    o[0] = P[0];
+    o[1] = P[1];
+    o[2] = P[2];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) o[3 + k] = g * G[k];
+}
+
+template <int LA, int LB>
+static int f64_flag_class(pcm_ctx *c, int k, const double *dP)
+{
+    PairClass &pc = c->cls[k];
+    if (pc.npair == 0) return PCM_OK;
+    f64_flag_kernel<LA, LB><<<(pc.npair + 127) / 128, 128, 0, c->stream>>>(
+        c->f64.off[k], pc.npair, c->f64.ord.p, pc.sp.p, pc.ia.p, pc.ib.p, pc.spA.p, pc.spB.p, c->sh_bf.p, pc.Q.p, dP,
+        c->nbf, c->opt.schwarz, c->f64.flag.p);
+    PCM_LAUNCHED(c);
+    return PCM_OK;
+}
+
+template <int LA, int LB>
+static int f64_coef_class(pcm_ctx *c, int k, const double *dP)
+{
+    PairClass &pc = c->cls[k];
+    if (pc.nesp == 0) return PCM_OK;
+    PCM_TRY(pc.elist.alloc(pc.npair));
+    f64_coef_kernel<LA, LB><<<(pc.nesp + 127) / 128, 128, 0, c->stream>>>(
+        pc.nesp, c->f64.off[k], c->f64.list.p + c->f64.eoff[k], c->f64.ord.p, pc.sp.p, pc.ia.p, pc.ib.p, pc.spA.p,
+        pc.spB.p, c->sh_atom.p, c->sh_off.p, c->sh_bf.p, c->cnorm.p, c->xyz.p, pc.Px.p, pc.Py.p, pc.Pz.p, pc.p.p,
+        pc.pref.p, dP, c->nbf, pc.elist.p, c->f64.rec.p + c->f64.roff[k]);
+    PCM_LAUNCHED(c);
+    return PCM_OK;
+}
+
+int f64_esp_prepare(pcm_ctx *c, const double *dP)
+{
+    F64Int &f = c->f64;
+    const int n = f.off[6];
+    for (int k = 0; k < 6; ++k) c->cls[k].nesp = c->cls[k].nesp_same = 0;
+    for (int k = 0; k <= 6; ++k) f.eoff[k] = 0;
+    if (n == 0) return PCM_OK;
+    PCM_TRY(f.flag.alloc(n));
+    PCM_TRY(f.list.alloc(n));
+    PCM_TRY(f.pos.alloc((size_t)n + 1));
+    PCM_TRY((f64_flag_class<0, 0>(c, 0, dP)));
+    PCM_TRY((f64_flag_class<1, 0>(c, 1, dP)));
+    PCM_TRY((f64_flag_class<1, 1>(c, 2, dP)));
+    PCM_TRY((f64_flag_class<2, 0>(c, 3, dP)));
+    PCM_TRY((f64_flag_class<2, 1>(c, 4, dP)));
+    PCM_TRY((f64_flag_class<2, 2>(c, 5, dP)));
+    PCM_TRY(compact_flags(c, f.flag.p, n, f.list.p, f.pos.p, c->iscal.p + 8));
+    F64Src src{};
+    for (int k = 0; k <= 6; ++k) src.off[k] = f.off[k];
+    f64_class_counts_kernel<<<1, 32, 0, c->stream>>>(src, f.pos.p, c->iscal.p);
+    PCM_LAUNCHED(c);
+    PCM_CUDA(cudaMemcpyAsync(f.eoff, c->iscal.p, 7 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    PCM_CUDA(cudaStreamSynchronize(c->stream));
+    static constexpr int REC[6] = {f64_rec(0), f64_rec(1), f64_rec(2), f64_rec(2), f64_rec(3), f64_rec(4)};
+    size_t total = 0;
+    for (int k = 0; k < 6; ++k) {
+        c->cls[k].nesp = f.eoff[k + 1] - f.eoff[k];
+        f.roff[k] = total;
+        total += (size_t)REC[k] * c->cls[k].nesp;
+    }
+    PCM_TRY(f.rec.alloc(std::max<size_t>(1, total)));
+    PCM_TRY((f64_coef_class<0, 0>(c, 0, dP)));
+    PCM_TRY((f64_coef_class<1, 0>(c, 1, dP)));
+    PCM_TRY((f64_coef_class<1, 1>(c, 2, dP)));
+    PCM_TRY((f64_coef_class<2, 0>(c, 3, dP)));
+    PCM_TRY((f64_coef_class<2, 1>(c, 4, dP)));
+    PCM_TRY((f64_coef_class<2, 2>(c, 5, dP)));
+    return PCM_OK;
+}
+
+// ---------------------------------------------------------------------------
+// main kernels
+// ---------------------------------------------------------------------------
+// FP32 value of a non-negative double from its high word (20 mantissa bits,
+// towards zero), without the conversion's FP64-pipe slot
+__device__ __forceinline__ float f64_trunc32(double v)
+{
+    return __int_as_float((max(__double2hiint(v), 0x38100000) - 0x38000000) << 3);
+}
+
+// what the kernels read of the points and of one class's sorted pairs
+struct F64Points {
+    int M, ntile;
+    const F64Pt *xyz;      // x, y, z, charge (Fock)
+    const int *cls;
+    const float4 *sph;
+    const double *cls_zeta;
+    float zmin2;             // smallest zeta^2: the smallest rho, the longest reach
+    const double *tab;
+};
+
+struct F64Pairs {
+    int n;                   // pairs of the launch
+    int stride;              // sorted pairs of all classes
+    const int *list;         // sorted positions of the pairs (null: 0 .. n-1 from first)
+    int first;
+    const float4 *info;
+    const double *P;         // 4 x stride
+    const double2 *rc;       // ncls x stride, or null
+    const double *rec;       // ESP records
+};
+
+__device__ __forceinline__ double2 f64_load_rc(const F64Pairs &a, const F64Points &t, int e, int pos)
+{
+    if (a.rc) return __ldg(a.rc + (size_t)e * a.stride + pos);
+    const double z = t.cls_zeta[e];
+    return f64_rho_cn(a.P[3 * (size_t)a.stride + pos], z * z);
+}
+
+// reach test: may a pair (info b) have T < farT at a point of the tile?
+__device__ __forceinline__ bool f64_reaches(const float4 &b, const float4 &s, float zmin2, float farT)
+{
+    const float dx = b.x - s.x, dy = b.y - s.y, dz = b.z - s.z;
+    const float d = fmaxf(sqrtf(dx * dx + dy * dy + dz * dz) * 0.99999f - 2e-5f - s.w, 0.f);
+    return b.w * zmin2 * d * d < 1.00001f * farT * (b.w + zmin2);
+}
+
+// resident blocks of 128 threads per SM the register allocation aims for: the
+// FP64 pipe is full with two or three warps per scheduler
+constexpr int f64_min_blocks(int terms) { return terms <= 11 ? 4 : (terms <= 24 ? 3 : 2); }
+
+// Point part of the integral gradient (gc of Eq. 22): per point the sums over
+// the ESP pairs of the derivatives with respect to P.  One point tile per block,
+// a lane per point; the block's four warps and the grid's rows share the pairs
+// in chunks of `ch` (at most 32: a lane per pair for the reach test).
+// part[row][component][slot].
+template <int L>
+__global__ void __launch_bounds__(128, f64_min_blocks(far_nterms(L)))
+    f64_grad_kernel(F64Pairs a, F64Points t, int ch, double *__restrict__ part)
+{
+    constexpr int NC = far_nterms(L);
+    constexpr int REC = f64_rec(L);
+    constexpr int LB = L + 1;      // highest b_n
+    constexpr float FT = (float)f64_far_T(LB);
+    __shared__ double red[4][3][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int tile = blockIdx.x;
+    const int slot = min(tile * 32 + lane, t.M - 1);
+    const F64Pt c = t.xyz[slot];
+    const int e = t.cls[slot];
+    const float4 sph = t.sph[tile];
+    double acc[3] = {0.0, 0.0, 0.0};
+    auto interact = [&](int j, int pos, bool reaches) {
+        const double2 *r = reinterpret_cast<const double2 *>(a.rec + (size_t)j * REC);
+        double v[REC];
+#pragma unroll
+        for (int i = 0; i < REC / 2; ++i) {
+            const double2 x = __ldg(r + i);
+            v[2 * i] = x.x;
+            v[2 * i + 1] = x.y;
+        }
+        double G[NC];
+#pragma unroll
+        for (int k = 0; k < NC; ++k) G[k] = v[3 + k];
+        const double X = v[0] - c.x, Y = v[1] - c.y, Z = v[2] - c.z;
+        const double R2 = fma(X, X, fma(Y, Y, Z * Z));
+        double b[LB + 1];
+        if (!reaches) {
+            f64_far<LB>(R2, b);
+        } else {
+            const double2 rc = f64_load_rc(a, t, e, pos);
+            const bool near = f64_trunc32(R2) * f64_trunc32(rc.x) < FT;
+            if (__any_sync(0xffffffffu, near)) {
+                f64_near<LB>(R2, rc.x, rc.y, near, t.tab, b);
+                if (!__all_sync(0xffffffffu, near)) {
+                    double bf[LB + 1];
+                    f64_far<LB>(R2, bf);
+#pragma unroll
+                    for (int n = 0; n <= LB; ++n) b[n] = near ? b[n] : bf[n];
+                }
+            } else {
+                f64_far<LB>(R2, b);
+            }
+        }
+        f64_dot_grad<L>(X, Y, Z, b, G, acc);
+    };
+    for (int j0 = (blockIdx.y * 4 + w) * ch; j0 < a.n; j0 += gridDim.y * 4 * ch) {
+        const bool act = lane < ch && j0 + lane < a.n;
+        int pos = 0;
+        bool nr = false;
+        if (act) {
+            pos = a.list[j0 + lane];
+            nr = f64_reaches(a.info[pos], sph, t.zmin2, FT);
+        }
+        const unsigned all = __ballot_sync(0xffffffffu, act), nm = __ballot_sync(0xffffffffu, nr);
+        for (unsigned m = all & ~nm; m; m &= m - 1) interact(j0 + __ffs(m) - 1, 0, false);
+        for (unsigned m = nm; m; m &= m - 1) {
+            const int o = __ffs(m) - 1;
+            interact(j0 + o, __shfl_sync(0xffffffffu, pos, o), true);
+        }
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) red[w][d][lane] = acc[d];
+    __syncthreads();
+    if (w == 0 && tile * 32 + lane < t.M) {
+        const size_t S = (size_t)t.ntile * 32;
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            part[((size_t)blockIdx.y * 3 + d) * S + tile * 32 + lane] =
+                (red[0][d][lane] + red[1][d][lane]) + (red[2][d][lane] + red[3][d][lane]);
+    }
+}
+
+// g[d][point] -= q times the sum of the partial rows, in row order
+__global__ void f64_grad_reduce_kernel(int M, int S, int rows, const double *__restrict__ part,
+                                       const int *__restrict__ idx, const double *__restrict__ q,
+                                       double *__restrict__ g)
+{
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= M) return;
+    const int k = idx[s];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        double v = 0.0;
+        for (int r = 0; r < rows; ++r) v += part[((size_t)r * 3 + d) * S + s];
+        g[(size_t)d * M + k] -= q[k] * v;
+    }
+}
+
+// the points' charges beside their coordinates
+__global__ void f64_point_charge_kernel(int M, const int *__restrict__ idx, const double *__restrict__ q,
+                                        F64Pt *__restrict__ xyz)
+{
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s < M) xyz[s].w = q[idx[s]];
+}
+
+// Fock accumulation: a warp per 32 sorted pairs (a lane per pair), over the
+// point tiles blockIdx.y, + gridDim.y, ...; S[row][term][pair] = sum_k q_k b_n
+// X^a Y^b Z^c per term of farfield.cuh (mapped to Hermite components by
+// f64_fold_kernel; a term costs one FMA per interaction, the Hermite recurrence
+// about two).
+template <int L>
+__global__ void __launch_bounds__(128, f64_min_blocks(far_nterms(L)))
+    f64_fock_kernel(F64Pairs a, F64Points t, double *__restrict__ S)
+{
+    constexpr int NC = far_nterms(L);
+    constexpr float FT = (float)f64_far_T(L);
+    const int lane = threadIdx.x & 31;
+    const int j = (blockIdx.x * 4 + (threadIdx.x >> 5)) * 32 + lane;
+    if (j - lane >= a.n) return;
+    const int jj = min(j, a.n - 1);
+    const int pos = a.list ? a.list[jj] : a.first + jj;
+    const double Px = a.P[pos], Py = a.P[(size_t)a.stride + pos], Pz = a.P[2 * (size_t)a.stride + pos];
+    const float4 info = a.info[pos];
+    double acc[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) acc[k] = 0.0;
+    for (int tile = blockIdx.y; tile < t.ntile; tile += gridDim.y) {
+        const bool reaches = __any_sync(0xffffffffu, f64_reaches(info, t.sph[tile], t.zmin2, FT));
+        const int s0 = tile * 32, s1 = min(t.M, s0 + 32);
+        if (!reaches) {
+            for (int s = s0; s < s1; ++s) {
+                const F64Pt c = t.xyz[s];
+                const double X = Px - c.x, Y = Py - c.y, Z = Pz - c.z;
+                double b[L + 1];
+                f64_far<L>(fma(X, X, fma(Y, Y, Z * Z)), b);
+#pragma unroll
+                for (int n = 0; n <= L; ++n) b[n] *= c.w;
+                f64_accumulate<L>(X, Y, Z, b, acc);
+            }
+        } else {
+            int cur = -1;
+            double2 rc = make_double2(1.0, 1.0);
+            float rf = 1.f;
+            for (int s = s0; s < s1; ++s) {
+                const F64Pt c = t.xyz[s];
+                const int e = t.cls[s];
+                if (e != cur) {
+                    cur = e;
+                    rc = f64_load_rc(a, t, e, pos);
+                    rf = f64_trunc32(rc.x);
+                }
+                const double X = Px - c.x, Y = Py - c.y, Z = Pz - c.z;
+                const double R2 = fma(X, X, fma(Y, Y, Z * Z));
+                const bool near = f64_trunc32(R2) * rf < FT;
+                double b[L + 1];
+                if (__any_sync(0xffffffffu, near)) {
+                    f64_near<L>(R2, rc.x, rc.y, near, t.tab, b);
+                    if (!__all_sync(0xffffffffu, near)) {
+                        double bf[L + 1];
+                        f64_far<L>(R2, bf);
+#pragma unroll
+                        for (int n = 0; n <= L; ++n) b[n] = near ? b[n] : bf[n];
+                    }
+                } else {
+                    f64_far<L>(R2, b);
+                }
+#pragma unroll
+                for (int n = 0; n <= L; ++n) b[n] *= c.w;
+                f64_accumulate<L>(X, Y, Z, b, acc);
+            }
+        }
+    }
+    if (j < a.n)
+#pragma unroll
+        for (int k = 0; k < NC; ++k) S[((size_t)blockIdx.y * NC + k) * a.n + j] = acc[k];
+}
+
+// W_tuv = sqrt(pi) / (2 sqrt(p)) sum over the terms (the transpose of the
+// mapping that made the ESP's coefficients) of the rows' sums, written at the
+// kept pair's place (ord) or, without ord, at j
+template <int L>
+__global__ void f64_fold_kernel(F64Pairs a, int rows, const double *__restrict__ S, const int *__restrict__ ord,
+                                int ldw, double *__restrict__ W)
+{
+    constexpr int NC = far_nterms(L);
+    constexpr int NH = nherm(L);
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= a.n) return;
+    double acc[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        double v = 0.0;
+        for (int r = 0; r < rows; ++r) v += S[((size_t)r * NC + k) * a.n + j];
+        acc[k] = v;
+    }
+    const int pos = a.list ? a.list[j] : a.first + j;
+    const double g = 0.88622692545275801365 / sqrt(a.P[3 * (size_t)a.stride + pos]);
+    constexpr FarContrib FC = far_contrib(L);
+    double out[NH];
+#pragma unroll
+    for (int h = 0; h < NH; ++h) out[h] = 0.0;
+#pragma unroll
+    for (int q = 0; q < FC.count; ++q) out[FC.h[q]] = fma(FC.w[q], acc[FC.term[q]], out[FC.h[q]]);
+    const int at = ord ? ord[pos] : j;
+#pragma unroll
+    for (int h = 0; h < NH; ++h) W[(size_t)h * ldw + at] = g * out[h];
+}
+
+// ---------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------
+static F64Points f64_points(pcm_ctx *c)
+{
+    F64Points t;
+    t.M = c->M;
+    t.ntile = c->f64.ntile;
+    t.xyz = c->f64.pt_xyz.p;
+    t.cls = c->f64.pt_cls.p;
+    t.sph = c->f64.pt_sph.p;
+    t.cls_zeta = c->cls_zeta.p;
+    t.zmin2 = (float)(c->h_cls_zeta[0] * c->h_cls_zeta[0]) * 0.99999f;
+    t.tab = c->f64.tab.p;
+    return t;
+}
+
+static F64Pairs f64_pairs(pcm_ctx *c, int k, bool esp)
+{
+    F64Int &f = c->f64;
+    F64Pairs a;
+    a.n = esp ? c->cls[k].nesp : c->cls[k].npair;
+    a.stride = f.off[6];
+    a.list = esp ? f.list.p + f.eoff[k] : nullptr;
+    a.first = f.off[k];
+    a.info = f.info.p;
+    a.P = f.P.p;
+    a.rc = f.use_rc ? f.rc.p : nullptr;
+    a.rec = esp ? f.rec.p + f.roff[k] : nullptr;
+    return a;
+}
+
+// chunk length and grid rows of a point-part launch over n pairs
+static void f64_grad_plan(int n, int ntile, int *ch, int *rows)
+{
+    *ch = (int)std::min<long long>(32, std::max<long long>(4, (long long)n * ntile / (4LL * F64_CTAS)));
+    const int want = (F64_CTAS + ntile - 1) / ntile;
+    *rows = std::max(1, std::min(want, (n + 4 * *ch - 1) / (4 * *ch)));
+}
+
+template <int L>
+static int f64_grad_launch(pcm_ctx *c, int k, int ch, int rows, double *part)
+{
+    f64_grad_kernel<L><<<dim3(c->f64.ntile, rows), 128, 0, c->stream>>>(f64_pairs(c, k, true), f64_points(c), ch,
+                                                                       part);
+    PCM_LAUNCHED(c);
+    return PCM_OK;
+}
+
+// gk[3][M] += the point part of the gradient over the ESP pairs
+int f64_grad_point(pcm_ctx *c, const double *dq, double *gk)
+{
+    const int nt = c->f64.ntile;
+    const size_t S = (size_t)nt * 32;
+    int ch[6], rows[6], total = 0;
+    for (int k = 0; k < 6; ++k) {
+        rows[k] = 0;
+        if (c->cls[k].nesp == 0) continue;
+        f64_grad_plan(c->cls[k].nesp, nt, &ch[k], &rows[k]);
+        total += rows[k];
+    }
+    if (total == 0) return PCM_OK;
+    PCM_TRY(c->esp_part.alloc(total * 3 * S));
+    double *part = c->esp_part.p;
+    for (int k = 0; k < 6; ++k) {
+        if (rows[k] == 0) continue;
+        switch (F64_LSUM[k]) {
+        case 0: PCM_TRY(f64_grad_launch<0>(c, k, ch[k], rows[k], part)); break;
+        case 1: PCM_TRY(f64_grad_launch<1>(c, k, ch[k], rows[k], part)); break;
+        case 2: PCM_TRY(f64_grad_launch<2>(c, k, ch[k], rows[k], part)); break;
+        case 3: PCM_TRY(f64_grad_launch<3>(c, k, ch[k], rows[k], part)); break;
+        case 4: PCM_TRY(f64_grad_launch<4>(c, k, ch[k], rows[k], part)); break;
+        }
+        part += (size_t)rows[k] * 3 * S;
+    }
+    f64_grad_reduce_kernel<<<(c->M + 127) / 128, 128, 0, c->stream>>>(c->M, (int)S, total, c->esp_part.p,
+                                                                     c->f64.pt_idx.p, dq, gk);
+    PCM_LAUNCHED(c);
+    return PCM_OK;
+}
+
+int f64_charges(pcm_ctx *c, const double *dq)
+{
+    f64_point_charge_kernel<<<(c->M + 127) / 128, 128, 0, c->stream>>>(c->M, c->f64.pt_idx.p, dq, c->f64.pt_xyz.p);
+    PCM_LAUNCHED(c);
+    return PCM_OK;
+}
+
+template <int L>
+static int f64_w_launch(pcm_ctx *c, const F64Pairs &a, const int *ord, double *W)
+{
+    const int nb = (a.n + 127) / 128;
+    const int rows = std::max(1, std::min(c->f64.ntile, (F64_CTAS + nb - 1) / nb));
+    PCM_TRY(c->f64.S.alloc((size_t)rows * far_nterms(L) * a.n));
+    f64_fock_kernel<L><<<dim3(nb, rows), 128, 0, c->stream>>>(a, f64_points(c), c->f64.S.p);
+    PCM_LAUNCHED(c);
+    f64_fold_kernel<L><<<nb, 128, 0, c->stream>>>(a, rows, c->f64.S.p, ord, a.n, W);
+    PCM_LAUNCHED(c);
+    return PCM_OK;
+}
+
+// W[nherm(L)][pairs] of class k for the charges of f64_charges: over the kept
+// pairs in kept order (the Fock correction, L = la + lb), or over the ESP pairs
+// in ESP order (the gradient, L = la + lb + 1)
+int f64_w(pcm_ctx *c, int k, bool esp, double *W)
+{
+    const F64Pairs a = f64_pairs(c, k, esp);
+    if (a.n == 0) return PCM_OK;
+    const int *ord = esp ? nullptr : c->f64.ord.p;
+    switch (F64_LSUM[k] + (esp ? 1 : 0)) {
+    case 0: return f64_w_launch<0>(c, a, ord, W);
+    case 1: return f64_w_launch<1>(c, a, ord, W);
+    case 2: return f64_w_launch<2>(c, a, ord, W);
+    case 3: return f64_w_launch<3>(c, a, ord, W);
+    case 4: return f64_w_launch<4>(c, a, ord, W);
+    case 5: return f64_w_launch<5>(c, a, ord, W);
+    }
+    return PCM_ERR_ARG;
+}
+
+}  // namespace pcm

@@ -401,6 +401,7 @@ int basis_build(pcm_ctx *c, int nshell, const int *shell_atom, const int *shell_
         c->pl_nprim = c->h_sh_nprim;
         c->pair_layout_ok = true;
     }
+    if (c->opt.precision == PCM_FP64) PCM_TRY(f64_prepare(c));
     return PCM_OK;
 }
 

@@ -20,7 +20,7 @@ constexpr int BOYS_GL = 24;
 constexpr int BOYS_PANELS = 16;
 
 // Gauss-Legendre nodes and weights on [-1, 1] by Newton iteration on P_n.
-static void gauss_legendre(int n, std::vector<double> &x, std::vector<double> &w)
+void gauss_legendre(int n, std::vector<double> &x, std::vector<double> &w)
 {
     x.resize(n);
     w.resize(n);
@@ -107,7 +107,7 @@ int boys_build_tables(pcm_ctx *c)
     boys_table_kernel<<<BOYS_NROW, BOYS_MCOL, 0, c->stream>>>(gx.p, gw.p, c->boys64.p, c->boys32.p);
     PCM_LAUNCHED(c);
     PCM_CUDA(cudaStreamSynchronize(c->stream));  // gx, gw are freed on return
-    return PCM_OK;
+    return c->opt.precision == PCM_FP64 ? f64_build_tables(c) : PCM_OK;
 }
 
 // ---------------------------------------------------------------------------
