@@ -113,11 +113,26 @@ struct F64Src {                            // kept pairs of the classes; first s
     const double *Px[6], *Py[6], *Pz[6], *p[6];
     int off[7];
 };
+// cells of the sorted pairs and their expansions (multipole64.cu)
+struct F64Mp {
+    bool on = false;
+    int ncell = 0;
+    DBuf<int> id, pcell;                   // grid cell -> cell; cell of every sorted pair
+    DBuf<int> range;                       // 6 x cells first sorted pair of each class, 6 x cells end
+    DBuf<double> cxyz;                     // centres
+    DBuf<int> crad;                        // radii (FP32 bits)
+    DBuf<unsigned char> order;             // tiles x cells: order of the expansion, 0: none
+    DBuf<double2> raw, M, mom;             // sums per class, moments, scaled moments (or their derivatives)
+    int lsplit = 1;
+    DBuf<double2> lam, tab;                // local expansions, their coefficients per set
+    DBuf<double> V;                        // sets x pairs
+};
 struct F64Int {
     DBuf<double> tab;                      // Boys table (f64.cuh)
     int ntile = 0;                         // tiles of 32 points
     DBuf<int> pt_idx, pt_cls;              // per slot: point, exponent class
     DBuf<F64Pt> pt_xyz;                    // per slot: coordinates, charge of the current call
+    DBuf<float4> pt_x32;                   // per slot: coordinates and zeta^-2 in FP32
     DBuf<float4> pt_sph;                   // per tile: bounding sphere
     int off[7] = {0, 0, 0, 0, 0, 0, 0};    // first sorted position of each class
     DBuf<int> ord;                         // sorted position -> kept pair of its class
@@ -133,6 +148,9 @@ struct F64Int {
     int eoff[7] = {0, 0, 0, 0, 0, 0, 0};   // first ESP pair of each class in list
     size_t roff[6] = {0, 0, 0, 0, 0, 0};   // first record of each class in rec
     DBuf<double> rec;
+    F64Mp mp;
+    size_t boff[6] = {0, 0, 0, 0, 0, 0};   // the same in B
+    DBuf<double> B;                        // ESP pairs' densities as harmonic shifts: (L+1)^2 x pairs per class
     DBuf<double> S;                        // Fock accumulators per term
 };
 
@@ -333,8 +351,14 @@ int f64_build_tables(pcm_ctx *c);
 int f64_prepare(pcm_ctx *c);
 int f64_esp_prepare(pcm_ctx *c, const double *dP);
 int f64_grad_point(pcm_ctx *c, const double *dq, double *gk);
-int f64_charges(pcm_ctx *c, const double *dq);
+int f64_charges(pcm_ctx *c, const double *dq, bool gradient);
 int f64_w(pcm_ctx *c, int k, bool esp, double *W);
+int mp_prepare(pcm_ctx *c, const F64Box &box, const F64Src &src, int bits, int shift);
+int mp_rows(pcm_ctx *c);
+int mp_order(pcm_ctx *c, float eps);
+int mp_grad_far(pcm_ctx *c, double *part);
+int mp_local(pcm_ctx *c);
+int mp_l2p(pcm_ctx *c, int L, int n, const int *list, int first);
 int surface_build(pcm_ctx *c, int natom, const double *xyz, const double *Z, const double *radius, int n);
 int basis_build(pcm_ctx *c, int nshell, const int *shell_atom, const int *shell_l, const int *shell_nprim,
                 const double *exps, const double *coefs);

@@ -34,8 +34,16 @@ constexpr int F64_MTOP = 5;
 constexpr int F64_INV_DT = 256;
 constexpr int F64_NROW = 54 * F64_INV_DT + 2;
 constexpr int F64_STRIDE = 6 * (F64_MTOP + 1);
+// A second table of the same layout follows: H_m(T) = F_m(T) - F_m's asymptotic
+// form = -int_1^inf u^2m e^(-T u^2) du, for T >= F64_H_MIN (its Taylor step is
+// as exact there; below, the two forms are subtracted).
+constexpr int F64_TABLE = F64_NROW * F64_STRIDE;
+constexpr double F64_H_MIN = 6.0;
 // adding 1.5 * 2^44 leaves round(256 T) in the low word of the sum
 constexpr double F64_MAGIC = 26388279066624.0;
+
+// ESP pair record: P, then the coefficients of the terms, padded to 16 bytes
+__host__ __device__ constexpr int f64_rec(int L) { return (3 + far_nterms(L) + 1) / 2 * 2; }
 
 // b_n of the far form; 1/R from the hardware estimate (2^-20) and one
 // third-order step: r0 (1 + e/2 + 3 e^2/8), e = 1 - R^2 r0^2, error 5 e^3 / 16 < 2^-58
@@ -154,6 +162,53 @@ __device__ __forceinline__ void f64_accumulate(double X, double Y, double Z, con
             S[k] = h == 0 ? S[k] + b[FT.n[k]] : fma(b[FT.n[k]], mono[h], S[k]);
         }
     }
+}
+
+// FP32 value of a non-negative double from its high word (20 mantissa bits,
+// towards zero), without the conversion's FP64-pipe slot
+__device__ __forceinline__ float f64_trunc32(double v)
+{
+    return __int_as_float((max(__double2hiint(v), 0x38100000) - 0x38000000) << 3);
+}
+
+// b_n of near interactions (lanes with `on`; T < f64_far_T) of pairs whose far form
+// comes from their cell's expansion: what the near form adds to it.
+template <int L>
+__device__ __forceinline__ void f64_near_minus_far(double R2, double2 rc, bool on, const double *__restrict__ tab,
+                                                   double (&b)[L + 1])
+{
+    const bool low = f64_trunc32(R2) * f64_trunc32(rc.x) < (float)F64_H_MIN;
+    f64_near<L>(R2, rc.x, rc.y, on, low ? tab : tab + F64_TABLE, b);
+    if (__any_sync(0xffffffffu, on && low)) {
+        double bf[L + 1];
+        f64_far<L>(R2, bf);
+#pragma unroll
+        for (int n = 0; n <= L; ++n) b[n] = low ? b[n] - bf[n] : b[n];
+    }
+#pragma unroll
+    for (int n = 0; n <= L; ++n) b[n] = on ? b[n] : 0.0;
+}
+
+// b_n of one interaction per lane, near or far form by T; zero for lanes whose
+// pair is `expanded` (their near part is left to f64_near_minus_far).
+template <int L>
+__device__ __forceinline__ void f64_terms(double R2, double2 rc, bool expanded, const double *__restrict__ tab,
+                                          double (&b)[L + 1])
+{
+    const bool near = f64_trunc32(R2) * f64_trunc32(rc.x) < (float)f64_far_T(L);
+    if (__any_sync(0xffffffffu, near && !expanded)) {
+        f64_near<L>(R2, rc.x, rc.y, near, tab, b);
+        if (!__all_sync(0xffffffffu, near)) {
+            double bf[L + 1];
+            f64_far<L>(R2, bf);
+#pragma unroll
+            for (int n = 0; n <= L; ++n) b[n] = near ? b[n] : bf[n];
+        }
+    } else {
+        f64_far<L>(R2, b);
+    }
+#pragma unroll
+    for (int n = 0; n <= L; ++n) b[n] = expanded ? 0.0 : b[n];
 }
 
 }  // namespace pcm

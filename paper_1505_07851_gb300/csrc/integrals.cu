@@ -787,7 +787,7 @@ static int fock_class(pcm_ctx *c, PairClass &pc, const double *dq, double *ddF)
 int fock_compute(pcm_ctx *c, const double *dq, double *ddF)
 {
     c->stats.integrals_fock = 0.0;
-    if (c->opt.precision == PCM_FP64) PCM_TRY(f64_charges(c, dq));
+    if (c->opt.precision == PCM_FP64) PCM_TRY(f64_charges(c, dq, false));
     PCM_TRY((fock_class<0, 0>(c, c->cls[0], dq, ddF)));
     PCM_TRY((fock_class<1, 0>(c, c->cls[1], dq, ddF)));
     PCM_TRY((fock_class<1, 1>(c, c->cls[2], dq, ddF)));
@@ -905,7 +905,7 @@ int grad_integrals(pcm_ctx *c, const double *dP, const double *dq, double *gk, d
         }
     } else {
         PCM_TRY(f64_grad_point(c, dq, gk));
-        PCM_TRY(f64_charges(c, dq));
+        PCM_TRY(f64_charges(c, dq, true));
     }
     return grad_pair_all(c, dP, dq, gpair);
 }

@@ -18,30 +18,38 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
 #include "context.h"
 #include "f64.cuh"
+#include "multipole64.cuh"
 
 namespace pcm {
 
 constexpr int F64_LSUM[6] = {0, 1, 2, 2, 3, 4};
 constexpr int F64_HBITS = 5;              // cells per side of the pairs' grid: 2^5
+constexpr double F64_CELL = 3.0;          // side of a cell (bohr)
 constexpr int F64_PBITS = 4;              // exponent bins within a cell
 constexpr int F64_PTBITS = 6;             // cells per side of the points' grid
 constexpr int F64_SORT_MIN = 4096;        // fewer pairs than this stay in kept order, fewer points than a quarter too
 constexpr int F64_RC_CLASSES = 16;        // up to this many exponent classes rho and cn are tabulated per (class, pair)
-// thread blocks that a launch aims at: two waves of 8 per SM, so that unequal blocks even out
-constexpr int F64_CTAS = 152 * 16;
+// from this many pairs and points on the cells' expansions are used: setting them up
+// costs about as much per pair as 130 (ss) to 250 (pp) points one by one.  Measured
+// without and with them: 60 atoms (2.9k points) 8.4 / 9.7 ms with d shells, 5.5 / 5.3
+// without; 80 atoms 9.3 / 7.6; 150 atoms 39.4 / 23.3; 300 atoms 158 / 63
+constexpr int F64_MP_PAIRS = 40000;
+constexpr int F64_MP_POINTS = 3000;
+// thread blocks that a launch aims at: many more than fit, so that blocks with few
+// expanded cells and blocks with many even out (300-atom Fock: 82.9 ms with 16 per
+// SM, 75.7 with 32, 73.4 with 64)
+constexpr int F64_CTAS = 152 * 64;
 
 __device__ inline double f64_comp_factor(int l, int c)
 {
     return l == 2 && (c == 1 || c == 2 || c == 4) ? 1.7320508075688772935 : 1.0;
 }
-
-// ESP pair record: P, then the coefficients of f64_dot, padded to 16 bytes
-__host__ __device__ constexpr int f64_rec(int L) { return (3 + far_nterms(L) + 1) / 2 * 2; }
 
 // ---------------------------------------------------------------------------
 // table of F_m / (2m-1)!! (f64.cuh): one warp per row, F_9 by quadrature (the
@@ -84,6 +92,25 @@ __global__ void f64_table_kernel(const double *__restrict__ gx, const double *__
         c[4] = F[m + 4] / (24.0 * df);
         c[5] = 0.0;
     }
+    // H_m upwards from H_0 = -sqrt(pi / T) erfc(sqrt T) / 2, all of one sign
+    double *hrow = tab + F64_TABLE + (size_t)row * F64_STRIDE;
+    const bool on = T >= F64_H_MIN - 0.1;
+    double H[TOP + 1];
+    H[0] = on ? -0.5 * sqrt(PCM_PI / T) * erfc(sqrt(T)) : 0.0;
+#pragma unroll
+    for (int m = 1; m <= TOP; ++m) H[m] = on ? fma((double)(2 * m - 1), H[m - 1], -eT) / (2.0 * T) : 0.0;
+    df = 1.0;
+#pragma unroll
+    for (int m = 0; m <= F64_MTOP; ++m) {
+        if (m > 1) df *= (double)(2 * m - 1);
+        double *c = hrow + 6 * m;
+        c[0] = H[m] / df;
+        c[1] = -H[m + 1] / df;
+        c[2] = H[m + 2] / (2.0 * df);
+        c[3] = -H[m + 3] / (6.0 * df);
+        c[4] = H[m + 4] / (24.0 * df);
+        c[5] = 0.0;
+    }
 }
 
 int f64_build_tables(pcm_ctx *c)
@@ -94,7 +121,7 @@ int f64_build_tables(pcm_ctx *c)
     PCM_TRY(g.alloc(2 * F64_GL));
     PCM_CUDA(cudaMemcpyAsync(g.p, x.data(), F64_GL * sizeof(double), cudaMemcpyHostToDevice, c->stream));
     PCM_CUDA(cudaMemcpyAsync(g.p + F64_GL, w.data(), F64_GL * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-    PCM_TRY(c->f64.tab.alloc((size_t)F64_NROW * F64_STRIDE));
+    PCM_TRY(c->f64.tab.alloc(2 * (size_t)F64_TABLE));
     f64_table_kernel<<<(F64_NROW + 3) / 4, 128, 0, c->stream>>>(g.p, g.p + F64_GL, c->f64.tab.p);
     PCM_LAUNCHED(c);
     PCM_CUDA(cudaStreamSynchronize(c->stream));  // g is freed on return
@@ -158,7 +185,8 @@ __global__ void f64_point_key_kernel(int M, const double *__restrict__ px, const
 __global__ void f64_point_tile_kernel(int M, const int *__restrict__ val, const double *__restrict__ px,
                                       const double *__restrict__ py, const double *__restrict__ pz,
                                       const int *__restrict__ pcls, int *__restrict__ idx, int *__restrict__ cls,
-                                      F64Pt *__restrict__ xyz, float4 *__restrict__ sph)
+                                      const double *__restrict__ cls_zeta, F64Pt *__restrict__ xyz,
+                                      float4 *__restrict__ x32, float4 *__restrict__ sph)
 {
     const int tile = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (tile * 32 >= M) return;
@@ -176,6 +204,7 @@ __global__ void f64_point_tile_kernel(int M, const int *__restrict__ val, const 
         idx[tile * 32 + rank] = k;
         cls[tile * 32 + rank] = e;
         xyz[tile * 32 + rank] = F64Pt{x, y, z, 0.0};
+        x32[tile * 32 + rank] = make_float4((float)x, (float)y, (float)z, (float)(1.0 / (cls_zeta[e] * cls_zeta[e])));
     }
     float lo[3] = {(float)x, (float)y, (float)z}, hi[3] = {(float)x, (float)y, (float)z};
 #pragma unroll
@@ -257,7 +286,9 @@ int f64_prepare(pcm_ctx *c)
         box.lo[d] = lo;
         ext = std::max(ext, hi - lo);
     }
-    box.inv = 1.0 / (ext * (1.0 + 1e-9));
+    // cells of F64_CELL (larger when the cavity has more than 32 of them a side)
+    const double cell = std::max(F64_CELL, ext * (1.0 + 1e-9) / (1 << F64_HBITS));
+    box.inv = 1.0 / (cell * (1 << F64_HBITS));
     F64Src src;
     int n = 0;
     for (int k = 0; k < 6; ++k) {
@@ -273,6 +304,7 @@ int f64_prepare(pcm_ctx *c)
     PCM_TRY(f.pt_idx.alloc(M));
     PCM_TRY(f.pt_cls.alloc(M));
     PCM_TRY(f.pt_xyz.alloc(M));
+    PCM_TRY(f.pt_x32.alloc(M));
     PCM_TRY(f.pt_sph.alloc(f.ntile));
     const bool sort_pts = M >= F64_SORT_MIN / 4;
     if (sort_pts) {
@@ -285,8 +317,10 @@ int f64_prepare(pcm_ctx *c)
     }
     f64_point_tile_kernel<<<(f.ntile + 3) / 4, 128, 0, c->stream>>>(M, sort_pts ? f.val.p : nullptr, c->px.p, c->py.p,
                                                                    c->pz.p, c->pcls.p, f.pt_idx.p, f.pt_cls.p,
-                                                                   f.pt_xyz.p, f.pt_sph.p);
+                                                                   c->cls_zeta.p, f.pt_xyz.p, f.pt_x32.p,
+                                                                   f.pt_sph.p);
     PCM_LAUNCHED(c);
+    f.mp.on = false;
     if (n == 0) return PCM_OK;
     PCM_TRY(f.ord.alloc(n));
     PCM_TRY(f.P.alloc(4 * (size_t)n));
@@ -305,6 +339,7 @@ int f64_prepare(pcm_ctx *c)
                                                                   c->cls_zeta.p, f.ord.p, f.P.p, f.info.p,
                                                                   f.use_rc ? f.rc.p : nullptr);
     PCM_LAUNCHED(c);
+    if (n >= F64_MP_PAIRS && M >= F64_MP_POINTS) PCM_TRY(mp_prepare(c, box, src, F64_HBITS, F64_PBITS));
     return PCM_OK;
 }
 
@@ -355,7 +390,7 @@ __global__ void f64_coef_kernel(int nesp, int off, const int *__restrict__ list,
                                 const double *__restrict__ Py, const double *__restrict__ Pz,
                                 const double *__restrict__ pp, const double *__restrict__ pref,
                                 const double *__restrict__ Pm, int nbf, int *__restrict__ elist,
-                                double *__restrict__ rec)
+                                double *__restrict__ rec, double *__restrict__ B_)
 {
     constexpr int L = LA + LB;
     constexpr int NH = nherm(L);
@@ -415,6 +450,16 @@ __global__ void f64_coef_kernel(int nesp, int off, const int *__restrict__ list,
     o[2] = P[2];
 #pragma unroll
     for (int k = 0; k < NC; ++k) o[3 + k] = g * G[k];
+    if (!B_) return;
+    // the same density as shifts of solid harmonics, for the cells' moments
+    constexpr MpMap MM = mp_map(L);
+    double b[(L + 1) * (L + 1)];
+#pragma unroll
+    for (int q = 0; q < (L + 1) * (L + 1); ++q) b[q] = 0.0;
+#pragma unroll
+    for (int i = 0; i < MM.count; ++i) b[MM.s[i]] = fma(MM.B[i], D[MM.h[i]], b[MM.s[i]]);
+#pragma unroll
+    for (int q = 0; q < (L + 1) * (L + 1); ++q) B_[(size_t)q * nesp + j] = g * b[q];
 }
 
 template <int LA, int LB>
@@ -438,7 +483,8 @@ static int f64_coef_class(pcm_ctx *c, int k, const double *dP)
     f64_coef_kernel<LA, LB><<<(pc.nesp + 127) / 128, 128, 0, c->stream>>>(
         pc.nesp, c->f64.off[k], c->f64.list.p + c->f64.eoff[k], c->f64.ord.p, pc.sp.p, pc.ia.p, pc.ib.p, pc.spA.p,
         pc.spB.p, c->sh_atom.p, c->sh_off.p, c->sh_bf.p, c->cnorm.p, c->xyz.p, pc.Px.p, pc.Py.p, pc.Pz.p, pc.p.p,
-        pc.pref.p, dP, c->nbf, pc.elist.p, c->f64.rec.p + c->f64.roff[k]);
+        pc.pref.p, dP, c->nbf, pc.elist.p, c->f64.rec.p + c->f64.roff[k],
+        c->f64.mp.on ? c->f64.B.p + c->f64.boff[k] : nullptr);
     PCM_LAUNCHED(c);
     return PCM_OK;
 }
@@ -467,13 +513,16 @@ int f64_esp_prepare(pcm_ctx *c, const double *dP)
     PCM_CUDA(cudaMemcpyAsync(f.eoff, c->iscal.p, 7 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     PCM_CUDA(cudaStreamSynchronize(c->stream));
     static constexpr int REC[6] = {f64_rec(0), f64_rec(1), f64_rec(2), f64_rec(2), f64_rec(3), f64_rec(4)};
-    size_t total = 0;
+    size_t total = 0, btotal = 0;
     for (int k = 0; k < 6; ++k) {
         c->cls[k].nesp = f.eoff[k + 1] - f.eoff[k];
         f.roff[k] = total;
         total += (size_t)REC[k] * c->cls[k].nesp;
+        f.boff[k] = btotal;
+        btotal += (size_t)((F64_LSUM[k] + 1) * (F64_LSUM[k] + 1)) * c->cls[k].nesp;
     }
     PCM_TRY(f.rec.alloc(std::max<size_t>(1, total)));
+    if (f.mp.on) PCM_TRY(f.B.alloc(std::max<size_t>(1, btotal)));
     PCM_TRY((f64_coef_class<0, 0>(c, 0, dP)));
     PCM_TRY((f64_coef_class<1, 0>(c, 1, dP)));
     PCM_TRY((f64_coef_class<1, 1>(c, 2, dP)));
@@ -486,18 +535,12 @@ int f64_esp_prepare(pcm_ctx *c, const double *dP)
 // ---------------------------------------------------------------------------
 // main kernels
 // ---------------------------------------------------------------------------
-// FP32 value of a non-negative double from its high word (20 mantissa bits,
-// towards zero), without the conversion's FP64-pipe slot
-__device__ __forceinline__ float f64_trunc32(double v)
-{
-    return __int_as_float((max(__double2hiint(v), 0x38100000) - 0x38000000) << 3);
-}
-
 // what the kernels read of the points and of one class's sorted pairs
 struct F64Points {
     int M, ntile;
     const F64Pt *xyz;      // x, y, z, charge (Fock)
     const int *cls;
+    const float4 *x32;       // x, y, z, zeta^-2 in FP32
     const float4 *sph;
     const double *cls_zeta;
     float zmin2;             // smallest zeta^2: the smallest rho, the longest reach
@@ -513,6 +556,9 @@ struct F64Pairs {
     const double *P;         // 4 x stride
     const double2 *rc;       // ncls x stride, or null
     const double *rec;       // ESP records
+    const int *cell;         // cell of every sorted pair, and the order of its expansion
+    const unsigned char *order;   // for every (tile, cell); null: no expansions
+    int ncell;
 };
 
 __device__ __forceinline__ double2 f64_load_rc(const F64Pairs &a, const F64Points &t, int e, int pos)
@@ -528,6 +574,13 @@ __device__ __forceinline__ bool f64_reaches(const float4 &b, const float4 &s, fl
     const float dx = b.x - s.x, dy = b.y - s.y, dz = b.z - s.z;
     const float d = fmaxf(sqrtf(dx * dx + dy * dy + dz * dz) * 0.99999f - 2e-5f - s.w, 0.f);
     return b.w * zmin2 * d * d < 1.00001f * farT * (b.w + zmin2);
+}
+
+// FP32 test of one interaction: T < farT with a margin for the FP32 rounding (the
+// near form holds to the table's end at T = 54); s = 1/p + 1/zeta^2 = 1/rho
+__device__ __forceinline__ bool f64_is_near(float x, float y, float z, float s, float farT)
+{
+    return fmaf(x, x, fmaf(y, y, z * z)) < (1.001f * farT + 0.05f) * s;
 }
 
 // resident blocks of 128 threads per SM the register allocation aims for: the
@@ -553,9 +606,13 @@ __global__ void __launch_bounds__(128, f64_min_blocks(far_nterms(L)))
     const int slot = min(tile * 32 + lane, t.M - 1);
     const F64Pt c = t.xyz[slot];
     const int e = t.cls[slot];
-    const float4 sph = t.sph[tile];
+    const float4 c32 = t.x32[slot], sph = t.sph[tile];
     double acc[3] = {0.0, 0.0, 0.0};
-    auto interact = [&](int j, int pos, bool reaches) {
+    // one interaction per lane with pair j of the list.  FAR: every lane beyond
+    // farT; NEAR: the near part of expanded pairs, lanes with `on`; else near or
+    // far by T
+    constexpr int FAR = 0, NEAR = 1, BOTH = 2;
+    auto interact = [&](auto kind, int j, bool on) {
         const double2 *r = reinterpret_cast<const double2 *>(a.rec + (size_t)j * REC);
         double v[REC];
 #pragma unroll
@@ -570,38 +627,47 @@ __global__ void __launch_bounds__(128, f64_min_blocks(far_nterms(L)))
         const double X = v[0] - c.x, Y = v[1] - c.y, Z = v[2] - c.z;
         const double R2 = fma(X, X, fma(Y, Y, Z * Z));
         double b[LB + 1];
-        if (!reaches) {
+        if constexpr (decltype(kind)::value == FAR)
             f64_far<LB>(R2, b);
-        } else {
-            const double2 rc = f64_load_rc(a, t, e, pos);
-            const bool near = f64_trunc32(R2) * f64_trunc32(rc.x) < FT;
-            if (__any_sync(0xffffffffu, near)) {
-                f64_near<LB>(R2, rc.x, rc.y, near, t.tab, b);
-                if (!__all_sync(0xffffffffu, near)) {
-                    double bf[LB + 1];
-                    f64_far<LB>(R2, bf);
-#pragma unroll
-                    for (int n = 0; n <= LB; ++n) b[n] = near ? b[n] : bf[n];
-                }
-            } else {
-                f64_far<LB>(R2, b);
-            }
-        }
+        else if constexpr (decltype(kind)::value == NEAR)
+            f64_near_minus_far<LB>(R2, f64_load_rc(a, t, e, a.list[j]), on, t.tab, b);
+        else
+            f64_terms<LB>(R2, f64_load_rc(a, t, e, a.list[j]), false, t.tab, b);
         f64_dot_grad<L>(X, Y, Z, b, G, acc);
     };
     for (int j0 = (blockIdx.y * 4 + w) * ch; j0 < a.n; j0 += gridDim.y * 4 * ch) {
+        // a lane per pair: does it reach the tile, is its cell expanded for it
         const bool act = lane < ch && j0 + lane < a.n;
-        int pos = 0;
-        bool nr = false;
+        bool nr = false, ex = false;
+        float4 info = make_float4(0.f, 0.f, 0.f, 1.f);
         if (act) {
-            pos = a.list[j0 + lane];
-            nr = f64_reaches(a.info[pos], sph, t.zmin2, FT);
+            const int pos = a.list[j0 + lane];
+            info = a.info[pos];
+            nr = f64_reaches(info, sph, t.zmin2, FT);
+            ex = a.order && a.order[(size_t)tile * a.ncell + a.cell[pos]] != 0;
         }
-        const unsigned all = __ballot_sync(0xffffffffu, act), nm = __ballot_sync(0xffffffffu, nr);
-        for (unsigned m = all & ~nm; m; m &= m - 1) interact(j0 + __ffs(m) - 1, 0, false);
-        for (unsigned m = nm; m; m &= m - 1) {
+        const unsigned nm = __ballot_sync(0xffffffffu, nr), em = __ballot_sync(0xffffffffu, ex);
+        const unsigned direct = __ballot_sync(0xffffffffu, act) & ~em;
+        for (unsigned m = direct & ~nm; m; m &= m - 1)
+            interact(std::integral_constant<int, FAR>{}, j0 + __ffs(m) - 1, true);
+        for (unsigned m = direct & nm; m; m &= m - 1)
+            interact(std::integral_constant<int, BOTH>{}, j0 + __ffs(m) - 1, true);
+        // expanded pairs that reach the tile: each lane (point) takes the next
+        // pair near it, so that the warp makes as many steps as its busiest lane
+        // has near pairs
+        unsigned near = 0;
+        for (unsigned m = nm & em; m; m &= m - 1) {
             const int o = __ffs(m) - 1;
-            interact(j0 + o, __shfl_sync(0xffffffffu, pos, o), true);
+            const float4 b = make_float4(__shfl_sync(0xffffffffu, info.x, o), __shfl_sync(0xffffffffu, info.y, o),
+                                         __shfl_sync(0xffffffffu, info.z, o), __shfl_sync(0xffffffffu, info.w, o));
+            near |= f64_is_near(b.x - c32.x, b.y - c32.y, b.z - c32.z, 1.f / b.w + c32.w, FT) ? 1u << o : 0u;
+        }
+        int o = 0;
+        while (__any_sync(0xffffffffu, near != 0)) {
+            const bool on = near != 0;
+            if (on) o = __ffs(near) - 1;
+            near &= near - 1;
+            interact(std::integral_constant<int, NEAR>{}, j0 + o, on);
         }
     }
 #pragma unroll
@@ -658,53 +724,69 @@ __global__ void __launch_bounds__(128, f64_min_blocks(far_nterms(L)))
     const int pos = a.list ? a.list[jj] : a.first + jj;
     const double Px = a.P[pos], Py = a.P[(size_t)a.stride + pos], Pz = a.P[2 * (size_t)a.stride + pos];
     const float4 info = a.info[pos];
+    const int cell = a.order ? a.cell[pos] : 0;
     double acc[NC];
 #pragma unroll
     for (int k = 0; k < NC; ++k) acc[k] = 0.0;
+    const float ip = 1.f / info.w;
     for (int tile = blockIdx.y; tile < t.ntile; tile += gridDim.y) {
-        const bool reaches = __any_sync(0xffffffffu, f64_reaches(info, t.sph[tile], t.zmin2, FT));
-        const int s0 = tile * 32, s1 = min(t.M, s0 + 32);
-        if (!reaches) {
-            for (int s = s0; s < s1; ++s) {
-                const F64Pt c = t.xyz[s];
-                const double X = Px - c.x, Y = Py - c.y, Z = Pz - c.z;
-                double b[L + 1];
-                f64_far<L>(fma(X, X, fma(Y, Y, Z * Z)), b);
+        const bool reaches = f64_reaches(info, t.sph[tile], t.zmin2, FT);
+        const bool expanded = a.order && a.order[(size_t)tile * a.ncell + cell] != 0;
+        const int s0 = tile * 32, nt = min(32, t.M - s0);
+        if (!__all_sync(0xffffffffu, expanded)) {
+            // one by one: every point, near or far by T where some pair reaches the tile
+            if (!__any_sync(0xffffffffu, reaches && !expanded)) {
+                for (int s = s0; s < s0 + nt; ++s) {
+                    const F64Pt c = t.xyz[s];
+                    const double X = Px - c.x, Y = Py - c.y, Z = Pz - c.z;
+                    double b[L + 1];
+                    f64_far<L>(fma(X, X, fma(Y, Y, Z * Z)), b);
+                    const double q = expanded ? 0.0 : c.w;
 #pragma unroll
-                for (int n = 0; n <= L; ++n) b[n] *= c.w;
-                f64_accumulate<L>(X, Y, Z, b, acc);
-            }
-        } else {
-            int cur = -1;
-            double2 rc = make_double2(1.0, 1.0);
-            float rf = 1.f;
-            for (int s = s0; s < s1; ++s) {
-                const F64Pt c = t.xyz[s];
-                const int e = t.cls[s];
-                if (e != cur) {
-                    cur = e;
-                    rc = f64_load_rc(a, t, e, pos);
-                    rf = f64_trunc32(rc.x);
+                    for (int n = 0; n <= L; ++n) b[n] *= q;
+                    f64_accumulate<L>(X, Y, Z, b, acc);
                 }
-                const double X = Px - c.x, Y = Py - c.y, Z = Pz - c.z;
-                const double R2 = fma(X, X, fma(Y, Y, Z * Z));
-                const bool near = f64_trunc32(R2) * rf < FT;
-                double b[L + 1];
-                if (__any_sync(0xffffffffu, near)) {
-                    f64_near<L>(R2, rc.x, rc.y, near, t.tab, b);
-                    if (!__all_sync(0xffffffffu, near)) {
-                        double bf[L + 1];
-                        f64_far<L>(R2, bf);
-#pragma unroll
-                        for (int n = 0; n <= L; ++n) b[n] = near ? b[n] : bf[n];
+            } else {
+                int cur = -1;
+                double2 rc = make_double2(1.0, 1.0);
+                for (int s = s0; s < s0 + nt; ++s) {
+                    const F64Pt c = t.xyz[s];
+                    const int e = t.cls[s];
+                    if (e != cur) {
+                        cur = e;
+                        rc = f64_load_rc(a, t, e, pos);
                     }
-                } else {
-                    f64_far<L>(R2, b);
-                }
+                    const double X = Px - c.x, Y = Py - c.y, Z = Pz - c.z;
+                    double b[L + 1];
+                    f64_terms<L>(fma(X, X, fma(Y, Y, Z * Z)), rc, expanded, t.tab, b);
 #pragma unroll
-                for (int n = 0; n <= L; ++n) b[n] *= c.w;
-                f64_accumulate<L>(X, Y, Z, b, acc);
+                    for (int n = 0; n <= L; ++n) b[n] *= c.w;
+                    f64_accumulate<L>(X, Y, Z, b, acc);
+                }
             }
+        }
+        if (!__any_sync(0xffffffffu, reaches && expanded)) continue;
+        // expanded pairs that reach the tile: each lane (pair) takes the next point
+        // near it, so that the warp makes as many steps as its busiest lane has
+        // near points
+        unsigned near = 0;
+        for (int i = 0; i < nt; ++i) {
+            const float4 c = t.x32[s0 + i];
+            near |= f64_is_near(info.x - c.x, info.y - c.y, info.z - c.z, ip + c.w, FT) ? 1u << i : 0u;
+        }
+        if (!expanded) near = 0;
+        int o = 0;
+        while (__any_sync(0xffffffffu, near != 0)) {
+            const bool on = near != 0;
+            if (on) o = __ffs(near) - 1;
+            near &= near - 1;
+            const F64Pt c = t.xyz[s0 + o];
+            const double X = Px - c.x, Y = Py - c.y, Z = Pz - c.z;
+            double b[L + 1];
+            f64_near_minus_far<L>(fma(X, X, fma(Y, Y, Z * Z)), f64_load_rc(a, t, t.cls[s0 + o], pos), on, t.tab, b);
+#pragma unroll
+            for (int n = 0; n <= L; ++n) b[n] *= c.w;
+            f64_accumulate<L>(X, Y, Z, b, acc);
         }
     }
     if (j < a.n)
@@ -716,8 +798,8 @@ __global__ void __launch_bounds__(128, f64_min_blocks(far_nterms(L)))
 // mapping that made the ESP's coefficients) of the rows' sums, written at the
 // kept pair's place (ord) or, without ord, at j
 template <int L>
-__global__ void f64_fold_kernel(F64Pairs a, int rows, const double *__restrict__ S, const int *__restrict__ ord,
-                                int ldw, double *__restrict__ W)
+__global__ void f64_fold_kernel(F64Pairs a, int rows, const double *__restrict__ S, const double *__restrict__ V,
+                                const int *__restrict__ ord, int ldw, double *__restrict__ W)
 {
     constexpr int NC = far_nterms(L);
     constexpr int NH = nherm(L);
@@ -738,6 +820,15 @@ __global__ void f64_fold_kernel(F64Pairs a, int rows, const double *__restrict__
     for (int h = 0; h < NH; ++h) out[h] = 0.0;
 #pragma unroll
     for (int q = 0; q < FC.count; ++q) out[FC.h[q]] = fma(FC.w[q], acc[FC.term[q]], out[FC.h[q]]);
+    if (V) {
+        // the cells' local expansions at the pair (multipole64.cu)
+        constexpr MpMap MM = mp_map(L);
+        double v[(L + 1) * (L + 1)];
+#pragma unroll
+        for (int q = 0; q < (L + 1) * (L + 1); ++q) v[q] = V[(size_t)q * a.n + j];
+#pragma unroll
+        for (int i = 0; i < MM.count; ++i) out[MM.h[i]] = fma(MM.V[i], v[MM.s[i]], out[MM.h[i]]);
+    }
     const int at = ord ? ord[pos] : j;
 #pragma unroll
     for (int h = 0; h < NH; ++h) W[(size_t)h * ldw + at] = g * out[h];
@@ -753,6 +844,7 @@ static F64Points f64_points(pcm_ctx *c)
     t.ntile = c->f64.ntile;
     t.xyz = c->f64.pt_xyz.p;
     t.cls = c->f64.pt_cls.p;
+    t.x32 = c->f64.pt_x32.p;
     t.sph = c->f64.pt_sph.p;
     t.cls_zeta = c->cls_zeta.p;
     t.zmin2 = (float)(c->h_cls_zeta[0] * c->h_cls_zeta[0]) * 0.99999f;
@@ -772,6 +864,9 @@ static F64Pairs f64_pairs(pcm_ctx *c, int k, bool esp)
     a.P = f.P.p;
     a.rc = f.use_rc ? f.rc.p : nullptr;
     a.rec = esp ? f.rec.p + f.roff[k] : nullptr;
+    a.cell = f.mp.pcell.p;
+    a.order = f.mp.on ? f.mp.order.p : nullptr;
+    a.ncell = f.mp.ncell;
     return a;
 }
 
@@ -805,8 +900,15 @@ int f64_grad_point(pcm_ctx *c, const double *dq, double *gk)
         total += rows[k];
     }
     if (total == 0) return PCM_OK;
+    const int far = c->f64.mp.on ? mp_rows(c) : 0;
+    total += far;
     PCM_TRY(c->esp_part.alloc(total * 3 * S));
     double *part = c->esp_part.p;
+    if (far) {
+        PCM_TRY(mp_order(c, MP_EPS_GRAD));
+        PCM_TRY(mp_grad_far(c, part));
+        part += (size_t)far * 3 * S;
+    }
     for (int k = 0; k < 6; ++k) {
         if (rows[k] == 0) continue;
         switch (F64_LSUM[k]) {
@@ -824,10 +926,14 @@ int f64_grad_point(pcm_ctx *c, const double *dq, double *gk)
     return PCM_OK;
 }
 
-int f64_charges(pcm_ctx *c, const double *dq)
+int f64_charges(pcm_ctx *c, const double *dq, bool gradient)
 {
     f64_point_charge_kernel<<<(c->M + 127) / 128, 128, 0, c->stream>>>(c->M, c->f64.pt_idx.p, dq, c->f64.pt_xyz.p);
     PCM_LAUNCHED(c);
+    if (c->f64.mp.on) {
+        PCM_TRY(mp_order(c, gradient ? MP_EPS_GRAD : MP_EPS));
+        PCM_TRY(mp_local(c));
+    }
     return PCM_OK;
 }
 
@@ -839,7 +945,9 @@ static int f64_w_launch(pcm_ctx *c, const F64Pairs &a, const int *ord, double *W
     PCM_TRY(c->f64.S.alloc((size_t)rows * far_nterms(L) * a.n));
     f64_fock_kernel<L><<<dim3(nb, rows), 128, 0, c->stream>>>(a, f64_points(c), c->f64.S.p);
     PCM_LAUNCHED(c);
-    f64_fold_kernel<L><<<nb, 128, 0, c->stream>>>(a, rows, c->f64.S.p, ord, a.n, W);
+    if (c->f64.mp.on) PCM_TRY(mp_l2p(c, L, a.n, a.list, a.first));
+    f64_fold_kernel<L><<<nb, 128, 0, c->stream>>>(a, rows, c->f64.S.p, c->f64.mp.on ? c->f64.mp.V.p : nullptr, ord,
+                                                 a.n, W);
     PCM_LAUNCHED(c);
     return PCM_OK;
 }

@@ -1,7 +1,9 @@
 """PCM_FP64 Fock correction and gradient integrals against the oracle at the
 sizes where their point tiles (32) and sorted pairs begin: surfaces below and
-above the sorting thresholds (1024 points, 4096 pairs), ragged last tiles, and
-more exponent classes than are tabulated (16).  FP64 bars of _parity."""
+above the sorting thresholds (1024 points, 4096 pairs), ragged last tiles, more
+exponent classes than are tabulated (16), and enough pairs (20000) for the
+cells' multipole and local expansions, in a compact and in a stretched molecule
+(more far tiles, higher orders).  FP64 bars of _parity."""
 import numpy as np
 import pytest
 
@@ -19,7 +21,16 @@ def _many_radii(natom, seed):
     return w
 
 
+def _stretched(natom, seed, d_shells):
+    w = workloads.small_cluster(natom, seed=seed, d_shells=d_shells)
+    half = np.arange(natom) >= natom // 2
+    w.mol.xyz[half] += np.array([20.0, -9.0, 5.0])
+    return w
+
+
 CASES = {
+    "cluster45_sp": lambda: workloads.small_cluster(45, seed=35),
+    "stretched52_spd": lambda: _stretched(52, 36, True),
     "water": lambda: workloads.config(0),
     "cluster5_spd": lambda: workloads.small_cluster(5, seed=31, d_shells=True),
     "cluster20_spd": lambda: workloads.small_cluster(20, seed=32, d_shells=True),
