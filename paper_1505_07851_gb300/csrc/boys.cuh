@@ -16,7 +16,8 @@ constexpr double BOYS_TMAX = 48.0;
 constexpr double BOYS_DT = 1.0 / 32.0;
 constexpr double BOYS_INV_DT = 32.0;
 constexpr int BOYS_NROW = 1540;            // rows 0 .. 48*32 (+ margin)
-constexpr int BOYS_STRIDE64 = 16;          // doubles per row: m = 0 .. 15
+constexpr int BOYS_STRIDE64 = 16;          // doubles per row: m = 0 .. 14, then T_i
+constexpr int BOYS_T64 = 15;
 constexpr int BOYS_STRIDE32 = 16;          // floats per row: F_0..F_9 (hi) then the lo parts of F_0..F_5
 constexpr int BOYS_LO32 = 10;              // offset of the lo parts
 constexpr int BOYS_MCOL = 16;              // columns generated
@@ -28,18 +29,38 @@ constexpr int BOYS_MCOL = 16;              // columns generated
 constexpr int BOYS_H32 = BOYS_NROW * BOYS_STRIDE32;
 constexpr int BOYS_ALLOC32 = 2 * BOYS_NROW * BOYS_STRIDE32;
 
+// x / 2 for a normal x or zero, by the exponent: the FP64 pipe is the bound
+__device__ __forceinline__ double half_by_bits(double x)
+{
+    const int h = __double2hiint(x);
+    return __hiloint2double((h & 0x7fffffff) ? h - 0x00100000 : h, __double2loint(x));
+}
+
+// -2 x for a positive normal x
+__device__ __forceinline__ double minus_twice_by_bits(double x)
+{
+    return __hiloint2double((__double2hiint(x) + 0x00100000) ^ 0x80000000, __double2loint(x));
+}
+
+// FP64.  The FP64 pipe bounds the callers, and comparisons and conversions take
+// its slots like an FMA: the branch and the row come from integer operations, T_i
+// from the row's last column, and the scalings by powers of two from the exponent
+// (20 instead of 25 FP64 instructions for an ss interaction, 33 instead of 39 for
+// ps; the same bits).  d is T - T_i exactly.  Potentials of a 100-atom s/p/d cluster
+// 32.3 -> 28.4 ms.
 template <int MM>
 __device__ __forceinline__ void boys_eval(double T, const double *__restrict__ tab, double (&F)[MM + 1])
 {
-    static_assert(MM + 6 < BOYS_STRIDE64, "Boys table too narrow");
-    if (T < BOYS_TMAX) {
-        const int i = min(max(__double2int_rn(T * BOYS_INV_DT), 0), BOYS_NROW - 1);
-        const double d = T - (double)i * BOYS_DT;      // exact: BOYS_DT is a power of two
+    static_assert(MM + 6 < BOYS_T64, "Boys table too narrow");
+    if (__double2hiint(T) < 0x40480000) {              // T < 48 = BOYS_TMAX, T >= 0
+        // adding 1.5 * 2^47 leaves round(32 T) (ties to even) in the low word
+        const int i = __double2loint(T + 211106232532992.0);
         const double *row = tab + (size_t)i * BOYS_STRIDE64;
         double r[MM + 7];
 #pragma unroll
         for (int k = 0; k < MM + 7; ++k) r[k] = __ldg(row + k);
-        const double e1 = -d, e2 = -d * 0.5, e3 = -d * (1.0 / 3.0), e4 = -d * 0.25, e5 = -d * 0.2,
+        const double d = T - __ldg(row + BOYS_T64);
+        const double e1 = -d, e2 = half_by_bits(-d), e3 = -d * (1.0 / 3.0), e4 = half_by_bits(e2), e5 = -d * 0.2,
                      e6 = -d * (1.0 / 6.0);
 #pragma unroll
         for (int m = 0; m <= MM; ++m) {
@@ -52,7 +73,7 @@ __device__ __forceinline__ void boys_eval(double T, const double *__restrict__ t
         }
     } else {
         const double rs = rsqrt(T);
-        const double half_inv_T = 0.5 * rs * rs;
+        const double half_inv_T = half_by_bits(rs) * rs;
         F[0] = 0.88622692545275801365 * rs;           // sqrt(pi) / 2
 #pragma unroll
         for (int m = 1; m <= MM; ++m) F[m] = F[m - 1] * (double)(2 * m - 1) * half_inv_T;

@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(ESP_NT) esp_kernel_f64(int nesp, int seglen, c
                     dot = sD[0][jj] * F[0];
                 } else {
                     double Rn[L + 1];
-                    double m2r = -2.0 * rho, f = 1.0;
+                    double m2r = minus_twice_by_bits(rho), f = 1.0;
 #pragma unroll
                     for (int n = 0; n <= L; ++n) {
                         Rn[n] = f * F[n];

@@ -72,7 +72,7 @@ __global__ void boys_table_kernel(const double *__restrict__ gx, const double *_
         }
         s += 0.5 * h * ps;
     }
-    tab64[(size_t)row * BOYS_STRIDE64 + m] = s;
+    tab64[(size_t)row * BOYS_STRIDE64 + m] = m == BOYS_T64 ? T : s;
     if (m < BOYS_LO32) tab32[(size_t)row * BOYS_STRIDE32 + m] = (float)s;
     if (m < BOYS_STRIDE32 - BOYS_LO32) tab32[(size_t)row * BOYS_STRIDE32 + BOYS_LO32 + m] = (float)(s - (double)(float)s);
     // Horner block for m <= 1 (layout in boys.cuh)
