@@ -113,6 +113,14 @@ struct F64Src {                            // kept pairs of the classes; first s
     const double *Px[6], *Py[6], *Pz[6], *p[6];
     int off[7];
 };
+// pairs of the PCM_MIXED Fock kernels in sorted order (order.cu)
+struct FockOrder {
+    bool on = false;
+    int off[7] = {0, 0, 0, 0, 0, 0, 0};    // first sorted position of each class
+    DBuf<int> ord;                         // sorted position -> pair of its class
+    DBuf<double> p;                        // exponent sums
+    DBuf<float> x32;                       // per class 6 x pairs: split centres
+};
 // cells of the sorted pairs and their expansions (multipole64.cu)
 struct F64Mp {
     bool on = false;
@@ -166,6 +174,7 @@ struct FockJob {
     const double *gp;                    // exponent sums of the pairs
     const float *Phl, *nc, *tiles;       // split pair centres, near constants, point tiles
     const int *tile_cls;                 // class of each point tile
+    const int *ord;                      // place of each pair in W, or null: its own
     double *W;                           // accumulators [nsplit][nherm][npair]
     int npair, ntile, tps, bx, by, pad;  // pairs, point tiles, tiles per split, pair block, split
 };
@@ -197,6 +206,7 @@ struct pcm_ctx {
     pcm::DBuf<float> boys32;
     // PCM_FP64 Fock and gradient integrals
     pcm::F64Int f64;
+    pcm::FockOrder fock_ord, grad_ord;     // PCM_MIXED: kept pairs, ESP pairs of a gradient call
     pcm::DBuf<unsigned> sort_key;          // scratch of sort_pairs
     pcm::DBuf<int> sort_val, sort_cnt;
 
@@ -346,6 +356,11 @@ void gauss_legendre(int n, std::vector<double> &x, std::vector<double> &w);
 int boys_build_tables(pcm_ctx *c);
 // stable radix sort of (key, value) pairs on the context's stream (sort.cu)
 int sort_pairs(pcm_ctx *c, int n, int bits, DBuf<unsigned> &key, DBuf<int> &val);
+// orders of primitive pairs (order.cu)
+F64Box cavity_box(pcm_ctx *c, double cell);
+F64Src kept_pairs(pcm_ctx *c, int off[7]);
+int pair_order(pcm_ctx *c, const F64Src &src, const F64Box &box, bool exponent_first, bool *sorted);
+int fock_order(pcm_ctx *c, const F64Src &src, const float *const x32[6], FockOrder &out);
 // PCM_FP64 integrals (integrals64.cu)
 int f64_build_tables(pcm_ctx *c);
 int f64_prepare(pcm_ctx *c);
@@ -374,11 +389,11 @@ int esp_packed_jobs(int L, int ppt, const EspJob *jobs, int njob, const float *b
 int fock_mixed_finish(pcm_ctx *c, double *ddF);
 // packed FP32x2 ESP with the far-field path (esp_packed.cu): pairs [jbeg, jend) of class pc
 int esp_packed(pcm_ctx *c, PairClass &pc, int L, int ppt, int jbeg, int jend, const int *blk, const int *bcls,
-               int nblk, double *part);
+               int nblk, int nplan, double *part);
 // packed FP32x2 Fock with the far-field path (fock_packed.cu)
 int fock_point_tiles_map(pcm_ctx *c);
-int fock_packed(pcm_ctx *c, int L, int npt, int npair, const double *gp, const float *Phl, DBuf<float> &nbuf,
-                const double *dq, int nsplit, double *W);
+int fock_packed(pcm_ctx *c, int L, int npt, int npair, const double *gp, const float *Phl, const int *ord,
+                DBuf<float> &nbuf, const double *dq, int nsplit, double *W);
 // matrix-free A for PCM_MIXED (matfree.cu)
 struct AFree;
 AFree afree(pcm_ctx *c);
@@ -395,6 +410,7 @@ int check_device_error(pcm_ctx *c, const char *where);
 int fock_mixed_class(pcm_ctx *c, int k, const double *dq, int nsplit, int ksplit, double *W, int npt);
 int fock_mixed_pairs_per_thread(pcm_ctx *c, int L, long long npair);
 int grad_point_mixed(pcm_ctx *c, int *total_rows);
+int grad_order_mixed(pcm_ctx *c);
 int grad_w_mixed(pcm_ctx *c, int k, const double *dq, int nsplit, int ksplit, double *W, int npt);
 int solver_prepare(pcm_ctx *c);
 int operator_build_async(pcm_ctx *c);   // A, 1/A_kk, preconditioner, FP32 A on the side stream

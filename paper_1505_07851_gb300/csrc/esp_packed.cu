@@ -309,21 +309,26 @@ __device__ __forceinline__ void esp_block(const EspJob &jb, const float *__restr
             const float4 n1 = sN[PK_NS + s];
             const float rf0 = n1.z, rf1 = n1.w;
             f2 X[PPT], Y[PPT], Z[PPT], R2[PPT];
-            bool nr = false;
+            bool nr[PPT], any = false;
 #pragma unroll
             for (int q = 0; q < PPT; ++q) {
                 X[q] = (Ax + nxh[q]) + (Bx + nxl[q]);
                 Y[q] = (Ay + nyh[q]) + (By + nyl[q]);
                 Z[q] = (Az + nzh[q]) + (Bz + nzl[q]);
                 R2[q] = fma2(X[q], X[q], fma2(Y[q], Y[q], Z[q] * Z[q]));
-                nr |= (R2[q].v.x < rf0) | (R2[q].v.y < rf1);
+                nr[q] = (R2[q].v.x < rf0) | (R2[q].v.y < rf1);
+                any |= nr[q];
             }
-            if (__any_sync(0xffffffffu, nr)) {
+            if (__any_sync(0xffffffffu, any)) {
+                // the near form only for those of the thread's points that need
+                // it somewhere in the warp
 #pragma unroll
                 for (int q = 0; q < PPT; ++q) {
-                    const f2 vf = far_value<L>(X[q], Y[q], Z[q], R2[q], sG, s);
-                    const f2 vn = near_value<L>(X[q], Y[q], Z[q], R2[q], sN, sD, boys, s);
-                    const f2 val(R2[q].v.x < rf0 ? vn.v.x : vf.v.x, R2[q].v.y < rf1 ? vn.v.y : vf.v.y);
+                    f2 val = far_value<L>(X[q], Y[q], Z[q], R2[q], sG, s);
+                    if (__any_sync(0xffffffffu, nr[q])) {
+                        const f2 vn = near_value<L>(X[q], Y[q], Z[q], R2[q], sN, sD, boys, s);
+                        val = f2(R2[q].v.x < rf0 ? vn.v.x : val.v.x, R2[q].v.y < rf1 ? vn.v.y : val.v.y);
+                    }
                     const f2 y = val - k32[q];
                     const f2 tt = a32[q] + y;
                     k32[q] = (tt - a32[q]) - y;
@@ -392,7 +397,8 @@ __global__ void __launch_bounds__(PK_NT, pk_min_blocks(L, PPT))
     esp_block<L, PPT>(jobs[blockIdx.x], boys, err);
 }
 
-// segments of ntile tiles for nblk point blocks: enough CTAs to fill the GPU
+// segments of ntile tiles for nblk point blocks (packed_plan_blocks, whatever the launch
+// takes): enough CTAs to fill the GPU
 static void pk_plan(int ntile, int nblk, int *tps, int *rows)
 {
     if (ntile <= 0) {
@@ -415,7 +421,7 @@ int esp_packed_rows(int npairs, int nblk)
 
 template <int L, int PPT>
 static int esp_packed_launch(pcm_ctx *c, PairClass &pc, int jbeg, int jend, const int *blk, const int *bcls,
-                             int nblk, double *part)
+                             int nblk, int nplan, double *part)
 {
     using Ly = PkLayout<L>;
     const int ntile = (jend - jbeg + PK_TP - 1) / PK_TP;
@@ -427,7 +433,7 @@ static int esp_packed_launch(pcm_ctx *c, PairClass &pc, int jbeg, int jend, cons
         pc.nesp, jbeg, jend, ntile, c->ncls, c->cls_zeta.p, pc.eP.p, pc.eD.p, pc.tfar.p, pc.tnear.p);
     PCM_LAUNCHED(c);
     int tps, rows;
-    pk_plan(ntile, nblk, &tps, &rows);
+    pk_plan(ntile, nplan, &tps, &rows);
     if (c->jobs) {
         // a batch: the blocks join one launch per class with the other molecules'
         const std::vector<int> &hoff = c->h_pblk[PPT == 4 ? 0 : 1], &hcls = c->h_pbcls[PPT == 4 ? 0 : 1];
@@ -464,12 +470,12 @@ static int esp_packed_launch(pcm_ctx *c, PairClass &pc, int jbeg, int jend, cons
 }
 
 int esp_packed(pcm_ctx *c, PairClass &pc, int L, int ppt, int jbeg, int jend, const int *blk, const int *bcls,
-               int nblk, double *part)
+               int nblk, int nplan, double *part)
 {
 #define PCM_PK(LL)                                                                                   \
     case LL:                                                                                         \
-        return ppt == 4 ? esp_packed_launch<LL, 4>(c, pc, jbeg, jend, blk, bcls, nblk, part)         \
-                        : esp_packed_launch<LL, 2>(c, pc, jbeg, jend, blk, bcls, nblk, part);
+        return ppt == 4 ? esp_packed_launch<LL, 4>(c, pc, jbeg, jend, blk, bcls, nblk, nplan, part)  \
+                        : esp_packed_launch<LL, 2>(c, pc, jbeg, jend, blk, bcls, nblk, nplan, part);
     switch (L) {
         PCM_PK(0)
         PCM_PK(1)

@@ -126,7 +126,8 @@ __device__ __forceinline__ void fock_block(int bx, int by, int npair, const doub
                                            const float *__restrict__ Phl, const float *__restrict__ nc, int ntile,
                                            int tps, const float *__restrict__ tiles,
                                            const int *__restrict__ tile_cls, const float *__restrict__ boys,
-                                           double *__restrict__ W, int *__restrict__ err)
+                                           const int *__restrict__ ord, double *__restrict__ W,
+                                           int *__restrict__ err)
 {
     constexpr int NH = nherm(L);
     constexpr int NSTAGE = 3;
@@ -204,16 +205,15 @@ __device__ __forceinline__ void fock_block(int bx, int by, int npair, const doub
             const f2 Hx(p0.x, p0.y), Hy(p0.z, p0.w), Hz(p1.x, p1.y), Q(p1.z, p1.w);
             const f2 Lx(p2.x, p2.y), Ly(p2.z, p2.w), Lz(p3.x, p3.y);
             f2 X[NPT], Y[NPT], Z[NPT], R2[NPT];
-            bool nr = false;
+            bool nr[NPT];
 #pragma unroll
             for (int i = 0; i < NPT; ++i) {
                 X[i] = (Pxh[i] + Hx) + (Pxl[i] + Lx);
                 Y[i] = (Pyh[i] + Hy) + (Pyl[i] + Ly);
                 Z[i] = (Pzh[i] + Hz) + (Pzl[i] + Lz);
                 R2[i] = fma2(X[i], X[i], fma2(Y[i], Y[i], Z[i] * Z[i]));
-                nr |= (R2[i].v.x < rf[i]) | (R2[i].v.y < rf[i]);
+                nr[i] = (R2[i].v.x < rf[i]) | (R2[i].v.y < rf[i]);
             }
-            const bool general = __any_sync(0xffffffffu, nr);
 #pragma unroll
             for (int i = 0; i < NPT; ++i) {
                 // far form: q (-1)^n (2n-1)!! R^-(2n+1), 1/R with one Newton step
@@ -227,7 +227,7 @@ __device__ __forceinline__ void fock_block(int bx, int by, int npair, const doub
 #pragma unroll
                     for (int n = 1; n <= L; ++n) Rn[n] = (Rn[n - 1] * rs2) * f2(-(float)(2 * n - 1));
                 }
-                if (general) {
+                if (__any_sync(0xffffffffu, nr[i])) {
                     // near form in the lanes that need it: q cn (-2 rho)^n F_n
                     const bool n0 = R2[i].v.x < rf[i], n1 = R2[i].v.y < rf[i];
                     const f2 rhv(rh[i]);
@@ -283,9 +283,10 @@ __device__ __forceinline__ void fock_block(int bx, int by, int npair, const doub
         if (r[i] < npair) {
             // the unit of the accumulators: sqrt(pi) / (2 sqrt(p))
             const double g = 0.88622692545275801365 / sqrt(gp[r[i]]);
+            const int at = ord ? ord[r[i]] : r[i];
 #pragma unroll
             for (int h = 0; h < NH; ++h)
-                W[((size_t)by * NH + h) * npair + r[i]] = g * ((double)ah[i][h] + (double)al[i][h]);
+                W[((size_t)by * NH + h) * npair + at] = g * ((double)ah[i][h] + (double)al[i][h]);
         }
 }
 
@@ -293,10 +294,10 @@ template <int L, int NPT>
 __global__ void __launch_bounds__(FK_NT, fk_min_blocks(L, NPT))
     fock_kernel_f32x2(int npair, const double *__restrict__ gp, const float *__restrict__ Phl,
                       const float *__restrict__ nc, int ntile, int tps, const float *__restrict__ tiles,
-                      const int *__restrict__ tile_cls, const float *__restrict__ boys, double *__restrict__ W,
-                      int *__restrict__ err)
+                      const int *__restrict__ tile_cls, const float *__restrict__ boys, const int *__restrict__ ord,
+                      double *__restrict__ W, int *__restrict__ err)
 {
-    fock_block<L, NPT>(blockIdx.x, blockIdx.y, npair, gp, Phl, nc, ntile, tps, tiles, tile_cls, boys, W, err);
+    fock_block<L, NPT>(blockIdx.x, blockIdx.y, npair, gp, Phl, nc, ntile, tps, tiles, tile_cls, boys, ord, W, err);
 }
 
 // The same for a table of blocks of many molecules (one launch per class)
@@ -305,12 +306,13 @@ __global__ void __launch_bounds__(FK_NT, fk_min_blocks(L, NPT))
     fock_jobs_kernel(const FockJob *__restrict__ jobs, const float *__restrict__ boys, int *__restrict__ err)
 {
     const FockJob &j = jobs[blockIdx.x];
-    fock_block<L, NPT>(j.bx, j.by, j.npair, j.gp, j.Phl, j.nc, j.ntile, j.tps, j.tiles, j.tile_cls, boys, j.W, err);
+    fock_block<L, NPT>(j.bx, j.by, j.npair, j.gp, j.Phl, j.nc, j.ntile, j.tps, j.tiles, j.tile_cls, boys, j.ord,
+                       j.W, err);
 }
 
 template <int L, int NPT>
-static int fock_packed_launch(pcm_ctx *c, int npair, const double *gp, const float *Phl, DBuf<float> &nbuf,
-                              const double *dq, int nsplit, double *W)
+static int fock_packed_launch(pcm_ctx *c, int npair, const double *gp, const float *Phl, const int *ord,
+                              DBuf<float> &nbuf, const double *dq, int nsplit, double *W)
 {
     const int ntile = c->fk_ntile;
     PCM_TRY(c->fk_tiles.alloc((size_t)std::max(1, ntile) * FK_TILE));
@@ -336,6 +338,7 @@ static int fock_packed_launch(pcm_ctx *c, int npair, const double *gp, const flo
                 fj.nc = nbuf.p;
                 fj.tiles = c->fk_tiles.p;
                 fj.tile_cls = c->fk_cls.p;
+                fj.ord = ord;
                 fj.W = W;
                 fj.npair = npair;
                 fj.ntile = ntile;
@@ -349,29 +352,29 @@ static int fock_packed_launch(pcm_ctx *c, int npair, const double *gp, const flo
     }
     dim3 grid(nb, nsplit);
     fock_kernel_f32x2<L, NPT><<<grid, FK_NT, 0, c->stream>>>(npair, gp, Phl, nbuf.p, ntile, tps, c->fk_tiles.p,
-                                                            c->fk_cls.p, c->boys32.p, W, c->dev_err.p);
+                                                            c->fk_cls.p, c->boys32.p, ord, W, c->dev_err.p);
     PCM_LAUNCHED(c);
     return PCM_OK;
 }
 
 // W[nsplit][nherm(L)][npair] over npair primitive pairs (exponent sums gp,
-// split centres Phl: 6 x npair, hi then lo) for charges dq; every split is
-// written (splits without tiles with zeros).  Two pairs per thread for L <= 2.
-int fock_packed(pcm_ctx *c, int L, int npt, int npair, const double *gp, const float *Phl, DBuf<float> &nbuf,
-                const double *dq, int nsplit, double *W)
+// split centres Phl: 6 x npair, hi then lo; pair r's place in W: ord[r], or r
+// without ord) for charges dq; every split is written (splits without tiles with zeros).  Two pairs per thread for L <= 2.
+int fock_packed(pcm_ctx *c, int L, int npt, int npair, const double *gp, const float *Phl, const int *ord,
+                DBuf<float> &nbuf, const double *dq, int nsplit, double *W)
 {
     if (npair <= 0) return PCM_OK;
     const bool two = npt == 2 && L <= 2;
     switch (L) {
-    case 0: return two ? fock_packed_launch<0, 2>(c, npair, gp, Phl, nbuf, dq, nsplit, W)
-                       : fock_packed_launch<0, 1>(c, npair, gp, Phl, nbuf, dq, nsplit, W);
-    case 1: return two ? fock_packed_launch<1, 2>(c, npair, gp, Phl, nbuf, dq, nsplit, W)
-                       : fock_packed_launch<1, 1>(c, npair, gp, Phl, nbuf, dq, nsplit, W);
-    case 2: return two ? fock_packed_launch<2, 2>(c, npair, gp, Phl, nbuf, dq, nsplit, W)
-                       : fock_packed_launch<2, 1>(c, npair, gp, Phl, nbuf, dq, nsplit, W);
-    case 3: return fock_packed_launch<3, 1>(c, npair, gp, Phl, nbuf, dq, nsplit, W);
-    case 4: return fock_packed_launch<4, 1>(c, npair, gp, Phl, nbuf, dq, nsplit, W);
-    case 5: return fock_packed_launch<5, 1>(c, npair, gp, Phl, nbuf, dq, nsplit, W);
+    case 0: return two ? fock_packed_launch<0, 2>(c, npair, gp, Phl, ord, nbuf, dq, nsplit, W)
+                       : fock_packed_launch<0, 1>(c, npair, gp, Phl, ord, nbuf, dq, nsplit, W);
+    case 1: return two ? fock_packed_launch<1, 2>(c, npair, gp, Phl, ord, nbuf, dq, nsplit, W)
+                       : fock_packed_launch<1, 1>(c, npair, gp, Phl, ord, nbuf, dq, nsplit, W);
+    case 2: return two ? fock_packed_launch<2, 2>(c, npair, gp, Phl, ord, nbuf, dq, nsplit, W)
+                       : fock_packed_launch<2, 1>(c, npair, gp, Phl, ord, nbuf, dq, nsplit, W);
+    case 3: return fock_packed_launch<3, 1>(c, npair, gp, Phl, ord, nbuf, dq, nsplit, W);
+    case 4: return fock_packed_launch<4, 1>(c, npair, gp, Phl, ord, nbuf, dq, nsplit, W);
+    case 5: return fock_packed_launch<5, 1>(c, npair, gp, Phl, ord, nbuf, dq, nsplit, W);
     }
     return PCM_ERR_ARG;
 }

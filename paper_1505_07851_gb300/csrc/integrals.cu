@@ -903,6 +903,7 @@ int grad_integrals(pcm_ctx *c, const double *dP, const double *dq, double *gk, d
                                                                                   gk);
             PCM_LAUNCHED(c);
         }
+        PCM_TRY(grad_order_mixed(c));
     } else {
         PCM_TRY(f64_grad_point(c, dq, gk));
         PCM_TRY(f64_charges(c, dq, true));

@@ -23,17 +23,16 @@
 
 #include "common.cuh"
 #include "context.h"
+#include "curve.cuh"
 #include "f64.cuh"
 #include "multipole64.cuh"
 
 namespace pcm {
 
 constexpr int F64_LSUM[6] = {0, 1, 2, 2, 3, 4};
-constexpr int F64_HBITS = 5;              // cells per side of the pairs' grid: 2^5
+constexpr int F64_SORT_POINTS = 1024;     // fewer points than this stay in library order
 constexpr double F64_CELL = 3.0;          // side of a cell (bohr)
-constexpr int F64_PBITS = 4;              // exponent bins within a cell
 constexpr int F64_PTBITS = 6;             // cells per side of the points' grid
-constexpr int F64_SORT_MIN = 4096;        // fewer pairs than this stay in kept order, fewer points than a quarter too
 constexpr int F64_RC_CLASSES = 16;        // up to this many exponent classes rho and cn are tabulated per (class, pair)
 // from this many pairs and points on the cells' expansions are used: setting them up
 // costs about as much per pair as 130 (ss) to 250 (pp) points one by one.  Measured
@@ -129,48 +128,8 @@ int f64_build_tables(pcm_ctx *c)
 }
 
 // ---------------------------------------------------------------------------
-// orders: a Hilbert curve over a cubic grid (Skilling, AIP Conf. Proc. 707, 381
-// (2004): axes to transposed index by Gray decoding of the exchanged bits)
+// orders of points and pairs
 // ---------------------------------------------------------------------------
-template <int BITS>
-__device__ __forceinline__ unsigned hilbert3(unsigned x, unsigned y, unsigned z)
-{
-    unsigned X[3] = {x, y, z};
-    for (unsigned q = 1u << (BITS - 1); q > 1; q >>= 1) {
-        const unsigned p = q - 1;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            if (X[i] & q) {
-                X[0] ^= p;
-            } else {
-                const unsigned t = (X[0] ^ X[i]) & p;
-                X[0] ^= t;
-                X[i] ^= t;
-            }
-        }
-    }
-    X[1] ^= X[0];
-    X[2] ^= X[1];
-    unsigned t = 0;
-    for (unsigned q = 1u << (BITS - 1); q > 1; q >>= 1)
-        if (X[2] & q) t ^= q - 1;
-    unsigned h = 0;
-    for (int b = BITS - 1; b >= 0; --b)
-        for (int i = 0; i < 3; ++i) h = (h << 1) | (((X[i] ^ t) >> b) & 1u);
-    return h;
-}
-
-template <int BITS>
-__device__ __forceinline__ unsigned curve_key(double x, double y, double z, const F64Box &b)
-{
-    const int top = (1 << BITS) - 1;
-    const double s = (double)(1 << BITS) * b.inv;
-    const int i = min(max((int)((x - b.lo[0]) * s), 0), top);
-    const int j = min(max((int)((y - b.lo[1]) * s), 0), top);
-    const int k = min(max((int)((z - b.lo[2]) * s), 0), top);
-    return hilbert3<BITS>(i, j, k);
-}
-
 __global__ void f64_point_key_kernel(int M, const double *__restrict__ px, const double *__restrict__ py,
                                      const double *__restrict__ pz, F64Box box, unsigned *__restrict__ key,
                                      int *__restrict__ val)
@@ -231,18 +190,6 @@ __device__ __forceinline__ int f64_class_of(const F64Src &s, int g)
     return k;
 }
 
-// class, cell along the curve, exponent bin (half octaves from 0.2, ascending)
-__global__ void f64_pair_key_kernel(int n, F64Src src, F64Box box, unsigned *__restrict__ key, int *__restrict__ val)
-{
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= n) return;
-    const int k = f64_class_of(src, g), r = g - src.off[k];
-    const unsigned h = curve_key<F64_HBITS>(src.Px[k][r], src.Py[k][r], src.Pz[k][r], box);
-    const int pb = min(max((int)floorf(2.f * log2f(5.f * (float)src.p[k][r])), 0), (1 << F64_PBITS) - 1);
-    key[g] = ((unsigned)k << (3 * F64_HBITS + F64_PBITS)) | (h << F64_PBITS) | (unsigned)pb;
-    val[g] = g;
-}
-
 // rho and cn of f64.cuh for exponent z2 = zeta^2
 __device__ __forceinline__ double2 f64_rho_cn(double p, double z2)
 {
@@ -275,38 +222,16 @@ int f64_prepare(pcm_ctx *c)
 {
     F64Int &f = c->f64;
     const int M = c->M;
-    F64Box box;
-    double ext = 1e-3;
-    for (int d = 0; d < 3; ++d) {
-        double lo = 1e300, hi = -1e300;
-        for (int I = 0; I < c->natom; ++I) {
-            lo = std::min(lo, c->h_xyz[3 * I + d] - c->h_radius[I]);
-            hi = std::max(hi, c->h_xyz[3 * I + d] + c->h_radius[I]);
-        }
-        box.lo[d] = lo;
-        ext = std::max(ext, hi - lo);
-    }
-    // cells of F64_CELL (larger when the cavity has more than 32 of them a side)
-    const double cell = std::max(F64_CELL, ext * (1.0 + 1e-9) / (1 << F64_HBITS));
-    box.inv = 1.0 / (cell * (1 << F64_HBITS));
-    F64Src src;
-    int n = 0;
-    for (int k = 0; k < 6; ++k) {
-        src.off[k] = f.off[k] = n;
-        src.Px[k] = c->cls[k].Px.p;
-        src.Py[k] = c->cls[k].Py.p;
-        src.Pz[k] = c->cls[k].Pz.p;
-        src.p[k] = c->cls[k].p.p;
-        n += c->cls[k].npair;
-    }
-    src.off[6] = f.off[6] = n;
+    const F64Box box = cavity_box(c, F64_CELL);
+    const F64Src src = kept_pairs(c, f.off);
+    const int n = f.off[6];
     f.ntile = (M + 31) / 32;
     PCM_TRY(f.pt_idx.alloc(M));
     PCM_TRY(f.pt_cls.alloc(M));
     PCM_TRY(f.pt_xyz.alloc(M));
     PCM_TRY(f.pt_x32.alloc(M));
     PCM_TRY(f.pt_sph.alloc(f.ntile));
-    const bool sort_pts = M >= F64_SORT_MIN / 4;
+    const bool sort_pts = M >= F64_SORT_POINTS;
     if (sort_pts) {
         PCM_TRY(f.key.alloc(M));
         PCM_TRY(f.val.alloc(M));
@@ -327,19 +252,14 @@ int f64_prepare(pcm_ctx *c)
     PCM_TRY(f.info.alloc(n));
     f.use_rc = c->ncls <= F64_RC_CLASSES;
     if (f.use_rc) PCM_TRY(f.rc.alloc((size_t)c->ncls * n));
-    const bool sort_pr = n >= F64_SORT_MIN;
-    if (sort_pr) {
-        PCM_TRY(f.key.alloc(n));   // the sort may have exchanged these with its scratch
-        PCM_TRY(f.val.alloc(n));
-        f64_pair_key_kernel<<<(n + 127) / 128, 128, 0, c->stream>>>(n, src, box, f.key.p, f.val.p);
-        PCM_LAUNCHED(c);
-        PCM_TRY(sort_pairs(c, n, 3 + 3 * F64_HBITS + F64_PBITS, f.key, f.val));
-    }
-    f64_pair_gather_kernel<<<(n + 127) / 128, 128, 0, c->stream>>>(n, src, sort_pr ? f.val.p : nullptr, c->ncls,
+    // within a cell by exponent
+    bool sorted;
+    PCM_TRY(pair_order(c, src, box, false, &sorted));
+    f64_pair_gather_kernel<<<(n + 127) / 128, 128, 0, c->stream>>>(n, src, sorted ? f.val.p : nullptr, c->ncls,
                                                                   c->cls_zeta.p, f.ord.p, f.P.p, f.info.p,
                                                                   f.use_rc ? f.rc.p : nullptr);
     PCM_LAUNCHED(c);
-    if (n >= F64_MP_PAIRS && M >= F64_MP_POINTS) PCM_TRY(mp_prepare(c, box, src, F64_HBITS, F64_PBITS));
+    if (n >= F64_MP_PAIRS && M >= F64_MP_POINTS) PCM_TRY(mp_prepare(c, box, src, CURVE_HBITS, CURVE_PBITS));
     return PCM_OK;
 }
 

@@ -842,7 +842,8 @@ static void esp_plan(int n, int nblk, int *seglen, int *rows)
 }
 
 template <int L, int PPT, bool PACKED>
-static int esp_mixed_launch(pcm_ctx *c, PairClass &pc, int k, const int *blk, const int *bcls, int nblk, double *part)
+static int esp_mixed_launch(pcm_ctx *c, PairClass &pc, int k, const int *blk, const int *bcls, int nblk, int nplan,
+                            double *part)
 {
     constexpr int NH = nherm(L);
     constexpr int F = 3 + 2 * NH;
@@ -860,7 +861,7 @@ static int esp_mixed_launch(pcm_ctx *c, PairClass &pc, int k, const int *blk, co
     }
     if (c->have_events) PCM_CUDA(cudaEventRecord(c->ev_a[k], c->stream));
     int sl, rows;
-    esp_plan(ns, nblk, &sl, &rows);
+    esp_plan(ns, nplan, &sl, &rows);
     if (rows > 0) {
         dim3 grid(nblk, rows);
         esp_kernel_f32<L, true, PPT><<<grid, MESP_NT, 0, c->stream>>>(n, 0, ns, sl, pc.eX32.p, pc.eC32.p, blk, bcls,
@@ -868,11 +869,11 @@ static int esp_mixed_launch(pcm_ctx *c, PairClass &pc, int k, const int *blk, co
         PCM_LAUNCHED(c);
         part += (size_t)rows * c->M;
     }
-    esp_plan(nx, nblk, &sl, &rows);
+    esp_plan(nx, nplan, &sl, &rows);
     if (rows > 0) {
         dim3 grid(nblk, rows);
         if constexpr (PACKED) {
-            PCM_TRY(esp_packed(c, pc, L, PPT, ns, n, blk, bcls, nblk, part));
+            PCM_TRY(esp_packed(c, pc, L, PPT, ns, n, blk, bcls, nblk, nplan, part));
         } else {
             esp_kernel_f32<L, false, PPT><<<grid, MESP_NT, 0, c->stream>>>(n, ns, n, sl, pc.eX32.p, pc.eC32.p, blk,
                                                                             bcls, c->p32.p, c->p32lo.p, c->boys32.p,
@@ -968,12 +969,22 @@ static int esp_ms_launch(pcm_ctx *c, PairClass &pc, int k, const int *blk, const
     return PCM_OK;
 }
 
+// Point blocks by which the packed variants cut a class's pairs into segments: the
+// same for 4 and 2 points per thread, so that the autotuner's choice between them,
+// which goes by the clock, does not change the sums.  2 points per thread, and 4 for
+// the s pairs of tuned batches (the usual choice there).
+static int packed_plan_blocks(const pcm_ctx *c, int k, const int nb[2])
+{
+    return c->jobs && c->opt.autotune && CLASS_L[k] == 0 ? nb[0] : nb[1];
+}
+
 // Variants of the FP32 ESP: pair-driven with 4 (v = 0) or 2 (v = 1) points per
 // thread (two pairs per packed instruction unless the context asks for scalar
 // FP32 instructions); MS-driven (v = 2).
 static int esp_launch_variant(pcm_ctx *c, int k, int v, DBuf<int> *blk, DBuf<int> *bcls, const int nb[2], double *part)
 {
     PairClass &pc = c->cls[k];
+    const int np = packed_plan_blocks(c, k, nb);
     if (v == 2) {
         const int d = esp_default_ppt(CLASS_L[k], false) == 4 ? 0 : 1;
         switch (CLASS_L[k]) {
@@ -986,10 +997,10 @@ static int esp_launch_variant(pcm_ctx *c, int k, int v, DBuf<int> *blk, DBuf<int
 #define PCM_ESPV(LL)                                                                                         \
     case LL:                                                                                                 \
         if (c->opt.fp32x2)                                                                                   \
-            return v == 0 ? esp_mixed_launch<LL, 4, true>(c, pc, k, blk[0].p, bcls[0].p, nb[0], part)        \
-                          : esp_mixed_launch<LL, 2, true>(c, pc, k, blk[1].p, bcls[1].p, nb[1], part);       \
-        return v == 0 ? esp_mixed_launch<LL, 4, false>(c, pc, k, blk[0].p, bcls[0].p, nb[0], part)           \
-                      : esp_mixed_launch<LL, 2, false>(c, pc, k, blk[1].p, bcls[1].p, nb[1], part);
+            return v == 0 ? esp_mixed_launch<LL, 4, true>(c, pc, k, blk[0].p, bcls[0].p, nb[0], np, part)      \
+                          : esp_mixed_launch<LL, 2, true>(c, pc, k, blk[1].p, bcls[1].p, nb[1], np, part);     \
+        return v == 0 ? esp_mixed_launch<LL, 4, false>(c, pc, k, blk[0].p, bcls[0].p, nb[0], nb[0], part)      \
+                      : esp_mixed_launch<LL, 2, false>(c, pc, k, blk[1].p, bcls[1].p, nb[1], nb[1], part);
     switch (CLASS_L[k]) {
         PCM_ESPV(0)
         PCM_ESPV(1)
@@ -1012,7 +1023,7 @@ static int esp_rows(pcm_ctx *c, int k, int nblk)
 // partial-sum rows of variant v of class k
 static int esp_rows_v(pcm_ctx *c, int k, int v, const int nb[2])
 {
-    if (v < 2) return esp_rows(c, k, nb[v]);
+    if (v < 2) return esp_rows(c, k, c->opt.fp32x2 ? packed_plan_blocks(c, k, nb) : nb[v]);
     const int d = esp_default_ppt(CLASS_L[k], false) == 4 ? 0 : 1;
     int sl, r1, mrows, ns, ks;
     esp_plan(c->cls[k].nesp_same, nb[d], &sl, &r1);
@@ -1131,7 +1142,13 @@ int fock_mixed_class(pcm_ctx *c, int k, const double *dq, int nsplit, int ksplit
     const int per = MF_NT * npt;
     const int nb = (pc.npair + per - 1) / per;
     dim3 grid(nb, nsplit);
-    if (c->opt.fp32x2) return fock_packed(c, CLASS_L[k], npt, pc.npair, pc.p.p, pc.Pxyz32.p, pc.fnear, dq, nsplit, W);
+    if (c->opt.fp32x2) {
+        const FockOrder &o = c->fock_ord;
+        if (!o.on)
+            return fock_packed(c, CLASS_L[k], npt, pc.npair, pc.p.p, pc.Pxyz32.p, nullptr, pc.fnear, dq, nsplit, W);
+        return fock_packed(c, CLASS_L[k], npt, pc.npair, o.p.p + o.off[k], o.x32.p + 6 * (size_t)o.off[k],
+                           o.ord.p + o.off[k], pc.fnear, dq, nsplit, W);
+    }
     switch (CLASS_L[k]) {
 #define PCM_FOCK_F32(LL)                                                                                           \
     case LL:                                                                                                       \
@@ -1238,6 +1255,28 @@ static void grad_w_launch(pcm_ctx *c, PairClass &pc, const double *dq, dim3 grid
                                                                c->ncls, c->cls_off.p, c->cls_zeta.p, c->boys32.p, W);
 }
 
+// sorted order of the ESP pairs for grad_w_mixed (after the point-part preparation)
+int grad_order_mixed(pcm_ctx *c)
+{
+    c->grad_ord.on = false;
+    if (!c->opt.fp32x2) return PCM_OK;
+    F64Src src;
+    const float *x32[6];
+    int n = 0;
+    for (int k = 0; k < 6; ++k) {
+        const PairClass &pc = c->cls[k];
+        src.off[k] = n;
+        src.Px[k] = pc.eP.p;
+        src.Py[k] = pc.eP.p + pc.nesp;
+        src.Pz[k] = pc.eP.p + 2 * (size_t)pc.nesp;
+        src.p[k] = pc.eP.p + 3 * (size_t)pc.nesp;
+        x32[k] = pc.eX32.p;
+        n += pc.nesp;
+    }
+    src.off[6] = n;
+    return fock_order(c, src, x32, c->grad_ord);
+}
+
 // W accumulation of the integral gradient: the Fock contraction with R up to
 // L + 1 over the ESP pairs (the packed far-field kernel of fock_packed.cu by
 // default; one pair per thread from L + 1 = 4 on)
@@ -1249,8 +1288,14 @@ int grad_w_mixed(pcm_ctx *c, int k, const double *dq, int nsplit, int ksplit, do
     const int per = MF_NT * npt;
     const int nb = (pc.nesp + per - 1) / per;
     dim3 grid(nb, nsplit);
-    if (c->opt.fp32x2)
-        return fock_packed(c, L1, npt, pc.nesp, pc.eP.p + 3 * (size_t)pc.nesp, pc.eX32.p, pc.fnear, dq, nsplit, W);
+    if (c->opt.fp32x2) {
+        const FockOrder &o = c->grad_ord;
+        if (!o.on)
+            return fock_packed(c, L1, npt, pc.nesp, pc.eP.p + 3 * (size_t)pc.nesp, pc.eX32.p, nullptr, pc.fnear, dq,
+                               nsplit, W);
+        return fock_packed(c, L1, npt, pc.nesp, o.p.p + o.off[k], o.x32.p + 6 * (size_t)o.off[k], o.ord.p + o.off[k],
+                           pc.fnear, dq, nsplit, W);
+    }
     switch (L1) {
     case 1: grad_w_launch<1>(c, pc, dq, grid, ksplit, W, npt); break;
     case 2: grad_w_launch<2>(c, pc, dq, grid, ksplit, W, npt); break;

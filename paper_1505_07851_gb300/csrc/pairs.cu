@@ -401,8 +401,13 @@ int basis_build(pcm_ctx *c, int nshell, const int *shell_atom, const int *shell_
         c->pl_nprim = c->h_sh_nprim;
         c->pair_layout_ok = true;
     }
-    if (c->opt.precision == PCM_FP64) PCM_TRY(f64_prepare(c));
-    return PCM_OK;
+    if (c->opt.precision == PCM_FP64) return f64_prepare(c);
+    c->fock_ord.on = false;
+    if (!c->opt.fp32x2) return PCM_OK;
+    int first[7];
+    const float *x32[6];
+    for (int k = 0; k < 6; ++k) x32[k] = c->cls[k].Pxyz32.p;
+    return fock_order(c, kept_pairs(c, first), x32, c->fock_ord);
 }
 
 }  // namespace pcm
