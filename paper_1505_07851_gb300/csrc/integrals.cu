@@ -246,11 +246,12 @@ __global__ void esp_reduce_kernel(int M, int nseg, const double *__restrict__ pa
     c[k] = s;
 }
 
-// Fock epilogue: one thread per shell pair.  For each kept primitive pair of
-// the shell pair, L_ab = -(2 pi/p) K sum_tuv E^{ab}_tuv W_tuv is contracted
-// with c_a c_b (Eq. 16) and summed in pair order (Eq. 17).  A diagonal shell
+// Fock epilogue: EPI_LANES lanes per shell pair share its kept primitive pairs.
+// For each, L_ab = -(2 pi/p) K sum_tuv E^{ab}_tuv W_tuv is contracted with c_a c_b
+// (Eq. 16); the lanes' sums are added by a butterfly (Eq. 17).  A diagonal shell
 // pair's off-diagonal primitive pair also adds its mirror image.  Both dF
 // blocks (A,B) and (B,A) are written; every element of dF is written.
+constexpr int EPI_LANES = 8;
 template <int LA, int LB>
 __global__ void fock_epilogue_kernel(int nsp, int npair, int nsplit, const int *__restrict__ spA,
                                      const int *__restrict__ spB, const int *__restrict__ sp_start,
@@ -265,14 +266,14 @@ __global__ void fock_epilogue_kernel(int nsp, int npair, int nsplit, const int *
     constexpr int L = LA + LB;
     constexpr int NH = nherm(L);
     constexpr int NA = ncart(LA), NB = ncart(LB);
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= nsp) return;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int s = min(t / EPI_LANES, nsp - 1);
     const int A = spA[s], B = spB[s];
     const double *RA = xyz + 3 * sh_atom[A], *RB = xyz + 3 * sh_atom[B];
     double G[NA * NB];
 #pragma unroll
     for (int t = 0; t < NA * NB; ++t) G[t] = 0.0;
-    for (int r = sp_start[s]; r < sp_start[s + 1]; ++r) {
+    for (int r = sp_start[s] + t % EPI_LANES; r < sp_start[s + 1]; r += EPI_LANES) {
         double w[NH];
 #pragma unroll
         for (int h = 0; h < NH; ++h) {
@@ -310,6 +311,11 @@ __global__ void fock_epilogue_kernel(int nsp, int npair, int nsplit, const int *
             }
         }
     }
+#pragma unroll
+    for (int i = 0; i < NA * NB; ++i)
+#pragma unroll
+        for (int o = EPI_LANES / 2; o > 0; o >>= 1) G[i] += __shfl_xor_sync(0xffffffffu, G[i], o);
+    if (t % EPI_LANES != 0 || t / EPI_LANES >= nsp) return;
     const int fa = sh_bf[A], fb = sh_bf[B];
 #pragma unroll
     for (int a = 0; a < NA; ++a)
@@ -708,7 +714,7 @@ static int fock_tune(pcm_ctx *c, int k, int L, const double *dq)
 template <int LA, int LB>
 static void fock_epilogue(pcm_ctx *c, PairClass &pc, int nsplit, const double *W, double *ddF)
 {
-    fock_epilogue_kernel<LA, LB><<<(pc.nsp + 127) / 128, 128, 0, c->stream>>>(
+    fock_epilogue_kernel<LA, LB><<<(unsigned)(((long long)pc.nsp * EPI_LANES + 127) / 128), 128, 0, c->stream>>>(
         pc.nsp, pc.npair, nsplit, pc.spA.p, pc.spB.p, pc.sp_start.p, pc.ia.p, pc.ib.p, c->sh_atom.p, c->sh_off.p,
         c->sh_bf.p, c->cnorm.p, c->xyz.p, pc.Px.p, pc.Py.p, pc.Pz.p, pc.p.p, pc.pref.p, W, c->nbf, ddF);
 }
