@@ -44,34 +44,27 @@ __device__ inline double dfact_even(int T)
     return r;
 }
 
-// TS: arithmetic of the Schwarz bound (FP64, or FP32 for PCM_MIXED, where a
-// bound off by 1e-6 relative only moves pairs at the cutoff whose
-// contributions are of the cutoff's size); the pair data are FP64 either way.
-template <int LA, int LB, typename TS>
-__global__ void pair_screen_kernel(long long ncand, int nsp, const long long *__restrict__ sp_cand,
-                                   const int *__restrict__ spA, const int *__restrict__ spB,
-                                   const int *__restrict__ sh_atom, const int *__restrict__ sh_nprim,
-                                   const int *__restrict__ sh_off, const double *__restrict__ exps,
-                                   const double *__restrict__ cnorm, const double *__restrict__ xyz, double thresh,
-                                   int *__restrict__ o_sp, int *__restrict__ o_i, int *__restrict__ o_j,
-                                   double *__restrict__ o_P, double *__restrict__ o_p, double *__restrict__ o_pref,
-                                   double *__restrict__ o_Q, unsigned char *__restrict__ flag)
+// what the screening reads of one class
+struct PairSrc {
+    int nsp;
+    const long long *sp_cand;          // first candidate of each shell pair (nsp + 1)
+    const int *spA, *spB, *sh_atom, *sh_nprim, *sh_off;
+    const double *exps, *cnorm, *xyz;
+};
+
+// shell pair s in [lo, hi] and primitives i, j of candidate g
+__device__ __forceinline__ void pair_locate(const PairSrc &p, long long g, int lo, int hi, int &s, int &i, int &j)
 {
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= ncand) return;
-    // shell pair holding candidate g
-    int lo = 0, hi = nsp - 1;
     while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (sp_cand[mid] <= g) lo = mid;
+        const int mid = (lo + hi + 1) >> 1;
+        if (p.sp_cand[mid] <= g) lo = mid;
         else hi = mid - 1;
     }
-    const int s = lo;
-    const int A = spA[s], B = spB[s];
-    int r = (int)(g - sp_cand[s]);
-    int i, j;
+    s = lo;
+    int r = (int)(g - p.sp_cand[s]);
+    const int A = p.spA[s], B = p.spB[s];
     if (A == B) {
-        const int n = sh_nprim[A];
+        const int n = p.sh_nprim[A];
         i = 0;
         while (r >= n - i) {
             r -= n - i;
@@ -79,14 +72,28 @@ __global__ void pair_screen_kernel(long long ncand, int nsp, const long long *__
         }
         j = i + r;
     } else {
-        const int nb = sh_nprim[B];
+        const int nb = p.sh_nprim[B];
         i = r / nb;
         j = r - i * nb;
     }
-    const double a = exps[sh_off[A] + i], b = exps[sh_off[B] + j];
-    const double *RA = xyz + 3 * sh_atom[A], *RB = xyz + 3 * sh_atom[B];
+}
+
+struct PairValues {
+    double P[3], p, pref, Q;
+};
+
+// Centre, exponent sum, prefactor and Schwarz bound of a primitive pair.  TS:
+// arithmetic of the bound (FP64, or FP32 for PCM_MIXED, where a bound off by 1e-6
+// relative only moves pairs at the cutoff whose contributions are of the cutoff's
+// size); the pair data are FP64 either way.
+template <int LA, int LB, typename TS>
+__device__ __forceinline__ PairValues pair_values(const PairSrc &src, int A, int B, int i, int j)
+{
+    PairValues v;
+    const double a = src.exps[src.sh_off[A] + i], b = src.exps[src.sh_off[B] + j];
+    const double *RA = src.xyz + 3 * src.sh_atom[A], *RB = src.xyz + 3 * src.sh_atom[B];
     const double p = a + b;
-    // one FP64 division per candidate (the FP64 pipe runs at 1/64 of FP32 here)
+    // one FP64 division per pair (the FP64 pipe runs at 1/64 of FP32 here)
     const double ip = 1.0 / p;
     double P[3], ab2 = 0.0;
     for (int d = 0; d < 3; ++d) {
@@ -151,112 +158,254 @@ __global__ void pair_screen_kernel(long long ncand, int nsp, const long long *__
             const double f = comp_factor(LA, ca) * comp_factor(LB, cb);
             qmax = fmax(qmax, f * f * fabs(eri));
         }
-    const double Q = fabs(cnorm[sh_off[A] + i] * cnorm[sh_off[B] + j]) * sqrt(qmax);
-    const bool keep = thresh <= 0.0 || Q >= thresh;
-    flag[g] = keep ? 1 : 0;
-    if (!keep) return;   // only kept candidates are gathered
-    o_sp[g] = s;
-    o_i[g] = i;
-    o_j[g] = j;
-    o_P[3 * g + 0] = P[0];
-    o_P[3 * g + 1] = P[1];
-    o_P[3 * g + 2] = P[2];
-    o_p[g] = p;
-    o_pref[g] = pref;
-    o_Q[g] = Q;
+    v.P[0] = P[0];
+    v.P[1] = P[1];
+    v.P[2] = P[2];
+    v.p = p;
+    v.pref = pref;
+    v.Q = fabs(src.cnorm[src.sh_off[A] + i] * src.cnorm[src.sh_off[B] + j]) * sqrt(qmax);
+    return v;
 }
 
-__global__ void pair_gather_kernel(int n, const int *__restrict__ idx, const int *__restrict__ c_sp,
-                                   const int *__restrict__ c_i, const int *__restrict__ c_j,
-                                   const double *__restrict__ c_P, const double *__restrict__ c_p,
-                                   const double *__restrict__ c_pref, const double *__restrict__ c_Q, int *sp, int *ia,
-                                   int *ib, double *Px, double *Py, double *Pz, double *p, double *pref, double *Q,
-                                   float *P32)
+// FP32 value of a double from its high word (20 mantissa bits, towards zero; values
+// below 2^-126 become that), without the conversion's FP64-pipe slot
+__device__ __forceinline__ float trunc32(double v)
 {
-    int r = blockIdx.x * blockDim.x + threadIdx.x;
+    const int h = __double2hiint(v);
+    const int m = max(h & 0x7fffffff, 0x38100000);
+    return __int_as_float((h & 0x80000000) | (min(m, 0x47efffff) - 0x38000000) << 3);
+}
+
+// log2 of an upper bound of the Schwarz bound from FP32 values: K = e^-x with
+// x = ab R^2 / p and, for the sums over Hermite terms, |E_t| <= (R + 1/2p + 4)^(la + lb)
+// and at most 2^14 terms of size max(1, p)^(la + lb)
+template <int LA, int LB>
+__device__ __forceinline__ float pair_bound_log2(const PairSrc &src, int A, int B, int i, int j)
+{
+    constexpr int LL = LA + LB;
+    const float a = trunc32(src.exps[src.sh_off[A] + i]), b = trunc32(src.exps[src.sh_off[B] + j]);
+    const double *RA = src.xyz + 3 * src.sh_atom[A], *RB = src.xyz + 3 * src.sh_atom[B];
+    float R2 = 0.f;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        // the truncated coordinates are off by up to 2^-20 of themselves
+        const float u = trunc32(RA[d]), w = trunc32(RB[d]);
+        const float t = fmaxf(fabsf(u - w) - 1e-6f * (fabsf(u) + fabsf(w)), 0.f);
+        R2 = fmaf(t, t, R2);
+    }
+    const float p = a + b;
+    const float x = 0.9999f * (a * b / p) * R2;
+    const float lp = __log2f(p);
+    const float lc = __log2f(fabsf(trunc32(src.cnorm[src.sh_off[A] + i]))) +
+                     __log2f(fabsf(trunc32(src.cnorm[src.sh_off[B] + j])));
+    float lq = lc + 2.6f - 1.25f * lp - 1.4426950f * x + 1.f;
+    if (LL > 0) lq += 0.5f * LL * fmaxf(lp, 0.f) + LL * __log2f(sqrtf(R2) + 0.5f / p + 4.1f) + 9.f;
+    return lq;
+}
+
+// Candidates kept (Q >= thresh).  Nearly all candidates of a large molecule are far
+// below the cutoff: the FP32 bound drops them before any FP64 work, which was all of
+// this kernel's time (45 FP64 instructions per candidate; 1000 atoms, 40 M ss
+// candidates: 3.3 ms).
+template <int LA, int LB, typename TS>
+__global__ void __launch_bounds__(128) pair_screen_kernel(long long ncand, PairSrc src, double thresh,
+                                                          float log2_thresh, unsigned char *__restrict__ flag)
+{
+    __shared__ int range[2];
+    const long long g0 = (long long)blockIdx.x * 128;
+    const long long g = g0 + threadIdx.x;
+    // the shell pairs of the block's first and last candidates bound every thread's search
+    if (threadIdx.x < 2) {
+        const long long t = threadIdx.x == 0 ? g0 : (g0 + 127 < ncand ? g0 + 127 : ncand - 1);
+        int lo = 0, hi = src.nsp - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (src.sp_cand[mid] <= t) lo = mid;
+            else hi = mid - 1;
+        }
+        range[threadIdx.x] = lo;
+    }
+    __syncthreads();
+    if (g >= ncand) return;
+    int s, i, j;
+    pair_locate(src, g, range[0], range[1], s, i, j);
+    const int A = src.spA[s], B = src.spB[s];
+    bool keep = thresh <= 0.0;
+    if (!keep && pair_bound_log2<LA, LB>(src, A, B, i, j) >= log2_thresh)
+        keep = pair_values<LA, LB, TS>(src, A, B, i, j).Q >= thresh;
+    flag[g] = keep ? 1 : 0;
+}
+
+// the kept pairs of a class: list[0 .. n) are its kept candidates + base
+template <int LA, int LB, typename TS>
+__global__ void __launch_bounds__(128) pair_gather_kernel(int n, PairSrc src, const int *__restrict__ list, int base,
+                                                          int *__restrict__ sp, int *__restrict__ ia,
+                                                          int *__restrict__ ib, double *__restrict__ Px,
+                                                          double *__restrict__ Py, double *__restrict__ Pz,
+                                                          double *__restrict__ p, double *__restrict__ pref,
+                                                          double *__restrict__ Q, float *__restrict__ P32)
+{
+    const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n) return;
-    const int g = idx[r];
-    sp[r] = c_sp[g];
-    ia[r] = c_i[g];
-    ib[r] = c_j[g];
-    Px[r] = c_P[3 * g + 0];
-    Py[r] = c_P[3 * g + 1];
-    Pz[r] = c_P[3 * g + 2];
-    p[r] = c_p[g];
-    pref[r] = c_pref[g];
-    Q[r] = c_Q[g];
+    int s, i, j;
+    pair_locate(src, list[r] - base, 0, src.nsp - 1, s, i, j);
+    const PairValues v = pair_values<LA, LB, TS>(src, src.spA[s], src.spB[s], i, j);
+    sp[r] = s;
+    ia[r] = i;
+    ib[r] = j;
+    Px[r] = v.P[0];
+    Py[r] = v.P[1];
+    Pz[r] = v.P[2];
+    p[r] = v.p;
+    pref[r] = v.pref;
+    Q[r] = v.Q;
     // FP32 hi/lo split of the centre: hi on a 2^-10 grid, so that differences of
     // hi parts are exact in FP32
     for (int d = 0; d < 3; ++d) {
-        const double v = c_P[3 * g + d];
-        const double h = rint(v * 1024.0) * (1.0 / 1024.0);
+        const double h = rint(v.P[d] * 1024.0) * (1.0 / 1024.0);
         P32[(size_t)d * n + r] = (float)h;
-        P32[(size_t)(3 + d) * n + r] = (float)(v - h);
+        P32[(size_t)(3 + d) * n + r] = (float)(v.P[d] - h);
     }
 }
 
-__global__ void sp_start_kernel(int nsp, const long long *__restrict__ sp_cand, const int *__restrict__ pos,
-                                int *__restrict__ sp_start)
+__device__ __forceinline__ int lower_bound(const int *__restrict__ v, int n, long long x)
 {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s <= nsp) sp_start[s] = pos[sp_cand[s]];
+    int lo = 0, hi = n;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (v[mid] < x) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
+struct ClassBase {
+    long long base[7];                 // first candidate of each class in the group's flags
+};
+
+// kept candidates before each class
+__global__ void class_first_kernel(ClassBase b, const int *__restrict__ list, const int *__restrict__ count,
+                                   int *__restrict__ first)
+{
+    if (threadIdx.x < 7) first[threadIdx.x] = lower_bound(list, *count, b.base[threadIdx.x]);
+}
+
+// first kept pair of each shell pair
+__global__ void sp_start_kernel(int nsp, const long long *__restrict__ sp_cand, const int *__restrict__ list, int n,
+                                int base, int *__restrict__ sp_start)
+{
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s <= nsp) sp_start[s] = lower_bound(list, n, base + sp_cand[s]);
+}
+
+static PairSrc pair_src(pcm_ctx *c, const PairClass &pc)
+{
+    PairSrc s;
+    s.nsp = pc.nsp;
+    s.sp_cand = pc.sp_cand.p;
+    s.spA = pc.spA.p;
+    s.spB = pc.spB.p;
+    s.sh_atom = c->sh_atom.p;
+    s.sh_nprim = c->sh_nprim.p;
+    s.sh_off = c->sh_off.p;
+    s.exps = c->exps.p;
+    s.cnorm = c->cnorm.p;
+    s.xyz = c->xyz.p;
+    return s;
 }
 
 template <int LA, int LB>
-static int screen_class(pcm_ctx *c, PairClass &pc)
+static int screen_launch(pcm_ctx *c, const PairClass &pc, unsigned char *flag)
 {
-    DBuf<int> &c_sp = c->si[0], &c_i = c->si[1], &c_j = c->si[2], &pos = c->si[3];
-    DBuf<double> &c_P = c->sd[0], &c_p = c->sd[1], &c_pref = c->sd[2], &c_Q = c->sd[3];
-    DBuf<unsigned char> &flag = c->su8[0];
-    const long long n = pc.ncand;
-    PCM_TRY(c_sp.alloc(n));
-    PCM_TRY(c_i.alloc(n));
-    PCM_TRY(c_j.alloc(n));
-    PCM_TRY(c_P.alloc(3 * n));
-    PCM_TRY(c_p.alloc(n));
-    PCM_TRY(c_pref.alloc(n));
-    PCM_TRY(c_Q.alloc(n));
-    PCM_TRY(flag.alloc(n));
-    PCM_TRY(pos.alloc(n + 1));
-    if (n > 0) {
-        const unsigned grid = (unsigned)((n + 127) / 128);
-        if (c->opt.precision == PCM_MIXED)
-            pair_screen_kernel<LA, LB, float><<<grid, 128, 0, c->stream>>>(
-                n, pc.nsp, pc.sp_cand.p, pc.spA.p, pc.spB.p, c->sh_atom.p, c->sh_nprim.p, c->sh_off.p, c->exps.p,
-                c->cnorm.p, c->xyz.p, c->opt.schwarz, c_sp.p, c_i.p, c_j.p, c_P.p, c_p.p, c_pref.p, c_Q.p, flag.p);
-        else
-            pair_screen_kernel<LA, LB, double><<<grid, 128, 0, c->stream>>>(
-                n, pc.nsp, pc.sp_cand.p, pc.spA.p, pc.spB.p, c->sh_atom.p, c->sh_nprim.p, c->sh_off.p, c->exps.p,
-                c->cnorm.p, c->xyz.p, c->opt.schwarz, c_sp.p, c_i.p, c_j.p, c_P.p, c_p.p, c_pref.p, c_Q.p, flag.p);
-        PCM_LAUNCHED(c);
-    }
-    DBuf<int> &idx = c->si[4];
-    PCM_TRY(idx.alloc(n));
-    PCM_TRY(compact_flags(c, flag.p, n, idx.p, pos.p, c->iscal.p));
-    int kept = 0;
-    PCM_CUDA(cudaMemcpyAsync(&kept, c->iscal.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    PCM_CUDA(cudaStreamSynchronize(c->stream));
-    pc.npair = kept;
-    PCM_TRY(pc.sp.alloc(kept));
-    PCM_TRY(pc.ia.alloc(kept));
-    PCM_TRY(pc.ib.alloc(kept));
-    PCM_TRY(pc.Px.alloc(kept));
-    PCM_TRY(pc.Py.alloc(kept));
-    PCM_TRY(pc.Pz.alloc(kept));
-    PCM_TRY(pc.p.alloc(kept));
-    PCM_TRY(pc.pref.alloc(kept));
-    PCM_TRY(pc.Q.alloc(kept));
-    PCM_TRY(pc.Pxyz32.alloc(6 * (size_t)kept));
-    if (kept > 0) {
-        pair_gather_kernel<<<(kept + 127) / 128, 128, 0, c->stream>>>(
-            kept, idx.p, c_sp.p, c_i.p, c_j.p, c_P.p, c_p.p, c_pref.p, c_Q.p, pc.sp.p, pc.ia.p, pc.ib.p, pc.Px.p,
-            pc.Py.p, pc.Pz.p, pc.p.p, pc.pref.p, pc.Q.p, pc.Pxyz32.p);
-        PCM_LAUNCHED(c);
-    }
-    PCM_TRY(pc.sp_start.alloc(pc.nsp + 1));
-    sp_start_kernel<<<(pc.nsp + 1 + 127) / 128, 128, 0, c->stream>>>(pc.nsp, pc.sp_cand.p, pos.p, pc.sp_start.p);
+    if (pc.ncand == 0) return PCM_OK;
+    const unsigned grid = (unsigned)((pc.ncand + 127) / 128);
+    const double t = c->opt.schwarz;
+    const float l = t > 0.0 ? (float)log2(t) : 0.f;
+    if (c->opt.precision == PCM_MIXED)
+        pair_screen_kernel<LA, LB, float><<<grid, 128, 0, c->stream>>>(pc.ncand, pair_src(c, pc), t, l, flag);
+    else
+        pair_screen_kernel<LA, LB, double><<<grid, 128, 0, c->stream>>>(pc.ncand, pair_src(c, pc), t, l, flag);
     PCM_LAUNCHED(c);
-    PCM_CUDA(cudaStreamSynchronize(c->stream));  // the scratch slots are reused by the next class
+    return PCM_OK;
+}
+
+template <int LA, int LB>
+static int gather_launch(pcm_ctx *c, PairClass &pc, const int *list, int base)
+{
+    const int n = pc.npair;
+    PCM_TRY(pc.sp.alloc(n));
+    PCM_TRY(pc.ia.alloc(n));
+    PCM_TRY(pc.ib.alloc(n));
+    PCM_TRY(pc.Px.alloc(n));
+    PCM_TRY(pc.Py.alloc(n));
+    PCM_TRY(pc.Pz.alloc(n));
+    PCM_TRY(pc.p.alloc(n));
+    PCM_TRY(pc.pref.alloc(n));
+    PCM_TRY(pc.Q.alloc(n));
+    PCM_TRY(pc.Pxyz32.alloc(6 * (size_t)n));
+    PCM_TRY(pc.sp_start.alloc(pc.nsp + 1));
+    if (pc.nsp == 0) return PCM_OK;
+    sp_start_kernel<<<(pc.nsp + 1 + 127) / 128, 128, 0, c->stream>>>(pc.nsp, pc.sp_cand.p, list, n, base,
+                                                                    pc.sp_start.p);
+    PCM_LAUNCHED(c);
+    if (n == 0) return PCM_OK;
+    if (c->opt.precision == PCM_MIXED)
+        pair_gather_kernel<LA, LB, float><<<(n + 127) / 128, 128, 0, c->stream>>>(
+            n, pair_src(c, pc), list, base, pc.sp.p, pc.ia.p, pc.ib.p, pc.Px.p, pc.Py.p, pc.Pz.p, pc.p.p, pc.pref.p,
+            pc.Q.p, pc.Pxyz32.p);
+    else
+        pair_gather_kernel<LA, LB, double><<<(n + 127) / 128, 128, 0, c->stream>>>(
+            n, pair_src(c, pc), list, base, pc.sp.p, pc.ia.p, pc.ib.p, pc.Px.p, pc.Py.p, pc.Pz.p, pc.p.p, pc.pref.p,
+            pc.Q.p, pc.Pxyz32.p);
+    PCM_LAUNCHED(c);
+    return PCM_OK;
+}
+
+// Screening of the classes [k0, k1) together: flags of all their candidates, one
+// compaction and one synchronisation, then the kept pairs' data.
+static int screen_classes(pcm_ctx *c, int k0, int k1)
+{
+    ClassBase b;
+    long long n = 0;
+    for (int k = 0; k < 7; ++k) {
+        b.base[k] = n;
+        if (k >= k0 && k < k1) n += c->cls[k].ncand;
+    }
+    DBuf<unsigned char> &flag = c->su8[0];
+    DBuf<int> &list = c->si[4];
+    PCM_TRY(flag.alloc(std::max(1LL, n)));
+    PCM_TRY(list.alloc(std::max(1LL, n)));
+    for (int k = k0; k < k1; ++k) {
+        unsigned char *f = flag.p + b.base[k];
+        switch (k) {
+        case 0: PCM_TRY((screen_launch<0, 0>(c, c->cls[k], f))); break;
+        case 1: PCM_TRY((screen_launch<1, 0>(c, c->cls[k], f))); break;
+        case 2: PCM_TRY((screen_launch<1, 1>(c, c->cls[k], f))); break;
+        case 3: PCM_TRY((screen_launch<2, 0>(c, c->cls[k], f))); break;
+        case 4: PCM_TRY((screen_launch<2, 1>(c, c->cls[k], f))); break;
+        case 5: PCM_TRY((screen_launch<2, 2>(c, c->cls[k], f))); break;
+        }
+    }
+    int first[7];
+    PCM_TRY(compact_flags(c, flag.p, n, list.p, nullptr, c->iscal.p + 8));
+    class_first_kernel<<<1, 32, 0, c->stream>>>(b, list.p, c->iscal.p + 8, c->iscal.p);
+    PCM_LAUNCHED(c);
+    PCM_CUDA(cudaMemcpyAsync(first, c->iscal.p, sizeof(first), cudaMemcpyDeviceToHost, c->stream));
+    PCM_CUDA(cudaStreamSynchronize(c->stream));
+    for (int k = k0; k < k1; ++k) {
+        PairClass &pc = c->cls[k];
+        pc.npair = first[k + 1] - first[k];
+        const int *l = list.p + first[k];
+        const int base = (int)b.base[k];
+        switch (k) {
+        case 0: PCM_TRY((gather_launch<0, 0>(c, pc, l, base))); break;
+        case 1: PCM_TRY((gather_launch<1, 0>(c, pc, l, base))); break;
+        case 2: PCM_TRY((gather_launch<1, 1>(c, pc, l, base))); break;
+        case 3: PCM_TRY((gather_launch<2, 0>(c, pc, l, base))); break;
+        case 4: PCM_TRY((gather_launch<2, 1>(c, pc, l, base))); break;
+        case 5: PCM_TRY((gather_launch<2, 2>(c, pc, l, base))); break;
+        }
+    }
     return PCM_OK;
 }
 
@@ -384,16 +533,18 @@ int basis_build(pcm_ctx *c, int nshell, const int *shell_atom, const int *shell_
             // cand is read by the copy before it goes out of scope
             PCM_CUDA(cudaStreamSynchronize(c->stream));
         }
-        switch (k) {
-        case 0: PCM_TRY((screen_class<0, 0>(c, pc))); break;
-        case 1: PCM_TRY((screen_class<1, 0>(c, pc))); break;
-        case 2: PCM_TRY((screen_class<1, 1>(c, pc))); break;
-        case 3: PCM_TRY((screen_class<2, 0>(c, pc))); break;
-        case 4: PCM_TRY((screen_class<2, 1>(c, pc))); break;
-        case 5: PCM_TRY((screen_class<2, 2>(c, pc))); break;
-        }
-        c->pairs_candidate += pc.ncand;
-        c->pairs_kept += pc.npair;
+    }
+    // all classes at once while their candidates can be numbered in 31 bits
+    long long total = 0;
+    for (int k = 0; k < 6; ++k) total += c->cls[k].ncand;
+    if (total < (1LL << 31) - 1) {
+        PCM_TRY(screen_classes(c, 0, 6));
+    } else {
+        for (int k = 0; k < 6; ++k) PCM_TRY(screen_classes(c, k, k + 1));
+    }
+    for (int k = 0; k < 6; ++k) {
+        c->pairs_candidate += c->cls[k].ncand;
+        c->pairs_kept += c->cls[k].npair;
     }
     if (!same_layout) {
         c->pl_atom = c->h_sh_atom;
