@@ -68,8 +68,10 @@ __global__ void esp_flag_kernel(int npair, const int *__restrict__ sp, const int
     flag[(size_t)npair + r] = (kept && !same) ? 1 : 0;
 }
 
+// list[j] - base: flag index of the class's ESP pair j; elist receives its kept pair
 template <int LA, int LB>
-__global__ void esp_coef_kernel(int nesp, const int *__restrict__ list, const int *__restrict__ sp,
+__global__ void esp_coef_kernel(int nesp, const int *__restrict__ list, int base, int npair,
+                                int *__restrict__ elist, const int *__restrict__ sp,
                                 const int *__restrict__ ia, const int *__restrict__ ib, const int *__restrict__ spA,
                                 const int *__restrict__ spB, const int *__restrict__ sh_atom,
                                 const int *__restrict__ sh_off, const int *__restrict__ sh_bf,
@@ -83,7 +85,8 @@ __global__ void esp_coef_kernel(int nesp, const int *__restrict__ list, const in
     constexpr int NH = nherm(L);
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= nesp) return;
-    const int r = list[j];
+    const int f = list[j] - base, r = f < npair ? f : f - npair;
+    elist[j] = r;
     const int s = sp[r];
     const int A = spA[s], B = spB[s];
     const int i1 = ia[r], i2 = ib[r];
@@ -518,35 +521,47 @@ static int launch_esp_class(pcm_ctx *c, PairClass &pc, const int *blk, int nblk,
     return PCM_OK;
 }
 
-template <int LA, int LB>
-static int esp_prepare_class(pcm_ctx *c, PairClass &pc, const double *dP)
+// first index in the compacted list of each class's same-atom and cross-atom flags
+struct EspBounds {
+    int at[13];
+};
+__global__ void esp_bounds_kernel(EspBounds b, const int *__restrict__ list, const int *__restrict__ count,
+                                  int *__restrict__ first)
 {
-    pc.nesp = 0;
+    if (threadIdx.x >= 13) return;
+    int lo = 0, hi = *count;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (list[mid] < b.at[threadIdx.x]) lo = mid + 1;
+        else hi = mid;
+    }
+    first[threadIdx.x] = lo;
+}
+
+template <int LA, int LB>
+static int esp_flag_class(pcm_ctx *c, PairClass &pc, const double *dP, unsigned char *flag)
+{
+    pc.nesp = pc.nesp_same = 0;
     if (pc.npair == 0) return PCM_OK;
-    PCM_TRY(c->flags8.alloc(2 * (size_t)pc.npair));
-    PCM_TRY(pc.elist.alloc(pc.npair));
     esp_flag_kernel<LA, LB><<<(pc.npair + 127) / 128, 128, 0, c->stream>>>(
         pc.npair, pc.sp.p, pc.ia.p, pc.ib.p, pc.spA.p, pc.spB.p, c->sh_bf.p, c->sh_atom.p, pc.Q.p, dP, c->nbf,
-        c->opt.schwarz, c->flags8.p);
+        c->opt.schwarz, flag);
     PCM_LAUNCHED(c);
-    // same-atom pairs first, then the others, each in pair order
-    PCM_TRY(compact_flags(c, c->flags8.p, pc.npair, pc.elist.p, nullptr, c->iscal.p));
-    int cnt[2] = {0, 0};
-    PCM_CUDA(cudaMemcpyAsync(&cnt[0], c->iscal.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    PCM_CUDA(cudaStreamSynchronize(c->stream));
-    PCM_TRY(compact_flags(c, c->flags8.p + pc.npair, pc.npair, pc.elist.p + cnt[0], nullptr, c->iscal.p + 1));
-    PCM_CUDA(cudaMemcpyAsync(&cnt[1], c->iscal.p + 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    PCM_CUDA(cudaStreamSynchronize(c->stream));
-    const int n = cnt[0] + cnt[1];
-    pc.nesp = n;
-    pc.nesp_same = cnt[0];
+    return PCM_OK;
+}
+
+template <int LA, int LB>
+static int esp_coef_class(pcm_ctx *c, PairClass &pc, const double *dP, const int *list, int base)
+{
+    const int n = pc.nesp;
     if (n == 0) return PCM_OK;
     constexpr int NH = nherm(LA + LB);
+    PCM_TRY(pc.elist.alloc(pc.npair));
     PCM_TRY(pc.eP.alloc(4 * (size_t)n));
     PCM_TRY(pc.eD.alloc((size_t)NH * n));
     esp_coef_kernel<LA, LB><<<(n + 127) / 128, 128, 0, c->stream>>>(
-        n, pc.elist.p, pc.sp.p, pc.ia.p, pc.ib.p, pc.spA.p, pc.spB.p, c->sh_atom.p, c->sh_off.p, c->sh_bf.p,
-        c->cnorm.p, c->xyz.p, pc.Px.p, pc.Py.p, pc.Pz.p, pc.p.p, pc.pref.p, dP, c->nbf, pc.eP.p, pc.eD.p);
+        n, list, base, pc.npair, pc.elist.p, pc.sp.p, pc.ia.p, pc.ib.p, pc.spA.p, pc.spB.p, c->sh_atom.p, c->sh_off.p,
+        c->sh_bf.p, c->cnorm.p, c->xyz.p, pc.Px.p, pc.Py.p, pc.Pz.p, pc.p.p, pc.pref.p, dP, c->nbf, pc.eP.p, pc.eD.p);
     PCM_LAUNCHED(c);
     return PCM_OK;
 }
@@ -565,15 +580,50 @@ static int esp_class_stats(pcm_ctx *c)
     return PCM_OK;
 }
 
-// density test and Hermite density coefficients of every class
+// Density test and Hermite density coefficients of every class; in each class the
+// same-atom pairs come first, then the others, each in pair order.  One compaction
+// over the flags of all classes and one synchronisation for their counts.
 int esp_prepare_all(pcm_ctx *c, const double *dP)
 {
-    PCM_TRY((esp_prepare_class<0, 0>(c, c->cls[0], dP)));
-    PCM_TRY((esp_prepare_class<1, 0>(c, c->cls[1], dP)));
-    PCM_TRY((esp_prepare_class<1, 1>(c, c->cls[2], dP)));
-    PCM_TRY((esp_prepare_class<2, 0>(c, c->cls[3], dP)));
-    PCM_TRY((esp_prepare_class<2, 1>(c, c->cls[4], dP)));
-    PCM_TRY((esp_prepare_class<2, 2>(c, c->cls[5], dP)));
+    EspBounds b;
+    long long n = 0;
+    for (int k = 0; k < 6; ++k) {
+        b.at[2 * k] = (int)n;
+        b.at[2 * k + 1] = (int)n + c->cls[k].npair;
+        n += 2LL * c->cls[k].npair;
+    }
+    b.at[12] = (int)n;
+    if (n >= (1LL << 31)) {
+        set_last_error("too many primitive pairs");
+        return PCM_ERR_UNSUPPORTED;
+    }
+    PCM_TRY(c->flags8.alloc(std::max(1LL, n)));
+    PCM_TRY(c->idx32.alloc(std::max(1LL, n)));
+    unsigned char *f = c->flags8.p;
+    PCM_TRY((esp_flag_class<0, 0>(c, c->cls[0], dP, f + b.at[0])));
+    PCM_TRY((esp_flag_class<1, 0>(c, c->cls[1], dP, f + b.at[2])));
+    PCM_TRY((esp_flag_class<1, 1>(c, c->cls[2], dP, f + b.at[4])));
+    PCM_TRY((esp_flag_class<2, 0>(c, c->cls[3], dP, f + b.at[6])));
+    PCM_TRY((esp_flag_class<2, 1>(c, c->cls[4], dP, f + b.at[8])));
+    PCM_TRY((esp_flag_class<2, 2>(c, c->cls[5], dP, f + b.at[10])));
+    if (n == 0) return PCM_OK;
+    int first[13];
+    PCM_TRY(compact_flags(c, f, n, c->idx32.p, nullptr, c->iscal.p + 16));
+    esp_bounds_kernel<<<1, 32, 0, c->stream>>>(b, c->idx32.p, c->iscal.p + 16, c->iscal.p);
+    PCM_LAUNCHED(c);
+    PCM_CUDA(cudaMemcpyAsync(first, c->iscal.p, sizeof(first), cudaMemcpyDeviceToHost, c->stream));
+    PCM_CUDA(cudaStreamSynchronize(c->stream));
+    for (int k = 0; k < 6; ++k) {
+        c->cls[k].nesp_same = first[2 * k + 1] - first[2 * k];
+        c->cls[k].nesp = first[2 * k + 2] - first[2 * k];
+    }
+    const int *l = c->idx32.p;
+    PCM_TRY((esp_coef_class<0, 0>(c, c->cls[0], dP, l + first[0], b.at[0])));
+    PCM_TRY((esp_coef_class<1, 0>(c, c->cls[1], dP, l + first[2], b.at[2])));
+    PCM_TRY((esp_coef_class<1, 1>(c, c->cls[2], dP, l + first[4], b.at[4])));
+    PCM_TRY((esp_coef_class<2, 0>(c, c->cls[3], dP, l + first[6], b.at[6])));
+    PCM_TRY((esp_coef_class<2, 1>(c, c->cls[4], dP, l + first[8], b.at[8])));
+    PCM_TRY((esp_coef_class<2, 2>(c, c->cls[5], dP, l + first[10], b.at[10])));
     return PCM_OK;
 }
 

@@ -90,13 +90,26 @@ __global__ void surface_candidates_kernel(int natom, int n, const double *__rest
     }
 }
 
-// flags of the kept candidates of one exponent class
-__global__ void class_flags_kernel(long long ncand, int n, const unsigned char *__restrict__ keep,
-                                   const int *__restrict__ atom_cls, int e, unsigned char *__restrict__ f)
+// exponent class of each kept candidate
+__global__ void class_key_kernel(int M, int n, const int *__restrict__ idx, const int *__restrict__ atom_cls,
+                                 unsigned *__restrict__ key)
 {
-    long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= ncand) return;
-    f[k] = (keep[k] && atom_cls[k / n] == e) ? 1 : 0;
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < M) key[j] = (unsigned)atom_cls[idx[j] / n];
+}
+
+// first point of each class in the sorted order (off[ncls] = M)
+__global__ void class_offsets_kernel(int M, int ncls, const unsigned *__restrict__ key, int *__restrict__ off)
+{
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e > ncls) return;
+    int lo = 0, hi = M;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (key[mid] < (unsigned)e) lo = mid + 1;
+        else hi = mid;
+    }
+    off[e] = lo;
 }
 
 __global__ void gather_points_kernel(int M, int n, const int *__restrict__ idx, const double *__restrict__ cx,
@@ -401,25 +414,30 @@ int surface_build(pcm_ctx *c, int natom, const double *xyz, const double *Z, con
         natom, n, c->xyz.p, c->radius.p, azeta.p, c->opt.switch_drop, cx.p, cy.p, cz.p, cS.p, keep.p);
     PCM_LAUNCHED(c);
 
-    // compaction class by class into library order
-    PCM_TRY(c->flags8.alloc(ncand));
-    PCM_TRY(c->idx32.alloc(ncand));
+    // kept candidates in candidate order, then a stable sort by class: library order
     PCM_TRY(c->iscal.alloc(64));
-    std::vector<int> counts(c->ncls);
     DBuf<int> &order = c->si[1];
     PCM_TRY(order.alloc(ncand));
+    PCM_TRY(compact_flags(c, keep.p, ncand, order.p, nullptr, c->iscal.p));
     int M = 0;
+    PCM_CUDA(cudaMemcpyAsync(&M, c->iscal.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    PCM_CUDA(cudaStreamSynchronize(c->stream));
     c->h_cls_off.assign(c->ncls + 1, 0);
-    for (int e = 0; e < c->ncls; ++e) {
-        class_flags_kernel<<<(unsigned)((ncand + 255) / 256), 256, 0, c->stream>>>(ncand, n, keep.p, acls.p, e,
-                                                                                  c->flags8.p);
+    c->h_cls_off[c->ncls] = M;
+    if (c->ncls > 1 && M > 0) {
+        DBuf<unsigned> &key = c->f64.key;
+        PCM_TRY(key.alloc(M));
+        PCM_TRY(c->cls_off.alloc(c->ncls + 1));
+        class_key_kernel<<<(M + 255) / 256, 256, 0, c->stream>>>(M, n, order.p, acls.p, key.p);
         PCM_LAUNCHED(c);
-        PCM_TRY(compact_flags(c, c->flags8.p, ncand, order.p + M, nullptr, c->iscal.p));
-        int cnt = 0;
-        PCM_CUDA(cudaMemcpyAsync(&cnt, c->iscal.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+        int bits = 1;
+        while ((1LL << bits) < c->ncls) ++bits;
+        PCM_TRY(sort_pairs(c, M, bits, key, order));
+        class_offsets_kernel<<<(c->ncls + 128) / 128, 128, 0, c->stream>>>(M, c->ncls, key.p, c->cls_off.p);
+        PCM_LAUNCHED(c);
+        PCM_CUDA(cudaMemcpyAsync(c->h_cls_off.data(), c->cls_off.p, (c->ncls + 1) * sizeof(int),
+                                 cudaMemcpyDeviceToHost, c->stream));
         PCM_CUDA(cudaStreamSynchronize(c->stream));
-        M += cnt;
-        c->h_cls_off[e + 1] = M;
     }
     c->M = M;
     if (M == 0) {
