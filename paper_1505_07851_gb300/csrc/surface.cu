@@ -30,7 +30,9 @@ __global__ void atom_zeta_kernel(int natom, const double *__restrict__ radius, d
 //   r_k = X_I + R_I u_i,  zeta_k = zeta_I
 //   S_k = prod_{J != I} (erfc(zeta_k (R_J - d)) + erfc(zeta_k (R_J + d))) / 2
 // (Eq. 9 with erf written as 1 - erfc).  An atom with zeta_k (d - R_J) > 6
-// contributes a factor that rounds to exactly 1 in FP64 and is skipped.
+// contributes a factor that rounds to exactly 1 in FP64 and is skipped; nearly all
+// are, by an FP32 test with a margin (the FP64 test decides the rest; surface of 300
+// atoms 1.09 -> 0.83 ms, of 1000 atoms 5.7 -> 3.8 ms).
 __global__ void surface_candidates_kernel(int natom, int n, const double *__restrict__ xyz,
                                           const double *__restrict__ radius, const double *__restrict__ azeta,
                                           double drop, double *__restrict__ cx, double *__restrict__ cy,
@@ -38,6 +40,7 @@ __global__ void surface_candidates_kernel(int natom, int n, const double *__rest
                                           unsigned char *__restrict__ keep)
 {
     __shared__ double sx[SURF_ATOM_TILE], sy[SURF_ATOM_TILE], sz[SURF_ATOM_TILE], sr[SURF_ATOM_TILE];
+    __shared__ float4 s32[SURF_ATOM_TILE];
     const long long ncand = (long long)natom * n;
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = k < ncand;
@@ -58,6 +61,9 @@ __global__ void surface_candidates_kernel(int natom, int n, const double *__rest
         zk = azeta[I];
     }
     const double reach = 6.0 / zk;
+    // FP32 rounding of two coordinates of up to `big`: below 2^-22 of it
+    const float fx = (float)rx, fy = (float)ry, fz = (float)rz, freach = (float)reach;
+    const float big = fmaxf(fabsf(fx), fmaxf(fabsf(fy), fabsf(fz)));
     double S = 1.0;
     for (int J0 = 0; J0 < natom; J0 += SURF_ATOM_TILE) {
         const int nj = min(SURF_ATOM_TILE, natom - J0);
@@ -67,11 +73,17 @@ __global__ void surface_candidates_kernel(int natom, int n, const double *__rest
             sy[j] = xyz[3 * (J0 + j) + 1];
             sz[j] = xyz[3 * (J0 + j) + 2];
             sr[j] = radius[J0 + j];
+            s32[j] = make_float4((float)sx[j], (float)sy[j], (float)sz[j], (float)sr[j]);
         }
         __syncthreads();
         if (active) {
             for (int j = 0; j < nj; ++j) {
                 if (J0 + j == I) continue;
+                const float4 q = s32[j];
+                const float ux = fx - q.x, uy = fy - q.y, uz = fz - q.z;
+                const float far = (q.w + freach) * 1.00001f +
+                                  1e-6f * (big + fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z))));
+                if (ux * ux + uy * uy + uz * uz > 1.00001f * far * far) continue;
                 const double dx = rx - sx[j], dy = ry - sy[j], dz = rz - sz[j];
                 const double d2 = dx * dx + dy * dy + dz * dz;
                 const double lim = sr[j] + reach;
