@@ -361,97 +361,142 @@ __global__ void grad_point_reduce_kernel(int M, int nseg, const double *__restri
 // (w_ab the density weights of the ESP prologue), and likewise for y, z and
 // for the centre of b.  Written to gfull[d][r] (A) and gfull[3 + d][r] (B) at
 // the kept-pair index r.
+//
+// The components a of the first shell go to the warps of a block, 32 pairs to its
+// lanes; W and the Hermite coefficients of the three directions are shared memory
+// tables (a column per lane), so that every loop bound can be the actual one:
+// t <= a_x + b_x + 1 (and y, z), innermost first with the six outputs sharing the
+// inner sums.  About 5000 FP64 instructions per dd pair; all of t + u + v <= L + 1
+// written out per output takes 36000 (dd pairs of 100 atoms: 1.06 ms).
 template <int LA, int LB>
-__global__ void grad_pair_kernel(int nesp, int npair, int nsplit, const int *__restrict__ elist,
-                                 const int *__restrict__ sp, const int *__restrict__ ia, const int *__restrict__ ib,
-                                 const int *__restrict__ spA, const int *__restrict__ spB,
-                                 const int *__restrict__ sh_atom, const int *__restrict__ sh_off,
-                                 const int *__restrict__ sh_bf, const double *__restrict__ exps,
-                                 const double *__restrict__ cnorm, const double *__restrict__ xyz,
-                                 const double *__restrict__ Px, const double *__restrict__ Py,
-                                 const double *__restrict__ Pz, const double *__restrict__ pp,
-                                 const double *__restrict__ pref, const double *__restrict__ Pm, int nbf,
-                                 const double *__restrict__ W, double *__restrict__ gfull)
+struct GradPairTables {
+    static constexpr int L1 = LA + LB + 1;
+    double w[nherm(L1)][32];
+    double e[3][LA + 2][LB + 2][L1 + 1][32];
+    double red[ncart(LA)][6][32];
+};
+
+template <int LA, int LB>
+__global__ void __launch_bounds__(32 * ncart(LA))
+    grad_pair_kernel(int nesp, int npair, int nsplit, const int *__restrict__ elist, const int *__restrict__ sp,
+                     const int *__restrict__ ia, const int *__restrict__ ib, const int *__restrict__ spA,
+                     const int *__restrict__ spB, const int *__restrict__ sh_atom, const int *__restrict__ sh_off,
+                     const int *__restrict__ sh_bf, const double *__restrict__ exps, const double *__restrict__ cnorm,
+                     const double *__restrict__ xyz, const double *__restrict__ Px, const double *__restrict__ Py,
+                     const double *__restrict__ Pz, const double *__restrict__ pp, const double *__restrict__ pref,
+                     const double *__restrict__ Pm, int nbf, const double *__restrict__ W, double *__restrict__ gfull)
 {
     constexpr int L1 = LA + LB + 1;
     constexpr int NH1 = nherm(L1);
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= nesp) return;
+    constexpr int NA = ncart(LA), NB = ncart(LB);
+    extern __shared__ double gp_smem[];
+    GradPairTables<LA, LB> &T = *reinterpret_cast<GradPairTables<LA, LB> *>(gp_smem);
+    const int lane = threadIdx.x & 31, a = threadIdx.x >> 5;
+    const int j = min(blockIdx.x * 32 + lane, nesp - 1);
+    for (int h = a; h < NH1; h += NA) {
+        double acc = 0.0;
+        for (int g = 0; g < nsplit; ++g) acc += W[((size_t)g * NH1 + h) * nesp + j];
+        T.w[h][lane] = acc;
+    }
     const int r = elist[j];
     const int s = sp[r];
     const int A = spA[s], B = spB[s];
     const int i1 = ia[r], i2 = ib[r];
     const bool mirror = (A != B) || (i1 != i2);
-    double w[NH1];
+    const double inv2p = 0.5 / pp[r];
+    for (int d = a; d < 3; d += NA) {
+        const double P = d == 0 ? Px[r] : (d == 1 ? Py[r] : Pz[r]);
+        E1T<LA + 1, LB + 1> E;
+        hermite_E1T<LA + 1, LB + 1>(P - xyz[3 * sh_atom[A] + d], P - xyz[3 * sh_atom[B] + d], inv2p, E);
 #pragma unroll
-    for (int h = 0; h < NH1; ++h) {
-        double acc = 0.0;
-        for (int g = 0; g < nsplit; ++g) acc += W[((size_t)g * NH1 + h) * nesp + j];
-        w[h] = acc;
+        for (int x = 0; x <= LA + 1; ++x)
+#pragma unroll
+            for (int y = 0; y <= LB + 1; ++y)
+#pragma unroll
+                for (int t = 0; t <= L1; ++t) T.e[d][x][y][t][lane] = E.e[x][y][t];
     }
-    const double p = pp[r];
-    const double P[3] = {Px[r], Py[r], Pz[r]};
-    const double *RA = xyz + 3 * sh_atom[A], *RB = xyz + 3 * sh_atom[B];
-    E1T<LA + 1, LB + 1> Ex, Ey, Ez;
-    const double inv2p = 0.5 / p;
-    hermite_E1T<LA + 1, LB + 1>(P[0] - RA[0], P[0] - RB[0], inv2p, Ex);
-    hermite_E1T<LA + 1, LB + 1>(P[1] - RA[1], P[1] - RB[1], inv2p, Ey);
-    hermite_E1T<LA + 1, LB + 1>(P[2] - RA[2], P[2] - RB[2], inv2p, Ez);
     const double al2 = 2.0 * exps[sh_off[A] + i1], be2 = 2.0 * exps[sh_off[B] + i2];
     const double cc = cnorm[sh_off[A] + i1] * cnorm[sh_off[B] + i2];
     const int fa = sh_bf[A], fb = sh_bf[B];
+    __syncthreads();
+    // derivative factors of one direction: A's centre, B's centre
+    auto dA = [&](int d, int x, int y, int t) {
+        const double v = al2 * T.e[d][x + 1][y][t][lane];
+        return x > 0 ? fma(-(double)x, T.e[d][x > 0 ? x - 1 : 0][y][t][lane], v) : v;
+    };
+    auto dB = [&](int d, int x, int y, int t) {
+        const double v = be2 * T.e[d][x][y + 1][t][lane];
+        return y > 0 ? fma(-(double)y, T.e[d][x][y > 0 ? y - 1 : 0][t][lane], v) : v;
+    };
     double gA[3] = {0.0, 0.0, 0.0}, gB[3] = {0.0, 0.0, 0.0};
+    int ax, ay, az;
+    cart_xyz(LA, a, ax, ay, az);
+#pragma unroll 1
+    for (int b = 0; b < NB; ++b) {
+        int bx, by, bz;
+        cart_xyz(LB, b, bx, by, bz);
+        double wab = Pm[(size_t)(fa + a) * nbf + fb + b];
+        if (mirror) wab += Pm[(size_t)(fb + b) * nbf + fa + a];
+        wab *= comp_factor_i(LA, a) * comp_factor_i(LB, b);
+        double Z0[L1 + 1], ZA[L1 + 1], ZB[L1 + 1];
 #pragma unroll
-    for (int a = 0; a < ncart(LA); ++a) {
-        const int ax = cart_e(LA, a, 0), ay = cart_e(LA, a, 1), az = cart_e(LA, a, 2);
-#pragma unroll
-        for (int b = 0; b < ncart(LB); ++b) {
-            const int bx = cart_e(LB, b, 0), by = cart_e(LB, b, 1), bz = cart_e(LB, b, 2);
-            double wab = Pm[(size_t)(fa + a) * nbf + fb + b];
-            if (mirror) wab += Pm[(size_t)(fb + b) * nbf + fa + a];
-            wab *= cc * comp_factor_i(LA, a) * comp_factor_i(LB, b);
-            // one-dimensional factors: plain, centre-A derivative, centre-B derivative
-            double X0[L1 + 1], XA[L1 + 1], XB[L1 + 1], Y0[L1 + 1], YA[L1 + 1], YB[L1 + 1];
-            double Z0[L1 + 1], ZA[L1 + 1], ZB[L1 + 1];
-#pragma unroll
-            for (int t = 0; t <= L1; ++t) {
-                X0[t] = Ex.e[ax][bx][t];
-                Y0[t] = Ey.e[ay][by][t];
-                Z0[t] = Ez.e[az][bz][t];
-                XA[t] = al2 * Ex.e[ax + 1][bx][t] - (ax > 0 ? ax * Ex.e[ax > 0 ? ax - 1 : 0][bx][t] : 0.0);
-                YA[t] = al2 * Ey.e[ay + 1][by][t] - (ay > 0 ? ay * Ey.e[ay > 0 ? ay - 1 : 0][by][t] : 0.0);
-                ZA[t] = al2 * Ez.e[az + 1][bz][t] - (az > 0 ? az * Ez.e[az > 0 ? az - 1 : 0][bz][t] : 0.0);
-                XB[t] = be2 * Ex.e[ax][bx + 1][t] - (bx > 0 ? bx * Ex.e[ax][bx > 0 ? bx - 1 : 0][t] : 0.0);
-                YB[t] = be2 * Ey.e[ay][by + 1][t] - (by > 0 ? by * Ey.e[ay][by > 0 ? by - 1 : 0][t] : 0.0);
-                ZB[t] = be2 * Ez.e[az][bz + 1][t] - (bz > 0 ? bz * Ez.e[az][bz > 0 ? bz - 1 : 0][t] : 0.0);
+        for (int v = 0; v <= L1; ++v)
+            if (v <= az + bz + 1) {
+                Z0[v] = T.e[2][az][bz][v][lane];
+                ZA[v] = dA(2, az, bz, v);
+                ZB[v] = dB(2, az, bz, v);
             }
-            double sA[3] = {0.0, 0.0, 0.0}, sB[3] = {0.0, 0.0, 0.0};
+        double sA[3] = {0.0, 0.0, 0.0}, sB[3] = {0.0, 0.0, 0.0};
+#pragma unroll 1
+        for (int t = 0; t <= ax + bx + 1; ++t) {
+            double y0 = 0.0, yA = 0.0, yB = 0.0, zA = 0.0, zB = 0.0;
+            const int um = min(ay + by + 1, L1 - t);
+#pragma unroll 1
+            for (int u = 0; u <= um; ++u) {
+                const int vm = min(az + bz + 1, L1 - t - u);
+                double v0 = 0.0, vA = 0.0, vB = 0.0;
 #pragma unroll
-            for (int t = 0; t <= L1; ++t)
-#pragma unroll
-                for (int u = 0; u <= L1 - t; ++u)
-#pragma unroll
-                    for (int v = 0; v <= L1 - t - u; ++v) {
-                        const double wh = w[hidx(t, u, v)];
-                        sA[0] += XA[t] * Y0[u] * Z0[v] * wh;
-                        sA[1] += X0[t] * YA[u] * Z0[v] * wh;
-                        sA[2] += X0[t] * Y0[u] * ZA[v] * wh;
-                        sB[0] += XB[t] * Y0[u] * Z0[v] * wh;
-                        sB[1] += X0[t] * YB[u] * Z0[v] * wh;
-                        sB[2] += X0[t] * Y0[u] * ZB[v] * wh;
+                for (int v = 0; v <= L1; ++v)
+                    if (v <= vm) {
+                        const double wh = T.w[hidx(t, u, v)][lane];
+                        v0 = fma(Z0[v], wh, v0);
+                        vA = fma(ZA[v], wh, vA);
+                        vB = fma(ZB[v], wh, vB);
                     }
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                gA[d] = fma(wab, sA[d], gA[d]);
-                gB[d] = fma(wab, sB[d], gB[d]);
+                const double Y0 = T.e[1][ay][by][u][lane];
+                y0 = fma(Y0, v0, y0);
+                yA = fma(dA(1, ay, by, u), v0, yA);
+                yB = fma(dB(1, ay, by, u), v0, yB);
+                zA = fma(Y0, vA, zA);
+                zB = fma(Y0, vB, zB);
             }
+            const double X0 = T.e[0][ax][bx][t][lane];
+            sA[0] = fma(dA(0, ax, bx, t), y0, sA[0]);
+            sB[0] = fma(dB(0, ax, bx, t), y0, sB[0]);
+            sA[1] = fma(X0, yA, sA[1]);
+            sB[1] = fma(X0, yB, sB[1]);
+            sA[2] = fma(X0, zA, sA[2]);
+            sB[2] = fma(X0, zB, sB[2]);
+        }
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            gA[d] = fma(wab, sA[d], gA[d]);
+            gB[d] = fma(wab, sB[d], gB[d]);
         }
     }
-    const double scale = -pref[r];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        gfull[(size_t)d * npair + r] = scale * gA[d];
-        gfull[(size_t)(3 + d) * npair + r] = scale * gB[d];
+        T.red[a][d][lane] = gA[d];
+        T.red[a][3 + d][lane] = gB[d];
+    }
+    __syncthreads();
+    if (blockIdx.x * 32 + lane >= nesp) return;
+    const double scale = -pref[r] * cc;
+    for (int d = a; d < 6; d += NA) {
+        double v = 0.0;
+#pragma unroll
+        for (int k = 0; k < NA; ++k) v += T.red[k][d][lane];
+        gfull[(size_t)d * npair + r] = scale * v;
     }
 }
 
@@ -916,7 +961,9 @@ static int grad_pair_class(pcm_ctx *c, PairClass &pc, const double *dP, const do
     }
     PCM_TRY(c->g_full.alloc(6 * (size_t)pc.npair));
     PCM_CUDA(cudaMemsetAsync(c->g_full.p, 0, 6 * (size_t)pc.npair * sizeof(double), c->stream));
-    grad_pair_kernel<LA, LB><<<(n + 127) / 128, 128, 0, c->stream>>>(
+    constexpr size_t gp = sizeof(GradPairTables<LA, LB>);
+    PCM_CUDA(cudaFuncSetAttribute(grad_pair_kernel<LA, LB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gp));
+    grad_pair_kernel<LA, LB><<<(n + 31) / 32, 32 * ncart(LA), gp, c->stream>>>(
         n, pc.npair, nsplit, pc.elist.p, pc.sp.p, pc.ia.p, pc.ib.p, pc.spA.p, pc.spB.p, c->sh_atom.p, c->sh_off.p,
         c->sh_bf.p, c->exps.p, c->cnorm.p, c->xyz.p, pc.Px.p, pc.Py.p, pc.Pz.p, pc.p.p, pc.pref.p, dP, c->nbf,
         c->fock_W.p, c->g_full.p);

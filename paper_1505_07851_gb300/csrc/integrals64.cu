@@ -714,6 +714,21 @@ __global__ void __launch_bounds__(128, f64_min_blocks(far_nterms(L)))
         for (int k = 0; k < NC; ++k) S[((size_t)blockIdx.y * NC + k) * a.n + j] = acc[k];
 }
 
+// sums of the rows into the first one, an accumulator per thread: classes with few
+// pairs are split over up to a row per tile
+__global__ void f64_rows_kernel(size_t n, int rows, double *__restrict__ S)
+{
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    int r = 0;
+    for (; r + 4 <= rows; r += 4)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] += S[(size_t)(r + k) * n + i];
+    for (; r < rows; ++r) v[0] += S[(size_t)r * n + i];
+    S[i] = (v[0] + v[1]) + (v[2] + v[3]);
+}
+
 // W_tuv = sqrt(pi) / (2 sqrt(p)) sum over the terms (the transpose of the
 // mapping that made the ESP's coefficients) of the rows' sums, written at the
 // kept pair's place (ord) or, without ord, at j
@@ -865,8 +880,13 @@ static int f64_w_launch(pcm_ctx *c, const F64Pairs &a, const int *ord, double *W
     PCM_TRY(c->f64.S.alloc((size_t)rows * far_nterms(L) * a.n));
     f64_fock_kernel<L><<<dim3(nb, rows), 128, 0, c->stream>>>(a, f64_points(c), c->f64.S.p);
     PCM_LAUNCHED(c);
+    if (rows > 2) {
+        const size_t ns = (size_t)far_nterms(L) * a.n;
+        f64_rows_kernel<<<(unsigned)((ns + 127) / 128), 128, 0, c->stream>>>(ns, rows, c->f64.S.p);
+        PCM_LAUNCHED(c);
+    }
     if (c->f64.mp.on) PCM_TRY(mp_l2p(c, L, a.n, a.list, a.first));
-    f64_fold_kernel<L><<<nb, 128, 0, c->stream>>>(a, rows, c->f64.S.p, c->f64.mp.on ? c->f64.mp.V.p : nullptr, ord,
+    f64_fold_kernel<L><<<(a.n + 31) / 32, 32, 0, c->stream>>>(a, rows > 2 ? 1 : rows, c->f64.S.p, c->f64.mp.on ? c->f64.mp.V.p : nullptr, ord,
                                                  a.n, W);
     PCM_LAUNCHED(c);
     return PCM_OK;
