@@ -149,24 +149,17 @@ __device__ __forceinline__ void boys_eval(float T, const float *__restrict__ tab
     }
 }
 
-// The same evaluation for two lanes (two independent arguments).  Both lanes
-// near: the row and offset are formed packed, the table Horner runs per lane
-// (each lane reads its own row).  Both far: the far branch packed.  Mixed:
-// each lane on its own.  Every lane's result equals the scalar boys_eval's.
+// The same evaluation for two lanes (two independent arguments), called by whole
+// warps.  The far branch runs packed for all threads when any lane of the warp is
+// far, the table's Horner per lane (each reads its own row) when any thread's lane is
+// near, and each lane keeps the form its argument calls for: three pieces at most,
+// where a branch per thread ran up to six (both near, both far, and each lane near or
+// far on its own).  Every lane's result equals the scalar boys_eval's.
 template <int MM>
 __device__ __forceinline__ void boys_eval2(f2 T, const float *__restrict__ tab, f2 (&F)[MM + 1])
 {
     const bool n0 = T.v.x < (float)BOYS_TMAX, n1 = T.v.y < (float)BOYS_TMAX;
-    if (n0 && n1) {
-        const f2 t = fma2(T, f2((float)BOYS_INV_DT), f2(12582912.0f));
-        const int i0 = __float_as_int(t.v.x) - 0x4B400000, i1 = __float_as_int(t.v.y) - 0x4B400000;
-        const f2 d = fma2(t + f2(-12582912.0f), f2(-(float)BOYS_DT), T);
-        float a[MM + 1], b[MM + 1];
-        boys_near32<MM>(i0, d.v.x, tab, a);
-        boys_near32<MM>(i1, d.v.y, tab, b);
-#pragma unroll
-        for (int m = 0; m <= MM; ++m) F[m] = f2(a[m], b[m]);
-    } else if (!n0 && !n1) {
+    if (__any_sync(0xffffffffu, !n0 || !n1)) {
         const f2 r0(rsqrtf(T.v.x), rsqrtf(T.v.y));
         const f2 e = fma2((T * f2(-1.f)) * r0, r0, f2(1.0f));
         const f2 rs = fma2(f2(0.5f) * r0, e, r0);
@@ -174,12 +167,24 @@ __device__ __forceinline__ void boys_eval2(f2 T, const float *__restrict__ tab, 
         F[0] = fma2(f2(BOYS_C_HI), rs, f2(BOYS_C_LO) * rs);
 #pragma unroll
         for (int m = 1; m <= MM; ++m) F[m] = (F[m - 1] * f2((float)(2 * m - 1))) * half_inv_T;
-    } else {
-        float a[MM + 1], b[MM + 1];
-        boys_eval<MM>(T.v.x, tab, a);
-        boys_eval<MM>(T.v.y, tab, b);
+    }
+    if (__any_sync(0xffffffffu, n0 || n1)) {
+        // far lanes read the table's last rows and drop the result
+        const f2 Tn(fminf(T.v.x, (float)BOYS_TMAX), fminf(T.v.y, (float)BOYS_TMAX));
+        const f2 t = fma2(Tn, f2((float)BOYS_INV_DT), f2(12582912.0f));
+        const f2 d = fma2(t + f2(-12582912.0f), f2(-(float)BOYS_DT), Tn);
+        if (__any_sync(0xffffffffu, n0)) {
+            float a[MM + 1];
+            boys_near32<MM>(__float_as_int(t.v.x) - 0x4B400000, d.v.x, tab, a);
 #pragma unroll
-        for (int m = 0; m <= MM; ++m) F[m] = f2(a[m], b[m]);
+            for (int m = 0; m <= MM; ++m) F[m].v.x = n0 ? a[m] : F[m].v.x;
+        }
+        if (__any_sync(0xffffffffu, n1)) {
+            float a[MM + 1];
+            boys_near32<MM>(__float_as_int(t.v.y) - 0x4B400000, d.v.y, tab, a);
+#pragma unroll
+            for (int m = 0; m <= MM; ++m) F[m].v.y = n1 ? a[m] : F[m].v.y;
+        }
     }
 }
 
