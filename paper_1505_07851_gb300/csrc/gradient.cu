@@ -23,6 +23,7 @@
 
 #include "common.cuh"
 #include "context.h"
+#include "f64.cuh"
 
 namespace pcm {
 
@@ -58,22 +59,29 @@ __global__ void atom_range_kernel(int M, int natom, const int *__restrict__ pato
 // An atom with zeta (d - R_J) > 6 has s_J = 1 in FP64 and does not enter S_k;
 // erf(zeta d) rounds to 1 for zeta d > 6.
 __device__ __forceinline__ double point_atom_coef(double zk, double qk, double wdiag, double ZJ, double RJ,
-                                                  double d2, int terms)
+                                                  float RJ32, double d2, int terms)
 {
-    const double d = sqrt(d2);
+    // 1/d from the hardware estimate and one step (f64.cuh) instead of a square root
+    // and two divisions, and FP32 tests: 14 FP64 instructions for an atom beyond
+    // both reaches instead of about 30
+    double rs[1];
+    f64_far<0>(d2, rs);
+    const double d = d2 * rs[0];
     double coef = 0.0;
     if (terms & PCM_GRAD_B) {
         const double a = zk * d;
-        const double gp = (a > 6.0) ? -1.0 / d2 : (TWO_OVER_SQRT_PI * zk * exp(-a * a) - erf(a) / d) / d;
+        const double gp = (f64_trunc32(a) > 6.f) ? -rs[0] * rs[0]
+                                                 : (TWO_OVER_SQRT_PI * zk * exp(-a * a) - erf(a) * rs[0]) * rs[0];
         coef += qk * ZJ * gp;
     }
-    if ((terms & PCM_GRAD_A) && zk * (d - RJ) <= 6.0) {
+    if ((terms & PCM_GRAD_A) && f64_trunc32(zk) * (f64_trunc32(d) * 0.99999f - RJ32) <= 6.001f &&
+        zk * (d - RJ) <= 6.0) {
         const double u = zk * (RJ - d), v = zk * (RJ + d);
         const double s = 0.5 * (erfc(u) + erfc(v));
         const double ds = zk * INV_SQRT_PI * (exp(-u * u) - exp(-v * v));
         coef -= wdiag * ds / s;
     }
-    return coef / d;
+    return coef * rs[0];
 }
 
 // point side: g[d][k] = sum_{J != I(k)} coef (r_k - R_J)_d  (initialises g)
@@ -84,6 +92,7 @@ __global__ void __launch_bounds__(GPT_NT) grad_point_side_kernel(
     const double *__restrict__ radius, double inv2f, int terms, double *__restrict__ g)
 {
     __shared__ double sx[GATOM_TILE], sy[GATOM_TILE], sz[GATOM_TILE], sZ[GATOM_TILE], sR[GATOM_TILE];
+    __shared__ float sR32[GATOM_TILE];
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     const bool active = k < M;
     const int kk = active ? k : 0;
@@ -100,13 +109,14 @@ __global__ void __launch_bounds__(GPT_NT) grad_point_side_kernel(
             sz[j] = xyz[3 * (J0 + j) + 2];
             sZ[j] = Z[J0 + j];
             sR[j] = radius[J0 + j];
+            sR32[j] = (float)sR[j] * 1.00001f;
         }
         __syncthreads();
         if (active)
             for (int j = 0; j < nj; ++j) {
                 if (J0 + j == I) continue;
                 const double dx = x - sx[j], dy = y - sy[j], dz = z - sz[j];
-                const double c = point_atom_coef(zk, qk, wdiag, sZ[j], sR[j], dx * dx + dy * dy + dz * dz, terms);
+                const double c = point_atom_coef(zk, qk, wdiag, sZ[j], sR[j], sR32[j], dx * dx + dy * dy + dz * dz, terms);
                 gx = fma(c, dx, gx);
                 gy = fma(c, dy, gy);
                 gz = fma(c, dz, gz);
@@ -129,13 +139,14 @@ __global__ void __launch_bounds__(GPT_NT) grad_atom_side_kernel(
     __shared__ double red[GPT_NT / 32];
     const int J = blockIdx.x;
     const double X = xyz[3 * J], Y = xyz[3 * J + 1], Zc = xyz[3 * J + 2], ZJ = Z[J], RJ = radius[J];
+    const float RJ32 = (float)RJ * 1.00001f;
     double a[3] = {0.0, 0.0, 0.0};
     for (int k = threadIdx.x; k < M; k += GPT_NT) {
         if (patom[k] == J) continue;
         const double zk = pzeta[k], qk = q[k];
         const double wdiag = qk * qk * (zk * SQRT_2_OVER_PI / pS[k]) * inv2f;
         const double dx = px[k] - X, dy = py[k] - Y, dz = pz[k] - Zc;
-        const double c = point_atom_coef(zk, qk, wdiag, ZJ, RJ, dx * dx + dy * dy + dz * dz, terms);
+        const double c = point_atom_coef(zk, qk, wdiag, ZJ, RJ, RJ32, dx * dx + dy * dy + dz * dz, terms);
         a[0] = fma(c, dx, a[0]);
         a[1] = fma(c, dy, a[1]);
         a[2] = fma(c, dz, a[2]);
