@@ -194,7 +194,8 @@ __device__ __forceinline__ float pair_bound_log2(const PairSrc &src, int A, int 
         R2 = fmaf(t, t, R2);
     }
     const float p = a + b;
-    const float x = 0.9999f * (a * b / p) * R2;
+    if (!(p > 1e-30f && p < 1e30f)) return INFINITY;   // beyond FP32: no bound
+    const float x = 0.9999f * (a / p * b) * R2;
     const float lp = __log2f(p);
     const float lc = __log2f(fabsf(trunc32(src.cnorm[src.sh_off[A] + i]))) +
                      __log2f(fabsf(trunc32(src.cnorm[src.sh_off[B] + j])));
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(128) pair_screen_kernel(long long ncand, PairS
     pair_locate(src, g, range[0], range[1], s, i, j);
     const int A = src.spA[s], B = src.spB[s];
     bool keep = thresh <= 0.0;
-    if (!keep && pair_bound_log2<LA, LB>(src, A, B, i, j) >= log2_thresh)
+    if (!keep && !(pair_bound_log2<LA, LB>(src, A, B, i, j) < log2_thresh))
         keep = pair_values<LA, LB, TS>(src, A, B, i, j).Q >= thresh;
     flag[g] = keep ? 1 : 0;
 }
