@@ -29,11 +29,11 @@ constexpr int BOYS_MCOL = 16;              // columns generated
 constexpr int BOYS_H32 = BOYS_NROW * BOYS_STRIDE32;
 constexpr int BOYS_ALLOC32 = 2 * BOYS_NROW * BOYS_STRIDE32;
 
-// x / 2 for a normal x or zero, by the exponent: the FP64 pipe is the bound
+// x / 2 by the exponent (the FP64 pipe is the bound); values below 2^-1022 stay as they are
 __device__ __forceinline__ double half_by_bits(double x)
 {
     const int h = __double2hiint(x);
-    return __hiloint2double((h & 0x7fffffff) ? h - 0x00100000 : h, __double2loint(x));
+    return __hiloint2double((h & 0x7ff00000) ? h - 0x00100000 : h, __double2loint(x));
 }
 
 // -2 x for a positive normal x
