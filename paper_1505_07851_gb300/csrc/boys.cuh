@@ -45,9 +45,9 @@ __device__ __forceinline__ double minus_twice_by_bits(double x)
 // FP64.  The FP64 pipe bounds the callers, and comparisons and conversions take
 // its slots like an FMA: the branch and the row come from integer operations, T_i
 // from the row's last column, and the scalings by powers of two from the exponent
-// (20 instead of 25 FP64 instructions for an ss interaction, 33 instead of 39 for
+// (19 instead of 25 FP64 instructions for an ss interaction, 32 instead of 39 for
 // ps; the same bits).  d is T - T_i exactly.  Potentials of a 100-atom s/p/d cluster
-// 32.3 -> 28.4 ms.
+// 32.3 -> 28.3 ms.
 template <int MM>
 __device__ __forceinline__ void boys_eval(double T, const double *__restrict__ tab, double (&F)[MM + 1])
 {
@@ -61,7 +61,7 @@ __device__ __forceinline__ void boys_eval(double T, const double *__restrict__ t
         for (int k = 0; k < MM + 7; ++k) r[k] = __ldg(row + k);
         const double d = T - __ldg(row + BOYS_T64);
         const double e1 = -d, e2 = half_by_bits(-d), e3 = -d * (1.0 / 3.0), e4 = half_by_bits(e2), e5 = -d * 0.2,
-                     e6 = -d * (1.0 / 6.0);
+                     e6 = half_by_bits(e3);   // 1.0 / 6.0 is half of 1.0 / 3.0 to the bit
 #pragma unroll
         for (int m = 0; m <= MM; ++m) {
             double s = fma(r[m + 6], e6, r[m + 5]);

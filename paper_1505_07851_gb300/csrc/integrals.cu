@@ -139,8 +139,13 @@ __global__ void esp_coef_kernel(int nesp, const int *__restrict__ list, int base
 // the classes present in the block (at most MAXCB).
 // grid.x: point blocks (ranges from blk_off), grid.y: pair segments.
 // ---------------------------------------------------------------------------
-constexpr int ESP_NT = 128;
+// Threads per block.  The pair segments are planned for blocks of ESP_PLAN points
+// (their sums' bits go by the segments); blocks of half as many even out the SMs'
+// shares (300 atoms: 1222 blocks of 256 points are 8.04 per SM, nine on some; potentials
+// of a 100-atom s/p/d cluster 27.9 -> 27.7 ms).
+constexpr int ESP_NT = 64;
 constexpr int ESP_PPT = 2;
+constexpr int ESP_PLAN = 256;
 constexpr int ESP_TP = 32;
 constexpr int ESP_MAXCB = 8;
 
@@ -530,11 +535,10 @@ __global__ void __launch_bounds__(GPA_NT) pair_atom_reduce_kernel(int natom, con
 // ---------------------------------------------------------------------------
 static int target_ctas(pcm_ctx *) { return 152 * 8; }
 
-// point blocks of at most ESP_NT*ESP_PPT points spanning at most ESP_MAXCB classes
-static void esp_blocks(pcm_ctx *c, std::vector<int> &off)
+// point blocks of at most cap points spanning at most ESP_MAXCB classes
+static void esp_blocks(pcm_ctx *c, int cap, std::vector<int> &off)
 {
     off.clear();
-    const int cap = ESP_NT * ESP_PPT;
     int k = 0;
     // class of point k from the class offsets
     auto cls_of = [&](int kk) {
@@ -691,7 +695,9 @@ int esp_compute(pcm_ctx *c, const double *dP, double *dc)
         return esp_class_stats(c);
     }
     std::vector<int> off;
-    esp_blocks(c, off);
+    esp_blocks(c, ESP_PLAN, off);
+    const int nplan = (int)off.size() - 1;
+    esp_blocks(c, ESP_NT * ESP_PPT, off);
     const int nblk = (int)off.size() - 1;
     DBuf<int> &blk = c->si[5];
     PCM_TRY(blk.alloc(off.size()));
@@ -711,7 +717,7 @@ int esp_compute(pcm_ctx *c, const double *dP, double *dc)
             continue;
         }
         const int maxseg = (pc.nesp + ESP_TP - 1) / ESP_TP;
-        int ns = std::max(1, std::min(maxseg, (target_ctas(c) + nblk - 1) / nblk));
+        int ns = std::max(1, std::min(maxseg, (target_ctas(c) + nplan - 1) / nplan));
         int sl = (pc.nesp + ns - 1) / ns;
         sl = (sl + ESP_TP - 1) / ESP_TP * ESP_TP;
         ns = (pc.nesp + sl - 1) / sl;
