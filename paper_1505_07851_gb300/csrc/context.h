@@ -401,6 +401,7 @@ int zeta_pairs(pcm_ctx *c, cudaStream_t s);
 int matfree_build(pcm_ctx *c, cudaStream_t s);
 int matfree_dfmv(pcm_ctx *c, const double *x, double *y, double *part, int *nparts);
 int matfree_mv32(pcm_ctx *c, const double *x, double *y);
+int row_sum_bound(pcm_ctx *c, cudaStream_t s);
 int persistent_pcg(pcm_ctx *c, const double *b, double *x, double delta, int max_iter, int *iters, int *conv,
                 double *rnorm);
 inline bool matrix_free(const pcm_ctx *c) { return c->mf_active; }

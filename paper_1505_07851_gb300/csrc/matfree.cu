@@ -1040,6 +1040,22 @@ __global__ void __launch_bounds__(MV_NT) near_abs_kernel(int M, const int *__res
     if (lane == 0) atomicMax(out, (unsigned long long)__double_as_longlong(mx));
 }
 
+// the row-sum bound of the inner products' fixed-point scale, once per operator
+int row_sum_bound(pcm_ctx *c, cudaStream_t s)
+{
+    const int M = c->M;
+    PCM_TRY(c->st_arow.alloc(1));
+    PCM_CUDA(cudaMemsetAsync(c->st_arow.p, 0, sizeof(double), s));
+    unsigned long long *o = reinterpret_cast<unsigned long long *>(c->st_arow.p);
+    if (matrix_free(c))
+        near_abs_kernel<<<std::min(4096, (M + 7) / 8), MV_NT, 0, s>>>(M, c->mf_off.p, c->mf_val32.p, o);
+    else
+        arow_kernel<<<std::min(4096, (M + 7) / 8), MV_NT, 0, s>>>(M, c->lda, c->A32.p, o);
+    PCM_LAUNCHED(c);
+    c->st_arow_ok = true;
+    return PCM_OK;
+}
+
 // Inner PCG from x = 0 on A x = b with the FP32 product (matrix-free, or the
 // stored A32 of PCM_MIXED) and the context's preconditioner, to ||r|| < delta
 // (recursively updated residual) or max_iter steps, in one cooperative launch.
@@ -1072,18 +1088,7 @@ int persistent_pcg(pcm_ctx *c, const double *b, double *x, double delta, int max
     PCM_TRY(c->mf_idot.alloc((size_t)grid));
     PCM_TRY(c->st_acc.alloc(M));
     PCM_TRY(c->st_pmax.alloc(2));
-    PCM_TRY(c->st_arow.alloc(1));
-    if (!c->st_arow_ok) {
-        // the row-sum bound of the fixed-point scale, once per operator
-        PCM_CUDA(cudaMemsetAsync(c->st_arow.p, 0, sizeof(double), c->stream));
-        unsigned long long *o = reinterpret_cast<unsigned long long *>(c->st_arow.p);
-        if (stored)
-            arow_kernel<<<std::min(4096, (M + 7) / 8), MV_NT, 0, c->stream>>>(M, c->lda, c->A32.p, o);
-        else
-            near_abs_kernel<<<std::min(4096, (M + 7) / 8), MV_NT, 0, c->stream>>>(M, c->mf_off.p, c->mf_val32.p, o);
-        PCM_LAUNCHED(c);
-        c->st_arow_ok = true;
-    }
+    if (!c->st_arow_ok) PCM_TRY(row_sum_bound(c, c->stream));
     PCM_CUDA(cudaMemsetAsync(c->st_acc.p, 0, (size_t)M * sizeof(unsigned long long), c->stream));
     PCM_CUDA(cudaMemsetAsync(c->st_pmax.p, 0, 2 * sizeof(unsigned), c->stream));
     // the stored product reads the direction in whole tiles: zero padding to ntb tiles
