@@ -54,13 +54,11 @@ __global__ void pts4_kernel(int M, const double *__restrict__ px, const double *
 }
 
 // near pairs of row k (r2_test32 < rc2, the diagonal included): count, or
-// write columns (ascending), exact values, and for the FP32 product the values
-// less the constant rsqrt(rc2) that product adds for each near pair
+// write columns (ascending)
 template <bool FILL>
 __global__ void __launch_bounds__(MV_NT) near_rows_kernel(int M, const float4 *__restrict__ pts, float rc2,
                                                           int *__restrict__ cnt, const int *__restrict__ off,
-                                                          AFree acc, int *__restrict__ col,
-                                                          double *__restrict__ val, float *__restrict__ val32)
+                                                          int *__restrict__ col)
 {
     __shared__ float4 sc[NL_CH];
     const int k = blockIdx.x * MV_NT + threadIdx.x;
@@ -74,19 +72,34 @@ __global__ void __launch_bounds__(MV_NT) near_rows_kernel(int M, const float4 *_
         if (k < M)
             for (int j = 0; j < nc; ++j)
                 if (r2_test32(a, sc[j]) < rc2) {
-                    if (FILL) {
-                        const double v = acc.exact(k, c0 + j);
-                        col[o] = c0 + j;
-                        val[o] = v;
-                        // the FP32 product adds rsqrt(rc2) for every near pair
-                        val32[o] = (float)(v - (double)rsqrt_fast(rc2));
-                        ++o;
-                    } else {
+                    if (FILL)
+                        col[o++] = c0 + j;
+                    else
                         ++n;
-                    }
                 }
     }
     if (!FILL && k < M) cnt[k] = n;
+}
+
+// exact values of the near pairs, and for the FP32 product the values less the
+// constant rsqrt(rc2) that product adds for each near pair.  A thread per pair: in
+// the row loops above a lane with a near pair holds up its warp for an FP64 erf
+// (46363 points: 6.4 ms, of which the distance tests are 1.1).
+__global__ void __launch_bounds__(MV_NT) near_values_kernel(int nnz, int M, const int *__restrict__ off,
+                                                            const int *__restrict__ col, float rc2, AFree acc,
+                                                            double *__restrict__ val, float *__restrict__ val32)
+{
+    const int e = blockIdx.x * MV_NT + threadIdx.x;
+    if (e >= nnz) return;
+    int lo = 0, hi = M - 1;   // the last row that starts at or before e (no row is empty)
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (off[mid] <= e) lo = mid;
+        else hi = mid - 1;
+    }
+    const double v = acc.exact(lo, col[e]);
+    val[e] = v;
+    val32[e] = (float)(v - (double)rsqrt_fast(rc2));
 }
 
 // exclusive scan of n ints by one block: off[0..n] (off[n] = total)
@@ -175,8 +188,7 @@ int matfree_build(pcm_ctx *c, cudaStream_t s)
     PCM_TRY(c->mf_cnt.alloc(M));
     const AFree acc = afree(c);
     const int nb = (M + MV_NT - 1) / MV_NT;
-    near_rows_kernel<false><<<nb, MV_NT, 0, s>>>(M, c->mf_pts.p, c->mf_rc2, c->mf_cnt.p, nullptr, acc, nullptr,
-                                                 nullptr, nullptr);
+    near_rows_kernel<false><<<nb, MV_NT, 0, s>>>(M, c->mf_pts.p, c->mf_rc2, c->mf_cnt.p, nullptr, nullptr);
     PCM_LAUNCHED(c);
     scan_one_block_kernel<<<1, 1024, 0, s>>>(M, c->mf_cnt.p, c->mf_off.p);
     PCM_LAUNCHED(c);
@@ -187,9 +199,13 @@ int matfree_build(pcm_ctx *c, cudaStream_t s)
     PCM_TRY(c->mf_col.alloc(std::max(1, nnz)));
     PCM_TRY(c->mf_val.alloc(std::max(1, nnz)));
     PCM_TRY(c->mf_val32.alloc(std::max(1, nnz)));
-    near_rows_kernel<true><<<nb, MV_NT, 0, s>>>(M, c->mf_pts.p, c->mf_rc2, nullptr, c->mf_off.p, acc, c->mf_col.p,
-                                                c->mf_val.p, c->mf_val32.p);
+    near_rows_kernel<true><<<nb, MV_NT, 0, s>>>(M, c->mf_pts.p, c->mf_rc2, nullptr, c->mf_off.p, c->mf_col.p);
     PCM_LAUNCHED(c);
+    if (nnz > 0) {
+        near_values_kernel<<<(nnz + MV_NT - 1) / MV_NT, MV_NT, 0, s>>>(nnz, M, c->mf_off.p, c->mf_col.p, c->mf_rc2,
+                                                                       acc, c->mf_val.p, c->mf_val32.p);
+        PCM_LAUNCHED(c);
+    }
     PCM_TRY(c->dinv.alloc(M));
     dinv_free_kernel<<<(M + 127) / 128, 128, 0, s>>>(M, c->pzeta.p, c->pS.p, c->dinv.p);
     PCM_LAUNCHED(c);
