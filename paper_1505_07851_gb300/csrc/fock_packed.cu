@@ -113,11 +113,11 @@ __device__ __forceinline__ void two_sum_f(float a, float b, float &s, float &e)
     e = (a - (s - bb)) + (b - bb);
 }
 
-// resident blocks per SM the register allocation aims for (no spills at these)
 // slots evaluated side by side before their votes: their chains overlap (one slot a
 // turn: Fock correction of 1000 atoms 70.4 ms, two turns unrolled 68.3, two ss slots
 // side by side as well 68.1; two ps slots spill)
 constexpr int fk_slots(int L) { return L == 0 ? 2 : 1; }
+// resident blocks per SM the register allocation aims for (no spills at these)
 constexpr int fk_min_blocks(int L, int NPT)
 {
     return L == 0 ? 5 : (L == 1 ? (NPT == 2 ? 4 : 5) : (L == 2 ? (NPT == 2 ? 3 : 4) : (L == 3 ? 3 : (L == 4 ? 2 : 1))));

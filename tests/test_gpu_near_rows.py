@@ -1,9 +1,9 @@
-"""Surfaces and the matrix-free operator's near rows where their FP32 tests and
-groups of 32 points can go wrong: fewer points than a group, ragged last groups,
-atoms with their own radii and point spacing, and molecules far from the origin
-(coarser FP32 coordinates).  The kept points are the oracle's; the products of a
-positive vector hold 1e-11 (accurate) and 1e-6 relative (FP32), the latter plus the
-rounding of the coordinates: 2 sqrt(3) 2^-24 |x| in a distance of 2 bohr or more."""
+"""Surfaces and the matrix-free operator's near rows where their FP32 tests can go
+wrong: fewer points than a warp, ragged last blocks, atoms with their own radii and
+point spacing, scattered atoms, and molecules far from the origin (coarser FP32
+coordinates).  The kept points are the oracle's; the products of a positive vector
+hold 1e-11 (accurate) and 1e-6 relative (FP32), the latter plus the rounding of the
+coordinates: 2 sqrt(3) 2^-24 |x| in a distance of 2 bohr or more."""
 import numpy as np
 import pytest
 
