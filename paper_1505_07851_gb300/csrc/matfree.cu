@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(MV_NT) near_rows_kernel(int M, const float4 *_
 // exact values of the near pairs, and for the FP32 product the values less the
 // constant rsqrt(rc2) that product adds for each near pair.  A thread per pair: in
 // the row loops above a lane with a near pair holds up its warp for an FP64 erf
-// (46363 points: 6.4 ms, of which the distance tests are 1.1).
+// (46363 points: 6.4 ms; 1.7 for the columns and 0.3 for the values so).
 __global__ void __launch_bounds__(MV_NT) near_values_kernel(int nnz, int M, const int *__restrict__ off,
                                                             const int *__restrict__ col, float rc2, AFree acc,
                                                             double *__restrict__ val, float *__restrict__ val32)
