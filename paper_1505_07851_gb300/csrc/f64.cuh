@@ -13,6 +13,8 @@
 // (U / (sqrt(pi) / (2 sqrt(p))) = 2 sqrt(rho / pi)), so both forms share the
 // polynomials.  Beyond f64_far_T the two agree to below 1e-16 relative.
 #pragma once
+#include <string.h>
+
 #include "common.cuh"
 #include "farfield.cuh"
 
@@ -62,13 +64,67 @@ __device__ __forceinline__ void f64_far(double R2, double (&b)[L + 1])
     }
 }
 
+// words of a double
+__host__ __device__ __forceinline__ int hi_word(double v)
+{
+#ifdef __CUDA_ARCH__
+    return __double2hiint(v);
+#else
+    long long b;
+    memcpy(&b, &v, sizeof(b));
+    return (int)(b >> 32);
+#endif
+}
+
+__host__ __device__ __forceinline__ unsigned lo_word(double v)
+{
+#ifdef __CUDA_ARCH__
+    return (unsigned)__double2loint(v);
+#else
+    long long b;
+    memcpy(&b, &v, sizeof(b));
+    return (unsigned)b;
+#endif
+}
+
+// FP32 value of a non-negative double from its high word (20 mantissa bits,
+// towards zero; values outside FP32's normal range become its smallest or largest),
+// without the conversion's FP64-pipe slot
+__host__ __device__ __forceinline__ float f64_trunc32(double v)
+{
+    int h = hi_word(v);
+    h = h < 0x38100000 ? 0x38100000 : (h > 0x47efffff ? 0x47efffff : h);
+    const int f = (h - 0x38000000) << 3;
+#ifdef __CUDA_ARCH__
+    return __int_as_float(f);
+#else
+    float x;
+    memcpy(&x, &f, sizeof(x));
+    return x;
+#endif
+}
+
+// T = rho R^2 below `top`?  In FP32 from the truncated factors: T itself may be
+// larger by up to 2^-19 of it.  Every read of the table is behind this test.
+__host__ __device__ __forceinline__ bool f64_below(double R2, double rho, float top)
+{
+    return f64_trunc32(R2) * f64_trunc32(rho) < top;
+}
+
+// row of the table from t = T + F64_MAGIC; the bound is for arguments that are no T
+__host__ __device__ __forceinline__ int f64_row(double t)
+{
+    const unsigned i = lo_word(t);
+    return (int)(i < (unsigned)F64_NROW ? i : (unsigned)F64_NROW - 1u);
+}
+
 // b_n of the near form; lanes without `use` read row 0 and return garbage
 template <int L>
 __device__ __forceinline__ void f64_near(double R2, double rho, double cn, bool use, const double *__restrict__ tab,
                                          double (&b)[L + 1])
 {
     const double t = fma(rho, R2, F64_MAGIC);
-    const int i = use ? __double2loint(t) : 0;
+    const int i = use ? f64_row(t) : 0;
     const double d = fma(rho, R2, F64_MAGIC - t);
     const double2 *row = reinterpret_cast<const double2 *>(tab + (size_t)i * F64_STRIDE);
     double f = cn;
@@ -164,20 +220,14 @@ __device__ __forceinline__ void f64_accumulate(double X, double Y, double Z, con
     }
 }
 
-// FP32 value of a non-negative double from its high word (20 mantissa bits,
-// towards zero), without the conversion's FP64-pipe slot
-__device__ __forceinline__ float f64_trunc32(double v)
-{
-    return __int_as_float((max(__double2hiint(v), 0x38100000) - 0x38000000) << 3);
-}
-
-// b_n of near interactions (lanes with `on`; T < f64_far_T) of pairs whose far form
-// comes from their cell's expansion: what the near form adds to it.
+// b_n of near interactions (lanes with `on`) of pairs whose far form comes from
+// their cell's expansion: what the near form adds to it, zero from f64_far_T on.
 template <int L>
 __device__ __forceinline__ void f64_near_minus_far(double R2, double2 rc, bool on, const double *__restrict__ tab,
                                                    double (&b)[L + 1])
 {
-    const bool low = f64_trunc32(R2) * f64_trunc32(rc.x) < (float)F64_H_MIN;
+    on = on && f64_below(R2, rc.x, (float)f64_far_T(L));
+    const bool low = f64_below(R2, rc.x, (float)F64_H_MIN);
     f64_near<L>(R2, rc.x, rc.y, on, low ? tab : tab + F64_TABLE, b);
     if (__any_sync(0xffffffffu, on && low)) {
         double bf[L + 1];
@@ -195,7 +245,7 @@ template <int L>
 __device__ __forceinline__ void f64_terms(double R2, double2 rc, bool expanded, const double *__restrict__ tab,
                                           double (&b)[L + 1])
 {
-    const bool near = f64_trunc32(R2) * f64_trunc32(rc.x) < (float)f64_far_T(L);
+    const bool near = f64_below(R2, rc.x, (float)f64_far_T(L));
     if (__any_sync(0xffffffffu, near && !expanded)) {
         f64_near<L>(R2, rc.x, rc.y, near, tab, b);
         if (!__all_sync(0xffffffffu, near)) {

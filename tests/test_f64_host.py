@@ -1,0 +1,59 @@
+"""Host evaluation of the rules that send FP64 interactions to tables and expansions
+(the same functions the kernels call, compiled for the CPU): no argument leaves the
+table, and every argument that the table serves is within its range."""
+import os
+import subprocess
+
+import pytest
+
+from paper_1505_07851_gb300 import build
+
+PRELUDE = """
+#include <stdio.h>
+#include <math.h>
+#include "f64.cuh"
+using namespace pcm;
+"""
+
+
+def run_host(tmp_path, body, include="f64.cuh"):
+    src = tmp_path / "host.cu"
+    src.write_text(PRELUDE.replace("f64.cuh", include) + body)
+    exe = tmp_path / "host"
+    cmd = [build.nvcc(), "-std=c++17", "--expt-relaxed-constexpr", *build.ARCH, "-I", build.CSRC, str(src), "-o", str(exe)]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+    return r.stdout.split()
+
+
+def test_table_rows(tmp_path):
+    """Squared distances and exponents over the whole range of doubles: T < f64_far_T is
+    decided as in 64 bits (within 2^-18), so that a row that is read holds T; and the row of
+    any double, NaN and infinity among them, is a row of the table."""
+    out = run_host(tmp_path, """
+int main()
+{
+    long bad = 0, near = 0;
+    for (int L = 0; L <= 5; ++L)
+        for (double r = 1e-30; r < 1e307; r *= 1.17)
+            for (double rho = 1e-20; rho < 1e30; rho *= 1.31) {
+                const double R2 = r, T = rho * R2, top = f64_far_T(L);
+                const bool n = f64_below(R2, rho, (float)top);
+                near += n;
+                if (n && !(T < top * (1 + 0x1p-18))) ++bad;
+                if (!n && !(T >= top * (1 - 0x1p-18))) ++bad;
+                if (n && abs(f64_row(T + F64_MAGIC) - (int)rint(T * F64_INV_DT)) > 1) ++bad;
+            }
+    const double odd[] = {0.0, 54.0, 55.0, 1e9, 1e16, 1e30, 1e300, INFINITY, -INFINITY, NAN, -NAN, -1.0, -1e30};
+    for (double t : odd)
+        for (double u : {t, t + F64_MAGIC}) {
+            const int i = f64_row(u);
+            if (i < 0 || i >= F64_NROW) ++bad;
+        }
+    printf("%ld %ld\\n", bad, near);
+    return 0;
+}
+""")
+    assert int(out[0]) == 0 and int(out[1]) > 100000
