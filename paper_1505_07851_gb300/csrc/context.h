@@ -108,6 +108,8 @@ struct __align__(16) F64Pt {
 };
 struct F64Box {
     double lo[3], inv;                     // lower corner, 1 / side of the cube around the cavity
+    double mid[3];                         // its centre: FP32 coordinates count from here
+    float slack;                           // bound of the error of a distance between two of them
 };
 struct F64Src {                            // kept pairs of the classes; first sorted position of each
     const double *Px[6], *Py[6], *Pz[6], *p[6];
@@ -137,15 +139,16 @@ struct F64Mp {
 };
 struct F64Int {
     DBuf<double> tab;                      // Boys table (f64.cuh)
+    F64Box box;
     int ntile = 0;                         // tiles of 32 points
     DBuf<int> pt_idx, pt_cls;              // per slot: point, exponent class
     DBuf<F64Pt> pt_xyz;                    // per slot: coordinates, charge of the current call
-    DBuf<float4> pt_x32;                   // per slot: coordinates and zeta^-2 in FP32
+    DBuf<float4> pt_x32;                   // per slot: coordinates from box.mid and zeta^-2 in FP32
     DBuf<float4> pt_sph;                   // per tile: bounding sphere
     int off[7] = {0, 0, 0, 0, 0, 0, 0};    // first sorted position of each class
     DBuf<int> ord;                         // sorted position -> kept pair of its class
     DBuf<double> P;                        // 4 x pairs: centre, exponent
-    DBuf<float4> info;                     // the same in FP32
+    DBuf<float4> info;                     // the same in FP32, from box.mid
     bool use_rc = false;
     DBuf<double2> rc;                      // exponent classes x pairs: rho, cn
     DBuf<unsigned> key;

@@ -111,6 +111,26 @@ __host__ __device__ __forceinline__ bool f64_below(double R2, double rho, float 
     return f64_trunc32(R2) * f64_trunc32(rho) < top;
 }
 
+// FP32 tests on coordinates from the middle of the cavity.  `slack` bounds the error
+// of a distance between two of them (context.h), so that both tests only err on the
+// side of the FP64 evaluation.
+//
+// may a pair (b: centre, exponent) have T < farT at a point of the tile (s: sphere)?
+__host__ __device__ __forceinline__ bool f64_reaches(const float4 &b, const float4 &s, float zmin2, float farT,
+                                                     float slack)
+{
+    const float dx = b.x - s.x, dy = b.y - s.y, dz = b.z - s.z;
+    const float d = fmaxf(sqrtf(dx * dx + dy * dy + dz * dz) * 0.99999f - slack - s.w, 0.f);
+    return b.w * zmin2 * d * d < 1.00001f * farT * (b.w + zmin2);
+}
+
+// T < farT for one interaction, s = 1/p + 1/zeta^2 = 1/rho?  A distance that is off by
+// slack leaves R^2 within 0.05% and `pad` = 2001 slack^2 of it.
+__host__ __device__ __forceinline__ bool f64_is_near(float x, float y, float z, float s, float farT, float pad)
+{
+    return fmaf(x, x, fmaf(y, y, z * z)) < fmaf(1.001f * farT + 0.05f, s, pad);
+}
+
 // row of the table from t = T + F64_MAGIC; the bound is for arguments that are no T
 __host__ __device__ __forceinline__ int f64_row(double t)
 {

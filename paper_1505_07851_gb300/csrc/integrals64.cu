@@ -144,7 +144,7 @@ __global__ void f64_point_key_kernel(int M, const double *__restrict__ px, const
 __global__ void f64_point_tile_kernel(int M, const int *__restrict__ val, const double *__restrict__ px,
                                       const double *__restrict__ py, const double *__restrict__ pz,
                                       const int *__restrict__ pcls, int *__restrict__ idx, int *__restrict__ cls,
-                                      const double *__restrict__ cls_zeta, F64Pt *__restrict__ xyz,
+                                      const double *__restrict__ cls_zeta, F64Box box, F64Pt *__restrict__ xyz,
                                       float4 *__restrict__ x32, float4 *__restrict__ sph)
 {
     const int tile = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -159,13 +159,14 @@ __global__ void f64_point_tile_kernel(int M, const int *__restrict__ val, const 
         rank += (eo < e || (eo == e && o < lane)) ? 1 : 0;
     }
     const double x = px[k], y = py[k], z = pz[k];
+    const float fx = (float)(x - box.mid[0]), fy = (float)(y - box.mid[1]), fz = (float)(z - box.mid[2]);
     if (lane < nt) {
         idx[tile * 32 + rank] = k;
         cls[tile * 32 + rank] = e;
         xyz[tile * 32 + rank] = F64Pt{x, y, z, 0.0};
-        x32[tile * 32 + rank] = make_float4((float)x, (float)y, (float)z, (float)(1.0 / (cls_zeta[e] * cls_zeta[e])));
+        x32[tile * 32 + rank] = make_float4(fx, fy, fz, (float)(1.0 / (cls_zeta[e] * cls_zeta[e])));
     }
-    float lo[3] = {(float)x, (float)y, (float)z}, hi[3] = {(float)x, (float)y, (float)z};
+    float lo[3] = {fx, fy, fz}, hi[3] = {fx, fy, fz};
 #pragma unroll
     for (int d = 0; d < 3; ++d)
 #pragma unroll
@@ -174,12 +175,11 @@ __global__ void f64_point_tile_kernel(int M, const int *__restrict__ val, const 
             hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
         }
     const float cx = 0.5f * (lo[0] + hi[0]), cy = 0.5f * (lo[1] + hi[1]), cz = 0.5f * (lo[2] + hi[2]);
-    const float dx = (float)x - cx, dy = (float)y - cy, dz = (float)z - cz;
+    const float dx = fx - cx, dy = fy - cy, dz = fz - cz;
     float r2 = dx * dx + dy * dy + dz * dz;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) r2 = fmaxf(r2, __shfl_xor_sync(0xffffffffu, r2, o));
-    // the margin covers the FP32 rounding of the coordinates and distances
-    if (lane == 0) sph[tile] = make_float4(cx, cy, cz, sqrtf(r2) * 1.0001f + 1e-4f);
+    if (lane == 0) sph[tile] = make_float4(cx, cy, cz, sqrtf(r2) * 1.0001f + box.slack);
 }
 
 __device__ __forceinline__ int f64_class_of(const F64Src &s, int g)
@@ -200,7 +200,7 @@ __device__ __forceinline__ double2 f64_rho_cn(double p, double z2)
 // sorted pair data: kept index, centre and exponent, FP32 copies for the tests,
 // and (for few exponent classes) rho and cn per class
 __global__ void f64_pair_gather_kernel(int n, F64Src src, const int *__restrict__ val, int ncls,
-                                       const double *__restrict__ cls_zeta, int *__restrict__ ord,
+                                       const double *__restrict__ cls_zeta, F64Box box, int *__restrict__ ord,
                                        double *__restrict__ P, float4 *__restrict__ info, double2 *__restrict__ rc)
 {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
@@ -212,7 +212,9 @@ __global__ void f64_pair_gather_kernel(int n, F64Src src, const int *__restrict_
     P[(size_t)n + g] = y;
     P[2 * (size_t)n + g] = z;
     P[3 * (size_t)n + g] = p;
-    info[g] = make_float4((float)x, (float)y, (float)z, (float)p);
+    // an exponent beyond 1e30 acts as that one (rho is zeta^2 either way)
+    info[g] = make_float4((float)(x - box.mid[0]), (float)(y - box.mid[1]), (float)(z - box.mid[2]),
+                          (float)fmin(p, 1e30));
     if (rc)
         for (int e = 0; e < ncls; ++e) rc[(size_t)e * n + g] = f64_rho_cn(p, cls_zeta[e] * cls_zeta[e]);
 }
@@ -222,7 +224,7 @@ int f64_prepare(pcm_ctx *c)
 {
     F64Int &f = c->f64;
     const int M = c->M;
-    const F64Box box = cavity_box(c, F64_CELL);
+    const F64Box box = f.box = cavity_box(c, F64_CELL);
     const F64Src src = kept_pairs(c, f.off);
     const int n = f.off[6];
     f.ntile = (M + 31) / 32;
@@ -242,7 +244,7 @@ int f64_prepare(pcm_ctx *c)
     }
     f64_point_tile_kernel<<<(f.ntile + 3) / 4, 128, 0, c->stream>>>(M, sort_pts ? f.val.p : nullptr, c->px.p, c->py.p,
                                                                    c->pz.p, c->pcls.p, f.pt_idx.p, f.pt_cls.p,
-                                                                   c->cls_zeta.p, f.pt_xyz.p, f.pt_x32.p,
+                                                                   c->cls_zeta.p, box, f.pt_xyz.p, f.pt_x32.p,
                                                                    f.pt_sph.p);
     PCM_LAUNCHED(c);
     f.mp.on = false;
@@ -256,7 +258,7 @@ int f64_prepare(pcm_ctx *c)
     bool sorted;
     PCM_TRY(pair_order(c, src, box, false, &sorted));
     f64_pair_gather_kernel<<<(n + 127) / 128, 128, 0, c->stream>>>(n, src, sorted ? f.val.p : nullptr, c->ncls,
-                                                                  c->cls_zeta.p, f.ord.p, f.P.p, f.info.p,
+                                                                  c->cls_zeta.p, box, f.ord.p, f.P.p, f.info.p,
                                                                   f.use_rc ? f.rc.p : nullptr);
     PCM_LAUNCHED(c);
     if (n >= F64_MP_PAIRS && M >= F64_MP_POINTS) PCM_TRY(mp_prepare(c, box, src, CURVE_HBITS, CURVE_PBITS));
@@ -464,6 +466,7 @@ struct F64Points {
     const float4 *sph;
     const double *cls_zeta;
     float zmin2;             // smallest zeta^2: the smallest rho, the longest reach
+    float slack, pad;        // error bounds of the FP32 tests (f64_reaches, f64_is_near)
     const double *tab;
 };
 
@@ -486,21 +489,6 @@ __device__ __forceinline__ double2 f64_load_rc(const F64Pairs &a, const F64Point
     if (a.rc) return __ldg(a.rc + (size_t)e * a.stride + pos);
     const double z = t.cls_zeta[e];
     return f64_rho_cn(a.P[3 * (size_t)a.stride + pos], z * z);
-}
-
-// reach test: may a pair (info b) have T < farT at a point of the tile?
-__device__ __forceinline__ bool f64_reaches(const float4 &b, const float4 &s, float zmin2, float farT)
-{
-    const float dx = b.x - s.x, dy = b.y - s.y, dz = b.z - s.z;
-    const float d = fmaxf(sqrtf(dx * dx + dy * dy + dz * dz) * 0.99999f - 2e-5f - s.w, 0.f);
-    return b.w * zmin2 * d * d < 1.00001f * farT * (b.w + zmin2);
-}
-
-// FP32 test of one interaction: T < farT with a margin for the FP32 rounding (the
-// near form holds to the table's end at T = 54); s = 1/p + 1/zeta^2 = 1/rho
-__device__ __forceinline__ bool f64_is_near(float x, float y, float z, float s, float farT)
-{
-    return fmaf(x, x, fmaf(y, y, z * z)) < (1.001f * farT + 0.05f) * s;
 }
 
 // resident blocks of 128 threads per SM the register allocation aims for: the
@@ -563,7 +551,7 @@ __global__ void __launch_bounds__(128, f64_min_blocks(far_nterms(L)))
         if (act) {
             const int pos = a.list[j0 + lane];
             info = a.info[pos];
-            nr = f64_reaches(info, sph, t.zmin2, FT);
+            nr = f64_reaches(info, sph, t.zmin2, FT, t.slack);
             ex = a.order && a.order[(size_t)tile * a.ncell + a.cell[pos]] != 0;
         }
         const unsigned nm = __ballot_sync(0xffffffffu, nr), em = __ballot_sync(0xffffffffu, ex);
@@ -580,7 +568,7 @@ __global__ void __launch_bounds__(128, f64_min_blocks(far_nterms(L)))
             const int o = __ffs(m) - 1;
             const float4 b = make_float4(__shfl_sync(0xffffffffu, info.x, o), __shfl_sync(0xffffffffu, info.y, o),
                                          __shfl_sync(0xffffffffu, info.z, o), __shfl_sync(0xffffffffu, info.w, o));
-            near |= f64_is_near(b.x - c32.x, b.y - c32.y, b.z - c32.z, 1.f / b.w + c32.w, FT) ? 1u << o : 0u;
+            near |= f64_is_near(b.x - c32.x, b.y - c32.y, b.z - c32.z, 1.f / b.w + c32.w, FT, t.pad) ? 1u << o : 0u;
         }
         int o = 0;
         while (__any_sync(0xffffffffu, near != 0)) {
@@ -650,7 +638,7 @@ __global__ void __launch_bounds__(128, f64_min_blocks(far_nterms(L)))
     for (int k = 0; k < NC; ++k) acc[k] = 0.0;
     const float ip = 1.f / info.w;
     for (int tile = blockIdx.y; tile < t.ntile; tile += gridDim.y) {
-        const bool reaches = f64_reaches(info, t.sph[tile], t.zmin2, FT);
+        const bool reaches = f64_reaches(info, t.sph[tile], t.zmin2, FT, t.slack);
         const bool expanded = a.order && a.order[(size_t)tile * a.ncell + cell] != 0;
         const int s0 = tile * 32, nt = min(32, t.M - s0);
         if (!__all_sync(0xffffffffu, expanded)) {
@@ -692,7 +680,7 @@ __global__ void __launch_bounds__(128, f64_min_blocks(far_nterms(L)))
         unsigned near = 0;
         for (int i = 0; i < nt; ++i) {
             const float4 c = t.x32[s0 + i];
-            near |= f64_is_near(info.x - c.x, info.y - c.y, info.z - c.z, ip + c.w, FT) ? 1u << i : 0u;
+            near |= f64_is_near(info.x - c.x, info.y - c.y, info.z - c.z, ip + c.w, FT, t.pad) ? 1u << i : 0u;
         }
         if (!expanded) near = 0;
         int o = 0;
@@ -783,6 +771,8 @@ static F64Points f64_points(pcm_ctx *c)
     t.sph = c->f64.pt_sph.p;
     t.cls_zeta = c->cls_zeta.p;
     t.zmin2 = (float)(c->h_cls_zeta[0] * c->h_cls_zeta[0]) * 0.99999f;
+    t.slack = c->f64.box.slack;
+    t.pad = 2001.f * t.slack * t.slack;
     t.tab = c->f64.tab.p;
     return t;
 }

@@ -112,7 +112,7 @@ __global__ void mp_cells_kernel(int n, const unsigned *__restrict__ key, int shi
 }
 
 // order of the expansion of a cell for a tile of points; 0: pair by pair
-__global__ void mp_order_kernel(int ntile, int ncell, int maxcell, const float4 *__restrict__ sph,
+__global__ void mp_order_kernel(int ntile, int ncell, int maxcell, F64Box box, const float4 *__restrict__ sph,
                                 const double *__restrict__ cxyz, const int *__restrict__ crad,
                                 const int *__restrict__ cbeg, const int *__restrict__ cend, float eps,
                                 unsigned char *__restrict__ order)
@@ -121,9 +121,10 @@ __global__ void mp_order_kernel(int ntile, int ncell, int maxcell, const float4 
     if (i >= ntile * ncell) return;
     const int t = i / ncell, c = i % ncell;
     const float4 s = sph[t];
-    const float dx = s.x - (float)cxyz[3 * c], dy = s.y - (float)cxyz[3 * c + 1], dz = s.z - (float)cxyz[3 * c + 2];
+    const float dx = s.x - (float)(cxyz[3 * c] - box.mid[0]), dy = s.y - (float)(cxyz[3 * c + 1] - box.mid[1]),
+                dz = s.z - (float)(cxyz[3 * c + 2] - box.mid[2]);
     const float r = fmaxf(__int_as_float(crad[c]), 1e-3f);
-    const float D = sqrtf(dx * dx + dy * dy + dz * dz) * 0.99999f - 2e-5f - s.w;
+    const float D = sqrtf(dx * dx + dy * dy + dz * dz) * 0.99999f - box.slack - s.w;
     int p = 0;
     if (D > r) {
         // two orders more for the pairs' own dipoles and quadrupoles
@@ -178,7 +179,7 @@ int mp_order(pcm_ctx *c, float eps)
     F64Mp &mp = c->f64.mp;
     const int no = mp.ncell * c->f64.ntile;
     mp_order_kernel<<<(no + 127) / 128, 128, 0, c->stream>>>(
-        c->f64.ntile, mp.ncell, mp.ncell, c->f64.pt_sph.p, mp.cxyz.p, mp.crad.p, mp.range.p,
+        c->f64.ntile, mp.ncell, mp.ncell, c->f64.box, c->f64.pt_sph.p, mp.cxyz.p, mp.crad.p, mp.range.p,
         mp.range.p + 6 * (size_t)mp.ncell, eps, mp.order.p);
     PCM_LAUNCHED(c);
     return PCM_OK;

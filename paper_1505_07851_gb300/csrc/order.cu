@@ -42,8 +42,13 @@ F64Box cavity_box(pcm_ctx *c, double cell)
             hi = std::max(hi, c->h_xyz[3 * I + d] + c->h_radius[I]);
         }
         box.lo[d] = lo;
+        box.mid[d] = lo + 0.5 * (hi - lo);
         ext = std::max(ext, hi - lo);
     }
+    // an FP32 coordinate of up to ext / 2 is off by 2^-25 of ext, the difference of two by
+    // 2^-23, so a distance by less than 2^-22; beyond 1e18 bohr, where squares leave
+    // FP32, there is no bound and every test errs on the FP64 side
+    box.slack = ext < 2e18 ? (float)(ext * 0x1p-21) : INFINITY;
     box.inv = 1.0 / (std::max(cell, ext * (1.0 + 1e-9) / (1 << CURVE_HBITS)) * (1 << CURVE_HBITS));
     return box;
 }

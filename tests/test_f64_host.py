@@ -57,3 +57,43 @@ int main()
 }
 """)
     assert int(out[0]) == 0 and int(out[1]) > 100000
+
+
+def test_fp32_distance_tests_are_safe(tmp_path):
+    """The FP32 tests never miss an interaction whose T, in 64 bits, is below the
+    threshold: cavities of 10 to 1e24 bohr, exponents from 1e-3 to 1e36, pairs and points
+    close together and far apart, at the same FP32 coordinates as the kernels'."""
+    out = run_host(tmp_path, """
+static double u() { static unsigned long long s = 42; s = s * 6364136223846793005ull + 1442695040888963407ull;
+                    return (double)(s >> 11) * 0x1p-53; }
+int main()
+{
+    long bad = 0, hit = 0;
+    for (double ext = 10.0; ext < 1e24; ext *= 7.0) {
+        const float slack = ext < 2e18 ? (float)(ext * 0x1p-21) : INFINITY, pad = 2001.f * slack * slack;
+        for (int i = 0; i < 20000; ++i) {
+            const double p = pow(10.0, u() * (i % 10 ? 6.0 : 39.0) - 3.0), z2 = 1.0 + 60.0 * u(), rho = p * z2 / (p + z2);
+            double P[3], C[3], R2 = 0.0;
+            const double far = sqrt(50.0 / rho) * 2.0 * u();
+            for (int d = 0; d < 3; ++d) {
+                P[d] = (u() - 0.5) * ext;
+                C[d] = fmin(fmax(P[d] + far * (u() - 0.5) * 2.0, -0.5 * ext), 0.5 * ext);
+                R2 += (P[d] - C[d]) * (P[d] - C[d]);
+            }
+            const float4 b = make_float4((float)P[0], (float)P[1], (float)P[2], (float)fmin(p, 1e30));
+            const float4 c = make_float4((float)C[0], (float)C[1], (float)C[2], (float)(1.0 / z2));
+            const float4 s = make_float4(c.x, c.y, c.z, slack);
+            for (int L = 0; L <= 5; ++L) {
+                const float top = (float)f64_far_T(L);
+                if (!(rho * R2 < top)) continue;
+                ++hit;
+                if (!f64_reaches(b, s, (float)z2 * 0.99999f, top, slack)) ++bad;
+                if (!f64_is_near(b.x - c.x, b.y - c.y, b.z - c.z, 1.f / b.w + c.w, top, pad)) ++bad;
+            }
+        }
+    }
+    printf("%ld %ld\\n", bad, hit);
+    return 0;
+}
+""")
+    assert int(out[0]) == 0 and int(out[1]) > 100000
