@@ -131,10 +131,10 @@ struct F64Mp {
     DBuf<int> range;                       // 6 x cells first sorted pair of each class, 6 x cells end
     DBuf<double> cxyz;                     // centres
     DBuf<int> crad;                        // radii (FP32 bits)
-    DBuf<unsigned char> order;             // tiles x cells: order of the expansion, 0: none
-    DBuf<double2> raw, M, mom;             // sums per class, moments, scaled moments (or their derivatives)
+    DBuf<unsigned char> order;             // tiles x cells: order of the expansion and its level, 0: none
+    DBuf<double2> raw, M, mom;             // sums per class, moments per level, their scaled derivatives
     int lsplit = 1;
-    DBuf<double2> lam, tab;                // local expansions, their coefficients per set
+    DBuf<double2> lam, tab;                // local expansions per level, their coefficients per set
     DBuf<double> V;                        // sets x pairs
 };
 struct F64Int {
@@ -373,10 +373,10 @@ int f64_charges(pcm_ctx *c, const double *dq, bool gradient);
 int f64_w(pcm_ctx *c, int k, bool esp, double *W);
 int mp_prepare(pcm_ctx *c, const F64Box &box, const F64Src &src, int bits, int shift);
 int mp_rows(pcm_ctx *c);
-int mp_order(pcm_ctx *c, float eps);
+int mp_order(pcm_ctx *c, bool gradient);
 int mp_grad_far(pcm_ctx *c, double *part);
 int mp_local(pcm_ctx *c);
-int mp_l2p(pcm_ctx *c, int L, int n, const int *list, int first);
+int mp_l2p(pcm_ctx *c, int level, int L, int n, const int *list, int first);
 int surface_build(pcm_ctx *c, int natom, const double *xyz, const double *Z, const double *radius, int n);
 int basis_build(pcm_ctx *c, int nshell, const int *shell_atom, const int *shell_l, const int *shell_nprim,
                 const double *exps, const double *coefs);

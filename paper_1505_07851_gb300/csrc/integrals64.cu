@@ -31,15 +31,20 @@ namespace pcm {
 
 constexpr int F64_LSUM[6] = {0, 1, 2, 2, 3, 4};
 constexpr int F64_SORT_POINTS = 1024;     // fewer points than this stay in library order
-constexpr double F64_CELL = 3.0;          // side of a cell (bohr)
+// side of a cell (bohr).  2.5 / 3.0: Fock correction of 150 s/sp atoms 28.5 / 29.4 ms, of 300
+// 92.2 / 88.9, gradient of 150 83.0 / 90.3, of 180 s/p/d atoms 170 / 179 (2.0: 30.6, 104.8, 83.8, 173)
+constexpr double F64_CELL = 2.5;
 constexpr int F64_PTBITS = 6;             // cells per side of the points' grid
 constexpr int F64_RC_CLASSES = 16;        // up to this many exponent classes rho and cn are tabulated per (class, pair)
-// from this many pairs and points on the cells' expansions are used: setting them up
-// costs about as much per pair as 130 (ss) to 250 (pp) points one by one.  Measured
-// without and with them: 60 atoms (2.9k points) 8.4 / 9.7 ms with d shells, 5.5 / 5.3
-// without; 80 atoms 9.3 / 7.6; 150 atoms 39.4 / 23.3; 300 atoms 158 / 63
+// From this many pairs and points on the cells' expansions are used: setting them up costs
+// as much per pair as some hundred points one by one, and more with d shells, whose
+// level is expanded for distant tiles only.  Measured without and with them, Fock
+// correction / gradient: s and p shells 3.4k points 8.56 / 8.81 and 25.5 / 26.1 ms, 4.2k
+// 12.5 / 11.8 and 37.2 / 35.2, 11.8k 158 / 92 (Fock); with d shells 4.6k 21.5 / 23.0 and
+// 64.0 / 64.3, 5.1k 26.0 / 26.4 and 76.9 / 74.1, 7.8k (gradient) 224 / 170
 constexpr int F64_MP_PAIRS = 40000;
-constexpr int F64_MP_POINTS = 3000;
+constexpr int F64_MP_POINTS = 3500;
+constexpr int F64_MP_POINTS_D = 5000;
 // thread blocks that a launch aims at: many more than fit, so that blocks with few
 // expanded cells and blocks with many even out (300-atom Fock: 82.9 ms with 16 per
 // SM, 75.7 with 32, 73.4 with 64)
@@ -261,7 +266,8 @@ int f64_prepare(pcm_ctx *c)
                                                                   c->cls_zeta.p, box, f.ord.p, f.P.p, f.info.p,
                                                                   f.use_rc ? f.rc.p : nullptr);
     PCM_LAUNCHED(c);
-    if (n >= F64_MP_PAIRS && M >= F64_MP_POINTS) PCM_TRY(mp_prepare(c, box, src, CURVE_HBITS, CURVE_PBITS));
+    const int points = f.off[6] > f.off[3] ? F64_MP_POINTS_D : F64_MP_POINTS;   // ds, dp or dd pairs
+    if (n >= F64_MP_PAIRS && M >= points) PCM_TRY(mp_prepare(c, box, src, CURVE_HBITS, CURVE_PBITS));
     return PCM_OK;
 }
 
@@ -481,8 +487,14 @@ struct F64Pairs {
     const double *rec;       // ESP records
     const int *cell;         // cell of every sorted pair, and the order of its expansion
     const unsigned char *order;   // for every (tile, cell); null: no expansions
+    unsigned char omask;     // bits of an order that say it serves the class
     int ncell;
 };
+
+__device__ __forceinline__ bool f64_expanded(const F64Pairs &a, int tile, int cell)
+{
+    return (a.order[(size_t)tile * a.ncell + cell] & a.omask) != 0;
+}
 
 __device__ __forceinline__ double2 f64_load_rc(const F64Pairs &a, const F64Points &t, int e, int pos)
 {
@@ -552,7 +564,7 @@ __global__ void __launch_bounds__(128, f64_min_blocks(far_nterms(L)))
             const int pos = a.list[j0 + lane];
             info = a.info[pos];
             nr = f64_reaches(info, sph, t.zmin2, FT, t.slack);
-            ex = a.order && a.order[(size_t)tile * a.ncell + a.cell[pos]] != 0;
+            ex = a.order && f64_expanded(a, tile, a.cell[pos]);
         }
         const unsigned nm = __ballot_sync(0xffffffffu, nr), em = __ballot_sync(0xffffffffu, ex);
         const unsigned direct = __ballot_sync(0xffffffffu, act) & ~em;
@@ -639,7 +651,7 @@ __global__ void __launch_bounds__(128, f64_min_blocks(far_nterms(L)))
     const float ip = 1.f / info.w;
     for (int tile = blockIdx.y; tile < t.ntile; tile += gridDim.y) {
         const bool reaches = f64_reaches(info, t.sph[tile], t.zmin2, FT, t.slack);
-        const bool expanded = a.order && a.order[(size_t)tile * a.ncell + cell] != 0;
+        const bool expanded = a.order && f64_expanded(a, tile, cell);
         const int s0 = tile * 32, nt = min(32, t.M - s0);
         if (!__all_sync(0xffffffffu, expanded)) {
             // one by one: every point, near or far by T where some pair reaches the tile
@@ -791,6 +803,7 @@ static F64Pairs f64_pairs(pcm_ctx *c, int k, bool esp)
     a.rec = esp ? f.rec.p + f.roff[k] : nullptr;
     a.cell = f.mp.pcell.p;
     a.order = f.mp.on ? f.mp.order.p : nullptr;
+    a.omask = mp_level(k) == 0 ? 0xff : MP_ALL;
     a.ncell = f.mp.ncell;
     return a;
 }
@@ -830,7 +843,7 @@ int f64_grad_point(pcm_ctx *c, const double *dq, double *gk)
     PCM_TRY(c->esp_part.alloc(total * 3 * S));
     double *part = c->esp_part.p;
     if (far) {
-        PCM_TRY(mp_order(c, MP_EPS_GRAD));
+        PCM_TRY(mp_order(c, true));
         PCM_TRY(mp_grad_far(c, part));
         part += (size_t)far * 3 * S;
     }
@@ -856,14 +869,14 @@ int f64_charges(pcm_ctx *c, const double *dq, bool gradient)
     f64_point_charge_kernel<<<(c->M + 127) / 128, 128, 0, c->stream>>>(c->M, c->f64.pt_idx.p, dq, c->f64.pt_xyz.p);
     PCM_LAUNCHED(c);
     if (c->f64.mp.on) {
-        PCM_TRY(mp_order(c, gradient ? MP_EPS_GRAD : MP_EPS));
+        PCM_TRY(mp_order(c, gradient));
         PCM_TRY(mp_local(c));
     }
     return PCM_OK;
 }
 
 template <int L>
-static int f64_w_launch(pcm_ctx *c, const F64Pairs &a, const int *ord, double *W)
+static int f64_w_launch(pcm_ctx *c, const F64Pairs &a, int level, const int *ord, double *W)
 {
     const int nb = (a.n + 127) / 128;
     const int rows = std::max(1, std::min(c->f64.ntile, (F64_CTAS + nb - 1) / nb));
@@ -875,7 +888,7 @@ static int f64_w_launch(pcm_ctx *c, const F64Pairs &a, const int *ord, double *W
         f64_rows_kernel<<<(unsigned)((ns + 127) / 128), 128, 0, c->stream>>>(ns, rows, c->f64.S.p);
         PCM_LAUNCHED(c);
     }
-    if (c->f64.mp.on) PCM_TRY(mp_l2p(c, L, a.n, a.list, a.first));
+    if (c->f64.mp.on) PCM_TRY(mp_l2p(c, level, L, a.n, a.list, a.first));
     f64_fold_kernel<L><<<(a.n + 31) / 32, 32, 0, c->stream>>>(a, rows > 2 ? 1 : rows, c->f64.S.p, c->f64.mp.on ? c->f64.mp.V.p : nullptr, ord,
                                                  a.n, W);
     PCM_LAUNCHED(c);
@@ -890,13 +903,14 @@ int f64_w(pcm_ctx *c, int k, bool esp, double *W)
     const F64Pairs a = f64_pairs(c, k, esp);
     if (a.n == 0) return PCM_OK;
     const int *ord = esp ? nullptr : c->f64.ord.p;
+    const int level = mp_level(k);
     switch (F64_LSUM[k] + (esp ? 1 : 0)) {
-    case 0: return f64_w_launch<0>(c, a, ord, W);
-    case 1: return f64_w_launch<1>(c, a, ord, W);
-    case 2: return f64_w_launch<2>(c, a, ord, W);
-    case 3: return f64_w_launch<3>(c, a, ord, W);
-    case 4: return f64_w_launch<4>(c, a, ord, W);
-    case 5: return f64_w_launch<5>(c, a, ord, W);
+    case 0: return f64_w_launch<0>(c, a, level, ord, W);
+    case 1: return f64_w_launch<1>(c, a, level, ord, W);
+    case 2: return f64_w_launch<2>(c, a, level, ord, W);
+    case 3: return f64_w_launch<3>(c, a, level, ord, W);
+    case 4: return f64_w_launch<4>(c, a, level, ord, W);
+    case 5: return f64_w_launch<5>(c, a, level, ord, W);
     }
     return PCM_ERR_ARG;
 }

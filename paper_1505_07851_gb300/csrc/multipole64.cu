@@ -20,10 +20,10 @@
 //   I_l^m = (2l-1)!! b_l ((x + iy)/r^2)^m / r,  u = z/r^2, v = 1/r^2,
 // three FP64 instructions per (l, m), then two per real sum.
 //
-// A cell is expanded for a tile of points when the first neglected term is below
-// a bound (MP_EPS) at the order MP_P or less (order from the ratio of the cell's
-// radius to the distance), and when the expansion costs less than its pairs do
-// one by one.  Pairs of such a cell that still have T < f64_far_T
+// A cell is expanded for a tile of points when some order up to MP_P leaves less
+// than its rounding out of any interaction (mp_order_for, with the highest
+// derivative that the classes of a level take), and when the expansion costs less
+// than its pairs do one by one.  Pairs of such a cell that still have T < f64_far_T
 // somewhere in the tile add near minus far form for those points.
 #include <math.h>
 
@@ -111,10 +111,12 @@ __global__ void mp_cells_kernel(int n, const unsigned *__restrict__ key, int shi
     atomicMax(&crad[cell], __float_as_int((float)sqrt(r2) * 1.000001f));
 }
 
-// order of the expansion of a cell for a tile of points; 0: pair by pair
+// Order of the expansion of a cell for a tile of points, with MP_ALL if it serves all
+// of the cell's classes, without if only those of level 0; 0: pair by pair.  extra:
+// derivatives beyond the pairs' own (the gradient's one)
 __global__ void mp_order_kernel(int ntile, int ncell, int maxcell, F64Box box, const float4 *__restrict__ sph,
                                 const double *__restrict__ cxyz, const int *__restrict__ crad,
-                                const int *__restrict__ cbeg, const int *__restrict__ cend, float eps,
+                                const int *__restrict__ cbeg, const int *__restrict__ cend, int extra,
                                 unsigned char *__restrict__ order)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -125,22 +127,28 @@ __global__ void mp_order_kernel(int ntile, int ncell, int maxcell, F64Box box, c
                 dz = s.z - (float)(cxyz[3 * c + 2] - box.mid[2]);
     const float r = fmaxf(__int_as_float(crad[c]), 1e-3f);
     const float D = sqrtf(dx * dx + dy * dy + dz * dz) * 0.99999f - box.slack - s.w;
-    int p = 0;
+    unsigned char o = 0;
     if (D > r) {
-        // two orders more for the pairs' own dipoles and quadrupoles
-        p = max(6, (int)ceilf(logf(eps) / logf(r / D)) + 2);
-        if (p > MP_P) {
-            p = 0;
-        } else {
-            // FP64 instructions per point: far forms of the cell's pairs
-            // (12 ... 95 by class) against 5 per (l, m) and 8 per m
-            const float cost[6] = {12.f, 19.f, 32.f, 32.f, 55.f, 95.f};
-            float direct = 0.f;
-            for (int k = 0; k < 6; ++k) direct += cost[k] * (float)(cend[k * maxcell + c] - cbeg[k * maxcell + c]);
-            if (direct < MP_GAIN * (2.5f * (p + 1) * (p + 2) + 8.f * (p + 1))) p = 0;
+        // FP64 instructions per point: far forms of the cell's pairs
+        // (12 ... 95 by class) against 5 per (l, m) and 8 per m
+        const float cost[6] = {12.f, 19.f, 32.f, 32.f, 55.f, 95.f};
+        const int deg[6] = {0, 1, 2, 2, 3, 4};
+        float direct[MP_LEVELS] = {0.f, 0.f};   // pairs up to each level
+        int n[MP_LEVELS] = {0, 0};
+        for (int k = 0; k < 6; ++k) {
+            const int pairs = cend[k * maxcell + c] - cbeg[k * maxcell + c];
+            for (int v = mp_level(k); v < MP_LEVELS; ++v) {
+                direct[v] += cost[k] * (float)pairs;
+                if (pairs > 0) n[v] = deg[k];
+            }
+        }
+        for (int v = 0; v < MP_LEVELS; ++v) {
+            const int p = mp_order_for(r / D, n[v] + extra);
+            if (p > 0 && direct[v] >= MP_GAIN * (2.5f * (p + 1) * (p + 2) + 8.f * (p + 1)))
+                o = (unsigned char)p | (v == MP_LEVELS - 1 ? MP_ALL : 0);
         }
     }
-    order[i] = (unsigned char)p;
+    order[i] = o;
 }
 
 int mp_prepare(pcm_ctx *c, const F64Box &box, const F64Src &src, int bits, int shift)
@@ -173,14 +181,14 @@ int mp_prepare(pcm_ctx *c, const F64Box &box, const F64Src &src, int bits, int s
     return PCM_OK;
 }
 
-// orders of the expansions for every (tile, cell) at the given accuracy
-int mp_order(pcm_ctx *c, float eps)
+// orders of the expansions for every (tile, cell)
+int mp_order(pcm_ctx *c, bool gradient)
 {
     F64Mp &mp = c->f64.mp;
     const int no = mp.ncell * c->f64.ntile;
     mp_order_kernel<<<(no + 127) / 128, 128, 0, c->stream>>>(
         c->f64.ntile, mp.ncell, mp.ncell, c->f64.box, c->f64.pt_sph.p, mp.cxyz.p, mp.crad.p, mp.range.p,
-        mp.range.p + 6 * (size_t)mp.ncell, eps, mp.order.p);
+        mp.range.p + 6 * (size_t)mp.ncell, gradient ? 1 : 0, mp.order.p);
     PCM_LAUNCHED(c);
     return PCM_OK;
 }
@@ -357,18 +365,27 @@ __global__ void __launch_bounds__(P2M_NT) mp_combine_kernel(int nsplit, bool fir
 }
 
 // the three sets of the moments' derivatives with respect to the pairs' centres,
-// scaled for mp_m2p_kernel: w_m (2l-1)!!
-__global__ void __launch_bounds__(P2M_NT) mp_scale_kernel(const double2 *__restrict__ M, double2 *__restrict__ out)
+// scaled for mp_m2p_kernel: w_m (2l-1)!!; of level 0 (blockIdx.y 0) and of both levels
+__global__ void __launch_bounds__(P2M_NT) mp_scale_kernel(int ncell, const double2 *__restrict__ M,
+                                                          double2 *__restrict__ out)
 {
+    __shared__ double2 v[MP_NLM];
     const int cell = blockIdx.x, i = threadIdx.x;
+    if (i < MP_NLM) {
+        v[i] = M[(size_t)cell * MP_NLM + i];
+        if (blockIdx.y > 0) {
+            const double2 x = M[((size_t)ncell + cell) * MP_NLM + i];
+            v[i] = make_double2(v[i].x + x.x, v[i].y + x.y);
+        }
+    }
+    __syncthreads();
     if (i >= MP_NLM) return;
     int m = 0;
     while (i >= mp_col(m + 1)) ++m;
     const int l = i - mp_col(m) + m;
-    const double2 *v = M + (size_t)cell * MP_NLM;
     const double s = c_mp.wd[i];
     const double2 a = mp_get(v, l - 1, m + 1), b = mp_get(v, l - 1, m - 1), z = mp_get(v, l - 1, m);
-    double2 *o = out + ((size_t)cell * MP_NLM + i) * 3;
+    double2 *o = out + (((size_t)blockIdx.y * ncell + cell) * MP_NLM + i) * 3;
     o[0] = make_double2(0.5 * s * (b.x - a.x), 0.5 * s * (b.y - a.y));
     // (-a - b) / (2i) = i (a + b) / 2
     o[1] = make_double2(-0.5 * s * (a.y + b.y), 0.5 * s * (a.x + b.x));
@@ -377,7 +394,8 @@ __global__ void __launch_bounds__(P2M_NT) mp_scale_kernel(const double2 *__restr
 
 // Point part of the gradient from the expanded cells: a warp per (tile, part of
 // the cells), a lane per point; part[row][component][slot] as f64_grad_kernel's
-// rows.  Nine FP64 instructions per (l, m): FP64-bound.
+// rows.  mom: the moments of level 0, then of all classes.  Nine FP64 instructions per
+// (l, m): FP64-bound.
 __global__ void __launch_bounds__(128) mp_m2p_kernel(int M, int ntile, int ncell, const F64Pt *__restrict__ xyz,
                                                      const unsigned char *__restrict__ order,
                                                      const double *__restrict__ cxyz, const double2 *__restrict__ mom,
@@ -391,14 +409,14 @@ __global__ void __launch_bounds__(128) mp_m2p_kernel(int M, int ntile, int ncell
 #pragma unroll
     for (int d = 0; d < NV; ++d) acc[d] = 0.0;
     for (int cell = blockIdx.y * 4 + w; cell < ncell; cell += 4 * gridDim.y) {
-        const int p = order[(size_t)tile * ncell + cell];
+        const int o8 = order[(size_t)tile * ncell + cell], p = o8 & ~MP_ALL;
         if (p == 0) continue;
         const double x = c.x - cxyz[3 * cell], y = c.y - cxyz[3 * cell + 1], z = c.z - cxyz[3 * cell + 2];
         double rs[1];
         f64_far<0>(fma(x, x, fma(y, y, z * z)), rs);
         const double v = rs[0] * rs[0], u = z * v, ex = x * v, ey = y * v;
         double er = rs[0], ei = 0.0;
-        const double2 *mc = mom + (size_t)cell * MP_NLM * NV;
+        const double2 *mc = mom + ((size_t)(o8 & MP_ALL ? ncell : 0) + cell) * MP_NLM * NV;
         for (int m = 0; m <= p; ++m) {
             const int o = mp_col(m) - m;
             double b1 = 1.0, b0 = 0.0, sr[NV], si[NV];
@@ -444,10 +462,11 @@ __global__ void __launch_bounds__(128) mp_m2p_kernel(int M, int ntile, int ncell
 constexpr int P2L_NW = 4;
 constexpr size_t P2L_SMEM = (size_t)P2L_NW * (2 * (MP_P + 1) * 33 + 2 * MP_NLM) * sizeof(double);
 
-// lam[split][cell][lm] = sum of q_k (2l-1)!!^-1 I_l^m(C_k - centre) over the
-// cell's tiles, a warp per share of the tiles: the lanes (points) write one
-// column m at a time to shared memory, then a lane per (l, part) adds its 32
-// values to the warp's sums.
+// lam[level][split][cell][lm] = sum of q_k (2l-1)!!^-1 I_l^m(C_k - centre) over the
+// cell's tiles (level 0: those expanded for it alone, level 1: those for all
+// classes), a warp per share of the tiles: the lanes (points) write one column m
+// at a time to shared memory, then a lane per (l, part) adds its 32 values to the
+// warp's sums.
 __global__ void __launch_bounds__(32 * P2L_NW) mp_p2l_kernel(int M, int ntile, int ncell,
                                                              const F64Pt *__restrict__ xyz,
                                                              const unsigned char *__restrict__ order,
@@ -461,8 +480,8 @@ __global__ void __launch_bounds__(32 * P2L_NW) mp_p2l_kernel(int M, int ntile, i
     __syncwarp();
     const double cx = cxyz[3 * cell], cy = cxyz[3 * cell + 1], cz = cxyz[3 * cell + 2];
     for (int tile = blockIdx.y * P2L_NW + w; tile < ntile; tile += gridDim.y * P2L_NW) {
-        const int p = order[(size_t)tile * ncell + cell];
-        if (p == 0) continue;
+        const int o8 = order[(size_t)tile * ncell + cell], p = o8 & ~MP_ALL;
+        if (p == 0 || (o8 & MP_ALL ? 1 : 0) != (int)blockIdx.z) continue;
         const bool on = tile * 32 + lane < M;
         const F64Pt c = xyz[min(tile * 32 + lane, M - 1)];
         const double x = c.x - cx, y = c.y - cy, z = c.z - cz;
@@ -501,7 +520,7 @@ __global__ void __launch_bounds__(32 * P2L_NW) mp_p2l_kernel(int M, int ntile, i
         }
     }
     __syncthreads();
-    double *out = reinterpret_cast<double *>(lam + ((size_t)blockIdx.y * ncell + cell) * MP_NLM);
+    double *out = reinterpret_cast<double *>(lam + (((size_t)blockIdx.z * gridDim.y + blockIdx.y) * ncell + cell) * MP_NLM);
     constexpr int ST = 2 * (MP_P + 1) * 33 + 2 * MP_NLM;
     for (int i = threadIdx.x; i < 2 * MP_NLM; i += 32 * P2L_NW) {
         double s = 0.0;
@@ -510,6 +529,7 @@ __global__ void __launch_bounds__(32 * P2L_NW) mp_p2l_kernel(int M, int ntile, i
     }
 }
 
+// lam: nsplit shares of the cell's tiles, those of a level and the ones above it.
 // Coefficients of V_s = sum_{l, m >= 0} b_l (Re e_m A + Im e_m B) for the sets s
 // = (n, mu, part) of a class: tab[cell][lm][s] = (A, B); one block per cell
 __global__ void __launch_bounds__(P2M_NT) mp_local_kernel(int ns, int nsplit, int ncell,
@@ -609,7 +629,7 @@ __global__ void __launch_bounds__(128) mp_l2p_kernel(int n, int stride, const in
 // host side
 // ---------------------------------------------------------------------------
 template <int L>
-static int mp_moments_class(pcm_ctx *c, int k, bool first)
+static int mp_moments_class(pcm_ctx *c, int k, bool first, double2 *M)
 {
     F64Int &f = c->f64;
     F64Mp &mp = f.mp;
@@ -624,7 +644,7 @@ static int mp_moments_class(pcm_ctx *c, int k, bool first)
         mp.ncell, mp.range.p + (size_t)k * mp.ncell, mp.range.p + (size_t)(6 + k) * mp.ncell, f.pos.p, f.eoff[k],
         f.rec.p + f.roff[k], f.B.p + f.boff[k], c->cls[k].nesp, mp.cxyz.p, mp.raw.p);
     PCM_LAUNCHED(c);
-    mp_combine_kernel<L><<<mp.ncell, P2M_NT, 0, c->stream>>>(split, first, mp.raw.p, mp.M.p);
+    mp_combine_kernel<L><<<mp.ncell, P2M_NT, 0, c->stream>>>(split, first, mp.raw.p, M);
     PCM_LAUNCHED(c);
     return PCM_OK;
 }
@@ -640,22 +660,26 @@ int mp_grad_far(pcm_ctx *c, double *part)
 {
     F64Int &f = c->f64;
     F64Mp &mp = f.mp;
-    PCM_TRY(mp.M.alloc((size_t)mp.ncell * MP_NLM));
-    bool first = true;
+    const size_t nm = (size_t)mp.ncell * MP_NLM;
+    PCM_TRY(mp.M.alloc(MP_LEVELS * nm));
+    PCM_CUDA(cudaMemsetAsync(mp.M.p, 0, MP_LEVELS * nm * sizeof(double2), c->stream));   // levels without pairs
+    bool first[MP_LEVELS] = {true, true};
     for (int k = 0; k < 6; ++k) {
         if (c->cls[k].nesp == 0) continue;
+        const int v = mp_level(k);
+        double2 *M = mp.M.p + v * nm;
         switch (k) {
-        case 0: PCM_TRY(mp_moments_class<0>(c, k, first)); break;
-        case 1: PCM_TRY(mp_moments_class<1>(c, k, first)); break;
+        case 0: PCM_TRY(mp_moments_class<0>(c, k, first[v], M)); break;
+        case 1: PCM_TRY(mp_moments_class<1>(c, k, first[v], M)); break;
         case 2:
-        case 3: PCM_TRY(mp_moments_class<2>(c, k, first)); break;
-        case 4: PCM_TRY(mp_moments_class<3>(c, k, first)); break;
-        case 5: PCM_TRY(mp_moments_class<4>(c, k, first)); break;
+        case 3: PCM_TRY(mp_moments_class<2>(c, k, first[v], M)); break;
+        case 4: PCM_TRY(mp_moments_class<3>(c, k, first[v], M)); break;
+        case 5: PCM_TRY(mp_moments_class<4>(c, k, first[v], M)); break;
         }
-        first = false;
+        first[v] = false;
     }
-    PCM_TRY(mp.mom.alloc((size_t)mp.ncell * MP_NLM * 3));
-    mp_scale_kernel<<<mp.ncell, P2M_NT, 0, c->stream>>>(mp.M.p, mp.mom.p);
+    PCM_TRY(mp.mom.alloc(MP_LEVELS * nm * 3));
+    mp_scale_kernel<<<dim3(mp.ncell, MP_LEVELS), P2M_NT, 0, c->stream>>>(mp.ncell, mp.M.p, mp.mom.p);
     PCM_LAUNCHED(c);
     mp_m2p_kernel<<<dim3(f.ntile, mp_rows(c)), 128, 0, c->stream>>>(c->M, f.ntile, mp.ncell, f.pt_xyz.p, mp.order.p,
                                                                    mp.cxyz.p, mp.mom.p, part);
@@ -669,23 +693,25 @@ int mp_local(pcm_ctx *c)
     F64Int &f = c->f64;
     F64Mp &mp = f.mp;
     mp.lsplit = std::max(1, std::min((f.ntile + P2L_NW - 1) / P2L_NW, (152 * 16 + mp.ncell - 1) / mp.ncell));
-    PCM_TRY(mp.lam.alloc((size_t)mp.lsplit * mp.ncell * MP_NLM));
+    PCM_TRY(mp.lam.alloc(MP_LEVELS * (size_t)mp.lsplit * mp.ncell * MP_NLM));
     PCM_CUDA(cudaFuncSetAttribute(mp_p2l_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P2L_SMEM));
-    mp_p2l_kernel<<<dim3(mp.ncell, mp.lsplit), 32 * P2L_NW, P2L_SMEM, c->stream>>>(
+    mp_p2l_kernel<<<dim3(mp.ncell, mp.lsplit, MP_LEVELS), 32 * P2L_NW, P2L_SMEM, c->stream>>>(
         c->M, f.ntile, mp.ncell, f.pt_xyz.p, mp.order.p, mp.cxyz.p, mp.lam.p);
     PCM_LAUNCHED(c);
     return PCM_OK;
 }
 
-// V[(L+1)^2][n] at the pairs (list, or the sorted positions from first)
-int mp_l2p(pcm_ctx *c, int L, int n, const int *list, int first)
+// V[(L+1)^2][n] at the pairs (list, or the sorted positions from first) of a level
+int mp_l2p(pcm_ctx *c, int level, int L, int n, const int *list, int first)
 {
     F64Int &f = c->f64;
     F64Mp &mp = f.mp;
     const int ns = (L + 1) * (L + 1);
     PCM_TRY(mp.V.alloc((size_t)ns * n));
     PCM_TRY(mp.tab.alloc((size_t)mp.ncell * MP_NLM * ns));
-    mp_local_kernel<<<mp.ncell, P2M_NT, 0, c->stream>>>(ns, mp.lsplit, mp.ncell, mp.lam.p, mp.tab.p);
+    mp_local_kernel<<<mp.ncell, P2M_NT, 0, c->stream>>>(ns, (MP_LEVELS - level) * mp.lsplit, mp.ncell,
+                                                        mp.lam.p + (size_t)level * mp.lsplit * mp.ncell * MP_NLM,
+                                                        mp.tab.p);
     PCM_LAUNCHED(c);
     const int nb = (n + 127) / 128;
     const int *pc = mp.pcell.p;

@@ -1,6 +1,7 @@
 """Host evaluation of the rules that send FP64 interactions to tables and expansions
 (the same functions the kernels call, compiled for the CPU): no argument leaves the
 table, and every argument that the table serves is within its range."""
+import math
 import os
 import subprocess
 
@@ -97,3 +98,33 @@ int main()
 }
 """)
     assert int(out[0]) == 0 and int(out[1]) > 100000
+
+
+def test_expansion_orders(tmp_path):
+    """The order of a cell's expansion: what it leaves out of an n-th derivative of 1/R,
+    summed in Python, is below 2n + 1 units of 2^-53 of the leading term, and one order
+    less leaves more."""
+    out = run_host(tmp_path, """
+int main()
+{
+    for (int n = 0; n <= 5; ++n)
+        for (int i = 1; i <= 120; ++i) printf("%d %d %d\\n", n, i, mp_order_for((float)i / 256.f, n));
+    printf("%d 0 0\\n", MP_P);
+    return 0;
+}
+""", include="multipole64.cuh")
+    v = [int(x) for x in out]
+    top = v[-3]
+
+    def left(x, n, p):
+        return sum(math.comb(l, n) * x ** (l - n) for l in range(p + 1, p + 400))
+
+    for n, i, p in zip(v[:-3:3], v[1:-3:3], v[2:-3:3]):
+        x, eps = i / 256.0, (2 * n + 1) * 2.0 ** -53
+        if p:
+            assert left(x, n, p) <= eps * 1.0001, (x, n, p)
+        if p > max(n, 1):
+            assert left(x, n, p - 1) > 0.9 * eps, (x, n, p)
+        if p == 0:
+            assert left(x, n, top) > 0.9 * eps, (x, n)
+    assert any(v[2:-3:3])

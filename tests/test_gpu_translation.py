@@ -8,13 +8,14 @@ element."""
 import numpy as np
 import pytest
 
+import _expansions
 import workloads
 from _parity import check
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("natom,d_shells", [(12, True), (80, True)])
+@pytest.mark.parametrize("natom,d_shells", [(12, True), (130, True)])
 def test_translation(natom, d_shells):
     import paper_1505_07851_gb300 as pcm
     w = workloads.small_cluster(natom, seed=71, d_shells=d_shells)
@@ -26,6 +27,7 @@ def test_translation(natom, d_shells):
             M = ctx.build_surface(w.mol.xyz + np.array(shift), w.mol.Z, w.mol.radius)
             b = w.basis
             ctx.set_basis(b.shell_atom, b.shell_l, b.shell_nprim, b.exps, b.coefs)
+            assert natom < 100 or _expansions.on(ctx.stats(), d_shells)
             q = np.random.default_rng(8).uniform(-1.0, 0.3, M) * 1e-2
             got.append((ctx.get_surface()[1], ctx.fock(q), ctx.gradient(q, w.P, terms="C")))
     assert np.array_equal(got[0][0], got[1][0])
