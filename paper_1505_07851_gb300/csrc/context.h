@@ -130,7 +130,7 @@ struct F64Mp {
     DBuf<int> id, pcell;                   // grid cell -> cell; cell of every sorted pair
     DBuf<int> range;                       // 6 x cells first sorted pair of each class, 6 x cells end
     DBuf<double> cxyz;                     // centres
-    DBuf<int> crad;                        // radii (FP32 bits)
+    DBuf<int> crad, cpmin;                 // radii, smallest exponents (FP32 bits)
     DBuf<unsigned char> order;             // tiles x cells: order of the expansion and its level, 0: none
     DBuf<double2> raw, M, mom;             // sums per class, moments per level, their scaled derivatives
     int lsplit = 1;

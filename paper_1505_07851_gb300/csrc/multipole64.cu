@@ -22,8 +22,9 @@
 //
 // A cell is expanded for a tile of points when some order up to MP_P leaves less
 // than its rounding out of any interaction (mp_order_for, with the highest
-// derivative that the classes of a level take), and when the expansion costs less
-// than its pairs do one by one.  Pairs of such a cell that still have T < f64_far_T
+// derivative that the classes of a level take), when all interactions have
+// T >= F64_H_MIN (the near form of more diffuse pairs is far below their far
+// form), and when the expansion costs less than its pairs do one by one.  Pairs of such a cell that still have T < f64_far_T
 // somewhere in the tile add near minus far form for those points.
 #include <math.h>
 
@@ -76,12 +77,13 @@ __global__ void mp_mark_kernel(int n, const unsigned *__restrict__ key, int shif
     if (g < n) flag[(key[g] >> shift) & mask] = 1;
 }
 
-// cell of every sorted pair, the cells' ranges per class, centres and radii
+// cell of every sorted pair, the cells' ranges per class, centres, radii and smallest
+// exponents
 __global__ void mp_cells_kernel(int n, const unsigned *__restrict__ key, int shift, unsigned mask,
                                 const int *__restrict__ id, F64Src src, F64Box box, int side,
                                 const double *__restrict__ P, int maxcell, int *__restrict__ pcell,
                                 int *__restrict__ cbeg, int *__restrict__ cend, double *__restrict__ cxyz,
-                                int *__restrict__ crad)
+                                int *__restrict__ crad, int *__restrict__ cpmin)
 {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= n) return;
@@ -109,6 +111,7 @@ __global__ void mp_cells_kernel(int n, const unsigned *__restrict__ key, int shi
     if (g == n - 1 || (key[g + 1] >> shift) != kg) cend[k * maxcell + cell] = g + 1;
     // largest distance (non-negative floats order as integers), rounded up
     atomicMax(&crad[cell], __float_as_int((float)sqrt(r2) * 1.000001f));
+    atomicMin(&cpmin[cell], __float_as_int((float)fmin(P[3 * (size_t)n + g], 1e30) * 0.999999f));
 }
 
 // Order of the expansion of a cell for a tile of points, with MP_ALL if it serves all
@@ -116,7 +119,8 @@ __global__ void mp_cells_kernel(int n, const unsigned *__restrict__ key, int shi
 // derivatives beyond the pairs' own (the gradient's one)
 __global__ void mp_order_kernel(int ntile, int ncell, int maxcell, F64Box box, const float4 *__restrict__ sph,
                                 const double *__restrict__ cxyz, const int *__restrict__ crad,
-                                const int *__restrict__ cbeg, const int *__restrict__ cend, int extra,
+                                const int *__restrict__ cpmin, float zmin2, const int *__restrict__ cbeg,
+                                const int *__restrict__ cend, int extra,
                                 unsigned char *__restrict__ order)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -128,7 +132,10 @@ __global__ void mp_order_kernel(int ntile, int ncell, int maxcell, F64Box box, c
     const float r = fmaxf(__int_as_float(crad[c]), 1e-3f);
     const float D = sqrtf(dx * dx + dy * dy + dz * dz) * 0.99999f - box.slack - s.w;
     unsigned char o = 0;
-    if (D > r) {
+    // smallest T of an interaction: below F64_H_MIN the near form is the difference of
+    // two larger numbers
+    const float pm = __int_as_float(cpmin[c]), rho = pm / (pm + zmin2) * zmin2;
+    if (D > r && rho * (D - r) * (D - r) >= 1.0001f * (float)F64_H_MIN) {
         // FP64 instructions per point: far forms of the cell's pairs
         // (12 ... 95 by class) against 5 per (l, m) and 8 per m
         const float cost[6] = {12.f, 19.f, 32.f, 32.f, 55.f, 95.f};
@@ -170,12 +177,15 @@ int mp_prepare(pcm_ctx *c, const F64Box &box, const F64Src &src, int bits, int s
     PCM_TRY(mp.range.alloc(12 * (size_t)cnt));
     PCM_TRY(mp.cxyz.alloc(3 * (size_t)cnt));
     PCM_TRY(mp.crad.alloc(cnt));
+    PCM_TRY(mp.cpmin.alloc(cnt));
     PCM_TRY(mp.order.alloc((size_t)cnt * c->f64.ntile));
     PCM_CUDA(cudaMemsetAsync(mp.range.p, 0, 12 * (size_t)cnt * sizeof(int), c->stream));
     PCM_CUDA(cudaMemsetAsync(mp.crad.p, 0, (size_t)cnt * sizeof(int), c->stream));
+    PCM_CUDA(cudaMemsetAsync(mp.cpmin.p, 0x7f, (size_t)cnt * sizeof(int), c->stream));   // above any exponent
     mp_cells_kernel<<<(n + 127) / 128, 128, 0, c->stream>>>(n, c->f64.key.p, shift, nc - 1, mp.id.p, src, box, side,
                                                            c->f64.P.p, cnt, mp.pcell.p, mp.range.p,
-                                                           mp.range.p + 6 * (size_t)cnt, mp.cxyz.p, mp.crad.p);
+                                                           mp.range.p + 6 * (size_t)cnt, mp.cxyz.p, mp.crad.p,
+                                                           mp.cpmin.p);
     PCM_LAUNCHED(c);
     mp.on = true;
     return PCM_OK;
@@ -187,7 +197,8 @@ int mp_order(pcm_ctx *c, bool gradient)
     F64Mp &mp = c->f64.mp;
     const int no = mp.ncell * c->f64.ntile;
     mp_order_kernel<<<(no + 127) / 128, 128, 0, c->stream>>>(
-        c->f64.ntile, mp.ncell, mp.ncell, c->f64.box, c->f64.pt_sph.p, mp.cxyz.p, mp.crad.p, mp.range.p,
+        c->f64.ntile, mp.ncell, mp.ncell, c->f64.box, c->f64.pt_sph.p, mp.cxyz.p, mp.crad.p,
+        mp.cpmin.p, (float)(c->h_cls_zeta[0] * c->h_cls_zeta[0]) * 0.99999f, mp.range.p,
         mp.range.p + 6 * (size_t)mp.ncell, gradient ? 1 : 0, mp.order.p);
     PCM_LAUNCHED(c);
     return PCM_OK;
