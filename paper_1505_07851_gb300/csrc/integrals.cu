@@ -254,13 +254,13 @@ __global__ void esp_reduce_kernel(int M, int nseg, const double *__restrict__ pa
     c[k] = s;
 }
 
-// Fock epilogue: EPI_LANES lanes per shell pair share its kept primitive pairs.
-// For each, L_ab = -(2 pi/p) K sum_tuv E^{ab}_tuv W_tuv is contracted with c_a c_b
+// Fock epilogue: LANES lanes per shell pair (EPI_LANES or one, fock_epilogue below) share
+// its kept primitive pairs.  For each, L_ab = -(2 pi/p) K sum_tuv E^{ab}_tuv W_tuv is contracted with c_a c_b
 // (Eq. 16); the lanes' sums are added by a butterfly (Eq. 17).  A diagonal shell
 // pair's off-diagonal primitive pair also adds its mirror image.  Both dF
 // blocks (A,B) and (B,A) are written; every element of dF is written.
 constexpr int EPI_LANES = 8;
-template <int LA, int LB>
+template <int LA, int LB, int LANES>
 __global__ void fock_epilogue_kernel(int nsp, int npair, int nsplit, const int *__restrict__ spA,
                                      const int *__restrict__ spB, const int *__restrict__ sp_start,
                                      const int *__restrict__ ia, const int *__restrict__ ib,
@@ -275,13 +275,13 @@ __global__ void fock_epilogue_kernel(int nsp, int npair, int nsplit, const int *
     constexpr int NH = nherm(L);
     constexpr int NA = ncart(LA), NB = ncart(LB);
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int s = min(t / EPI_LANES, nsp - 1);
+    const int s = min(t / LANES, nsp - 1);
     const int A = spA[s], B = spB[s];
     const double *RA = xyz + 3 * sh_atom[A], *RB = xyz + 3 * sh_atom[B];
     double G[NA * NB];
 #pragma unroll
     for (int t = 0; t < NA * NB; ++t) G[t] = 0.0;
-    for (int r = sp_start[s] + t % EPI_LANES; r < sp_start[s + 1]; r += EPI_LANES) {
+    for (int r = sp_start[s] + t % LANES; r < sp_start[s + 1]; r += LANES) {
         double w[NH];
 #pragma unroll
         for (int h = 0; h < NH; ++h) {
@@ -322,8 +322,8 @@ __global__ void fock_epilogue_kernel(int nsp, int npair, int nsplit, const int *
 #pragma unroll
     for (int i = 0; i < NA * NB; ++i)
 #pragma unroll
-        for (int o = EPI_LANES / 2; o > 0; o >>= 1) G[i] += __shfl_xor_sync(0xffffffffu, G[i], o);
-    if (t % EPI_LANES != 0 || t / EPI_LANES >= nsp) return;
+        for (int o = LANES / 2; o > 0; o >>= 1) G[i] += __shfl_xor_sync(0xffffffffu, G[i], o);
+    if (t % LANES != 0 || t / LANES >= nsp) return;
     const int fa = sh_bf[A], fb = sh_bf[B];
 #pragma unroll
     for (int a = 0; a < NA; ++a)
@@ -812,12 +812,32 @@ static int fock_tune(pcm_ctx *c, int k, int L, const double *dq)
     return PCM_OK;
 }
 
+template <int LA, int LB, int LANES>
+static void fock_epilogue_launch(pcm_ctx *c, PairClass &pc, int nsplit, const double *W, double *ddF)
+{
+    fock_epilogue_kernel<LA, LB, LANES><<<(unsigned)(((long long)pc.nsp * LANES + 127) / 128), 128, 0, c->stream>>>(
+        pc.nsp, pc.npair, nsplit, pc.spA.p, pc.spB.p, pc.sp_start.p, pc.ia.p, pc.ib.p, c->sh_atom.p, c->sh_off.p,
+        c->sh_bf.p, c->cnorm.p, c->xyz.p, pc.Px.p, pc.Py.p, pc.Pz.p, pc.p.p, pc.pref.p, W, c->nbf, ddF);
+}
+
+// EPI_LANES lanes per shell pair while a class has so few elements of dF that a thread per
+// shell pair leaves the chip waiting for each thread's chain of primitive pairs; beyond,
+// the lanes' butterflies (and lanes without a pair: most shell pairs of a large molecule
+// keep none) cost more.  The line is lower where shell pairs have few primitive pairs to
+// share.  Eight lanes / one, in us: dd 7.6k elements 177 / 209, 408k 610 / 284, 4.5M 1500 /
+// 703; dp 14k 79 / 184, 818k 500 / 338, 9.1M 2000 / 1100; ds 678k 172 / 141, 7.5M 773 / 410; pp
+// 150k 98 / 300, 1.1M 276 / 343, 4.6M 640 / 586; ps 684k 127 / 154, 7.6M 665 / 416; ss 284k 36 /
+// 38, 3.2M 205 / 100 (40 to 1000 atoms).
+constexpr int EPI_PAIRS = 3;
+constexpr long long EPI_ELEMENTS = 1 << 21, EPI_ELEMENTS_FEW = 1 << 18;
 template <int LA, int LB>
 static void fock_epilogue(pcm_ctx *c, PairClass &pc, int nsplit, const double *W, double *ddF)
 {
-    fock_epilogue_kernel<LA, LB><<<(unsigned)(((long long)pc.nsp * EPI_LANES + 127) / 128), 128, 0, c->stream>>>(
-        pc.nsp, pc.npair, nsplit, pc.spA.p, pc.spB.p, pc.sp_start.p, pc.ia.p, pc.ib.p, c->sh_atom.p, c->sh_off.p,
-        c->sh_bf.p, c->cnorm.p, c->xyz.p, pc.Px.p, pc.Py.p, pc.Pz.p, pc.p.p, pc.pref.p, W, c->nbf, ddF);
+    const long long limit = pc.ncand >= (long long)EPI_PAIRS * pc.nsp ? EPI_ELEMENTS : EPI_ELEMENTS_FEW;
+    if ((long long)pc.nsp * ncart(LA) * ncart(LB) <= limit)
+        fock_epilogue_launch<LA, LB, EPI_LANES>(c, pc, nsplit, W, ddF);
+    else
+        fock_epilogue_launch<LA, LB, 1>(c, pc, nsplit, W, ddF);
 }
 
 // the Fock epilogues a batch deferred until its packed blocks had run
