@@ -50,6 +50,12 @@ constexpr int F64_MP_POINTS_D = 5000;
 // SM, 75.7 with 32, 73.4 with 64)
 constexpr int F64_CTAS = 152 * 64;
 
+// scratch that a context keeps: the partial sums of a Fock launch (more than this only
+// where one row of them takes more; it takes rows from d classes, which have few pairs)
+// and the table of rho and cn
+constexpr size_t F64_S_BYTES = (size_t)128 << 20;
+constexpr size_t F64_RC_BYTES = (size_t)1 << 30;
+
 __device__ inline double f64_comp_factor(int l, int c)
 {
     return l == 2 && (c == 1 || c == 2 || c == 4) ? 1.7320508075688772935 : 1.0;
@@ -257,7 +263,7 @@ int f64_prepare(pcm_ctx *c)
     PCM_TRY(f.ord.alloc(n));
     PCM_TRY(f.P.alloc(4 * (size_t)n));
     PCM_TRY(f.info.alloc(n));
-    f.use_rc = c->ncls <= F64_RC_CLASSES;
+    f.use_rc = c->ncls <= F64_RC_CLASSES && (size_t)c->ncls * n * sizeof(double2) <= F64_RC_BYTES;
     if (f.use_rc) PCM_TRY(f.rc.alloc((size_t)c->ncls * n));
     // within a cell by exponent
     bool sorted;
@@ -879,7 +885,8 @@ template <int L>
 static int f64_w_launch(pcm_ctx *c, const F64Pairs &a, int level, const int *ord, double *W)
 {
     const int nb = (a.n + 127) / 128;
-    const int rows = std::max(1, std::min(c->f64.ntile, (F64_CTAS + nb - 1) / nb));
+    const int fit = (int)std::min<size_t>(1 << 20, F64_S_BYTES / (sizeof(double) * far_nterms(L) * a.n));
+    const int rows = std::max(1, std::min({c->f64.ntile, (F64_CTAS + nb - 1) / nb, fit}));
     PCM_TRY(c->f64.S.alloc((size_t)rows * far_nterms(L) * a.n));
     f64_fock_kernel<L><<<dim3(nb, rows), 128, 0, c->stream>>>(a, f64_points(c), c->f64.S.p);
     PCM_LAUNCHED(c);

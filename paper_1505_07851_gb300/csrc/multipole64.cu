@@ -227,6 +227,8 @@ __device__ __forceinline__ double2 mp_power(double x, double y, int m)
     return make_double2(er, ei);
 }
 
+// scratch of the raw sums: the cells go in groups of this much
+constexpr size_t P2M_RAW_BYTES = (size_t)128 << 20;
 constexpr int P2M_NP = 32;                          // pairs per batch, a lane each
 constexpr int P2M_NW = (MP_P + 2) / 2;              // warp w fills columns w and MP_P - w: MP_P + 2 rows each
 constexpr int P2M_NT = 32 * P2M_NW;
@@ -244,7 +246,7 @@ __host__ __device__ constexpr size_t p2m_smem(int L)
 // per (l, m) adds the pairs' terms in pair order.  FP64-bound: about 50 warp
 // instructions per pair for the columns and 13 (2 + 2 (L+1)^2) for the sums.
 template <int L>
-__global__ void __launch_bounds__(P2M_NT) mp_p2m_kernel(int ncell, const int *__restrict__ beg,
+__global__ void __launch_bounds__(P2M_NT) mp_p2m_kernel(const int *__restrict__ beg,
                                                         const int *__restrict__ end, const int *__restrict__ pos,
                                                         int e0, const double *__restrict__ rec,
                                                         const double *__restrict__ B, int nesp,
@@ -541,9 +543,10 @@ __global__ void __launch_bounds__(32 * P2L_NW) mp_p2l_kernel(int M, int ntile, i
 }
 
 // lam: nsplit shares of the cell's tiles, those of a level and the ones above it.
-// Coefficients of V_s = sum_{l, m >= 0} b_l (Re e_m A + Im e_m B) for the sets s
-// = (n, mu, part) of a class: tab[cell][lm][s] = (A, B); one block per cell
-__global__ void __launch_bounds__(P2M_NT) mp_local_kernel(int ns, int nsplit, int ncell,
+// Coefficients of V_s = sum_{l, m >= 0} b_l (Re e_m A + Im e_m B) for ns sets s
+// = (n, mu, part) of a class from s0 on: tab[cell][lm][s - s0] = (A, B); one block per
+// cell
+__global__ void __launch_bounds__(P2M_NT) mp_local_kernel(int s0, int ns, int nsplit, int ncell,
                                                           const double2 *__restrict__ lam, double2 *__restrict__ tab)
 {
     __shared__ double2 L[MP_NLM];
@@ -564,7 +567,7 @@ __global__ void __launch_bounds__(P2M_NT) mp_local_kernel(int ns, int nsplit, in
     if (i >= MP_NLM) return;
     const double h = c_mp.hn[i];
     double2 *o = tab + ((size_t)cell * MP_NLM + i) * ns;
-    for (int s = 0; s < ns; ++s) {
+    for (int s = s0; s < s0 + ns; ++s) {
         int n = 0;
         while ((n + 1) * (n + 1) <= s) ++n;
         const int q = s - n * n, mu = (q + 1) / 2;
@@ -578,11 +581,11 @@ __global__ void __launch_bounds__(P2M_NT) mp_local_kernel(int ns, int nsplit, in
             al = make_double2(a.x + sg * b.x, -a.y + sg * b.y);
             be = make_double2(a.y + sg * b.y, a.x - sg * b.x);   // i (conj(a) - sg b)
         }
-        o[s] = (q == 0 || (q & 1)) ? make_double2(h * al.x, h * be.x) : make_double2(h * al.y, h * be.y);
+        o[s - s0] = (q == 0 || (q & 1)) ? make_double2(h * al.x, h * be.x) : make_double2(h * al.y, h * be.y);
     }
 }
 
-// V[s][pair] for the sets s0 .. s0 + NS of ns: a lane per sorted pair, reading its
+// V[s][pair] for NS sets: a lane per sorted pair, reading its
 // own cell's coefficients (the pairs of a cell follow one another, so a warp reads
 // one cell or a few; taking the cells of a warp in turn instead cost the d classes,
 // with few pairs per cell, five times as much).
@@ -590,8 +593,7 @@ template <int NS>
 __global__ void __launch_bounds__(128) mp_l2p_kernel(int n, int stride, const int *__restrict__ list, int first,
                                                      const double *__restrict__ P, const int *__restrict__ pcell,
                                                      const double *__restrict__ cxyz,
-                                                     const double2 *__restrict__ tab, int ns, int s0,
-                                                     double *__restrict__ V)
+                                                     const double2 *__restrict__ tab, double *__restrict__ V)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const int jj = min(j, n - 1);
@@ -600,7 +602,7 @@ __global__ void __launch_bounds__(128) mp_l2p_kernel(int n, int stride, const in
     const double x = P[pos] - cxyz[3 * cell], y = P[(size_t)stride + pos] - cxyz[3 * cell + 1],
                  z = P[2 * (size_t)stride + pos] - cxyz[3 * cell + 2];
     const double r2 = fma(x, x, fma(y, y, z * z));
-    const double2 *t = tab + (size_t)cell * MP_NLM * ns + s0;
+    const double2 *t = tab + (size_t)cell * MP_NLM * NS;
     double out[NS];
 #pragma unroll
     for (int s = 0; s < NS; ++s) out[s] = 0.0;
@@ -610,7 +612,7 @@ __global__ void __launch_bounds__(128) mp_l2p_kernel(int n, int stride, const in
         double b1 = 1.0, b0 = 0.0, sa[NS], sb[NS];
 #pragma unroll
         for (int s = 0; s < NS; ++s) {
-            const double2 a = __ldg(t + (size_t)(o + m) * ns + s);
+            const double2 a = __ldg(t + (size_t)(o + m) * NS + s);
             sa[s] = a.x;
             sb[s] = a.y;
         }
@@ -618,7 +620,7 @@ __global__ void __launch_bounds__(128) mp_l2p_kernel(int n, int stride, const in
             const double b = fma(z, b1, c_mp.ngam[o + l] * (r2 * b0));
 #pragma unroll
             for (int s = 0; s < NS; ++s) {
-                const double2 a = __ldg(t + (size_t)(o + l) * ns + s);
+                const double2 a = __ldg(t + (size_t)(o + l) * NS + s);
                 sa[s] = fma(b, a.x, sa[s]);
                 sb[s] = fma(b, a.y, sb[s]);
             }
@@ -633,7 +635,7 @@ __global__ void __launch_bounds__(128) mp_l2p_kernel(int n, int stride, const in
     }
     if (j < n)
 #pragma unroll
-        for (int s = 0; s < NS; ++s) V[(size_t)(s0 + s) * n + j] = out[s];
+        for (int s = 0; s < NS; ++s) V[(size_t)s * n + j] = out[s];
 }
 
 // ---------------------------------------------------------------------------
@@ -648,15 +650,21 @@ static int mp_moments_class(pcm_ctx *c, int k, bool first, double2 *M)
     // several blocks share a cell's pairs where a class has many; d classes have few
     const int split = L <= 1 ? 4 : (L == 2 ? 2 : 1);
     static_assert(p2m_smem(L) + 8 <= 227 * 1024, "shared memory");
-    PCM_TRY(mp.raw.alloc((size_t)mp.ncell * split * NS * MP_NLM));
+    const size_t per = (size_t)split * NS * MP_NLM;   // raw sums per cell
+    const int group = (int)std::min<size_t>(mp.ncell, P2M_RAW_BYTES / (per * sizeof(double2)));
+    PCM_TRY(mp.raw.alloc(group * per));
     PCM_CUDA(cudaFuncSetAttribute(mp_p2m_kernel<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)p2m_smem(L) + 8));
-    mp_p2m_kernel<L><<<dim3(mp.ncell, split), P2M_NT, p2m_smem(L) + 8, c->stream>>>(
-        mp.ncell, mp.range.p + (size_t)k * mp.ncell, mp.range.p + (size_t)(6 + k) * mp.ncell, f.pos.p, f.eoff[k],
-        f.rec.p + f.roff[k], f.B.p + f.boff[k], c->cls[k].nesp, mp.cxyz.p, mp.raw.p);
-    PCM_LAUNCHED(c);
-    mp_combine_kernel<L><<<mp.ncell, P2M_NT, 0, c->stream>>>(split, first, mp.raw.p, M);
-    PCM_LAUNCHED(c);
+    for (int c0 = 0; c0 < mp.ncell; c0 += group) {
+        const int nc = std::min(group, mp.ncell - c0);
+        const int *beg = mp.range.p + (size_t)k * mp.ncell + c0, *end = mp.range.p + (size_t)(6 + k) * mp.ncell + c0;
+        mp_p2m_kernel<L><<<dim3(nc, split), P2M_NT, p2m_smem(L) + 8, c->stream>>>(
+            beg, end, f.pos.p, f.eoff[k], f.rec.p + f.roff[k], f.B.p + f.boff[k], c->cls[k].nesp,
+            mp.cxyz.p + 3 * (size_t)c0, mp.raw.p);
+        PCM_LAUNCHED(c);
+        mp_combine_kernel<L><<<nc, P2M_NT, 0, c->stream>>>(split, first, mp.raw.p, M + (size_t)c0 * MP_NLM);
+        PCM_LAUNCHED(c);
+    }
     return PCM_OK;
 }
 
@@ -719,20 +727,21 @@ int mp_l2p(pcm_ctx *c, int level, int L, int n, const int *list, int first)
     F64Mp &mp = f.mp;
     const int ns = (L + 1) * (L + 1);
     PCM_TRY(mp.V.alloc((size_t)ns * n));
-    PCM_TRY(mp.tab.alloc((size_t)mp.ncell * MP_NLM * ns));
-    mp_local_kernel<<<mp.ncell, P2M_NT, 0, c->stream>>>(ns, (MP_LEVELS - level) * mp.lsplit, mp.ncell,
-                                                        mp.lam.p + (size_t)level * mp.lsplit * mp.ncell * MP_NLM,
-                                                        mp.tab.p);
-    PCM_LAUNCHED(c);
+    PCM_TRY(mp.tab.alloc((size_t)mp.ncell * MP_NLM * std::min(ns, 9)));
     const int nb = (n + 127) / 128;
     const int *pc = mp.pcell.p;
 #define PCM_L2P(N, S0)                                                                                            \
     do {                                                                                                          \
-        mp_l2p_kernel<N><<<nb, 128, 0, c->stream>>>(n, f.off[6], list, first, f.P.p, pc, mp.cxyz.p, mp.tab.p, ns, \
-                                                    S0, mp.V.p);                                                 \
+        mp_local_kernel<<<mp.ncell, P2M_NT, 0, c->stream>>>(                                                      \
+            S0, N, (MP_LEVELS - level) * mp.lsplit, mp.ncell,                                                     \
+            mp.lam.p + (size_t)level * mp.lsplit * mp.ncell * MP_NLM, mp.tab.p);                                  \
+        PCM_LAUNCHED(c);                                                                                          \
+        mp_l2p_kernel<N><<<nb, 128, 0, c->stream>>>(n, f.off[6], list, first, f.P.p, pc, mp.cxyz.p, mp.tab.p,     \
+                                                    mp.V.p + (size_t)(S0) * n);                                   \
         PCM_LAUNCHED(c);                                                                                          \
     } while (0)
-    // at most nine sets per launch, so that their sums stay in registers
+    // at most nine sets per launch, so that their sums stay in registers and their
+    // coefficients take 71 KB per cell
     switch (L) {
     case 0: PCM_L2P(1, 0); break;
     case 1: PCM_L2P(4, 0); break;
