@@ -972,7 +972,10 @@ static int esp_ms_launch(pcm_ctx *c, PairClass &pc, int k, const int *blk, const
 // Point blocks by which the packed variants cut a class's pairs into segments: the
 // same for 4 and 2 points per thread, so that the autotuner's choice between them,
 // which goes by the clock, does not change the sums.  2 points per thread, and 4 for
-// the s pairs of tuned batches (the usual choice there).
+// the s pairs of tuned batches: half the point blocks is twice the segments, each
+// with its own sums, and other segments would move the batches' potentials in
+// their last FP32 bits (their charges by 1e-6).  Computed before the autotuner's
+// trials, which run outside the batch's launch, so that they time what will run.
 static int packed_plan_blocks(const pcm_ctx *c, int k, const int nb[2])
 {
     return c->jobs && c->opt.autotune && CLASS_L[k] == 0 ? nb[0] : nb[1];
@@ -980,11 +983,11 @@ static int packed_plan_blocks(const pcm_ctx *c, int k, const int nb[2])
 
 // Variants of the FP32 ESP: pair-driven with 4 (v = 0) or 2 (v = 1) points per
 // thread (two pairs per packed instruction unless the context asks for scalar
-// FP32 instructions); MS-driven (v = 2).
-static int esp_launch_variant(pcm_ctx *c, int k, int v, DBuf<int> *blk, DBuf<int> *bcls, const int nb[2], double *part)
+// FP32 instructions); MS-driven (v = 2).  np: the packed variants' plan.
+static int esp_launch_variant(pcm_ctx *c, int k, int v, DBuf<int> *blk, DBuf<int> *bcls, const int nb[2], int np,
+                              double *part)
 {
     PairClass &pc = c->cls[k];
-    const int np = packed_plan_blocks(c, k, nb);
     if (v == 2) {
         const int d = esp_default_ppt(CLASS_L[k], false) == 4 ? 0 : 1;
         switch (CLASS_L[k]) {
@@ -1021,9 +1024,9 @@ static int esp_rows(pcm_ctx *c, int k, int nblk)
 }
 
 // partial-sum rows of variant v of class k
-static int esp_rows_v(pcm_ctx *c, int k, int v, const int nb[2])
+static int esp_rows_v(pcm_ctx *c, int k, int v, const int nb[2], int np)
 {
-    if (v < 2) return esp_rows(c, k, c->opt.fp32x2 ? packed_plan_blocks(c, k, nb) : nb[v]);
+    if (v < 2) return esp_rows(c, k, c->opt.fp32x2 ? np : nb[v]);
     const int d = esp_default_ppt(CLASS_L[k], false) == 4 ? 0 : 1;
     int sl, r1, mrows, ns, ks;
     esp_plan(c->cls[k].nesp_same, nb[d], &sl, &r1);
@@ -1034,7 +1037,7 @@ static int esp_rows_v(pcm_ctx *c, int k, int v, const int nb[2])
 // The autotuner's trial for class k: every candidate run once untimed, then
 // once timed with CUDA events on the context's stream; the fastest is
 // remembered for this GPU, kernel family, angular momentum and size bucket.
-static int esp_tune(pcm_ctx *c, int k, DBuf<int> *blk, DBuf<int> *bcls, const int nb[2], int *choice)
+static int esp_tune(pcm_ctx *c, int k, DBuf<int> *blk, DBuf<int> *bcls, const int nb[2], int np, int *choice)
 {
     // a batch member: its packed blocks join one launch with every other
     // molecule's, so only the packed layouts are candidates (their own record)
@@ -1056,11 +1059,11 @@ static int esp_tune(pcm_ctx *c, int k, DBuf<int> *blk, DBuf<int> *bcls, const in
     // candidates: pair-driven with 4 or 2 points per thread; MS-driven for L <= 2 (not in batches)
     const int nv = (L <= 2 && !batching) ? 3 : 2;
     int rmax = 1;
-    for (int v = 0; v < nv; ++v) rmax = std::max(rmax, esp_rows_v(c, k, v, nb));
+    for (int v = 0; v < nv; ++v) rmax = std::max(rmax, esp_rows_v(c, k, v, nb, np));
     PCM_TRY(c->esp_part.alloc((size_t)rmax * c->M));
     // one untimed pass first: the first launch of a variant also allocates
     // its tile buffers and loads its code, which is not what it costs per call
-    for (int v = 0; v < nv; ++v) PCM_TRY(esp_launch_variant(c, k, v, blk, bcls, nb, c->esp_part.p));
+    for (int v = 0; v < nv; ++v) PCM_TRY(esp_launch_variant(c, k, v, blk, bcls, nb, np, c->esp_part.p));
     PCM_CUDA(cudaStreamSynchronize(c->stream));
     cudaEvent_t e[4];
     for (int i = 0; i <= nv; ++i) PCM_CUDA(cudaEventCreate(&e[i]));
@@ -1068,7 +1071,7 @@ static int esp_tune(pcm_ctx *c, int k, DBuf<int> *blk, DBuf<int> *bcls, const in
     int st = PCM_OK;
     PCM_CUDA(cudaEventRecord(e[0], c->stream));
     for (int v = 0; v < nv && st == PCM_OK; ++v) {
-        st = esp_launch_variant(c, k, v, blk, bcls, nb, c->esp_part.p);
+        st = esp_launch_variant(c, k, v, blk, bcls, nb, np, c->esp_part.p);
         if (st == PCM_OK) PCM_CUDA(cudaEventRecord(e[v + 1], c->stream));
     }
     if (st == PCM_OK) {
@@ -1090,15 +1093,16 @@ int esp_compute_mixed(pcm_ctx *c, double *dc)
     int nb[2];
     PCM_TRY(mixed_point_blocks(c, nb));
     DBuf<int> *blk = &c->si[4], *bcls = &c->si[6];  // blk[0..1], bcls[0..1]
-    int var[6], rows[6], total = 0;
+    int var[6], rows[6], plan[6], total = 0;
     for (int k = 0; k < 6; ++k) {
+        plan[k] = packed_plan_blocks(c, k, nb);
         var[k] = esp_default_ppt(CLASS_L[k], c->opt.fp32x2) == 4 ? 0 : 1;
         if (c->opt.esp_variant >= 0) {
             if (c->opt.esp_variant < 2 || CLASS_L[k] <= 2) var[k] = c->opt.esp_variant;
         } else if (c->opt.autotune && c->cls[k].nesp > 0) {
-            PCM_TRY(esp_tune(c, k, blk, bcls, nb, &var[k]));
+            PCM_TRY(esp_tune(c, k, blk, bcls, nb, plan[k], &var[k]));
         }
-        rows[k] = c->cls[k].nesp > 0 ? esp_rows_v(c, k, var[k], nb) : 0;
+        rows[k] = c->cls[k].nesp > 0 ? esp_rows_v(c, k, var[k], nb, plan[k]) : 0;
         total += rows[k];
     }
     if (total == 0) {
@@ -1113,7 +1117,8 @@ int esp_compute_mixed(pcm_ctx *c, double *dc)
     int base = 0;
     for (int k = 0; k < 6; ++k) {
         if (c->cls[k].nesp == 0) continue;
-        PCM_TRY(esp_launch_variant(c, k, var[k], blk, bcls, nb, c->esp_part.p + (size_t)base * c->M));
+        PCM_TRY(esp_launch_variant(c, k, var[k], blk, bcls, nb, plan[k],
+                                   c->esp_part.p + (size_t)base * c->M));
         base += rows[k];
     }
     c->esp_total_rows = total;
