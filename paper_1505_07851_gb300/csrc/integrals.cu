@@ -590,7 +590,6 @@ __global__ void esp_bounds_kernel(EspBounds b, const int *__restrict__ list, con
 template <int LA, int LB>
 static int esp_flag_class(pcm_ctx *c, PairClass &pc, const double *dP, unsigned char *flag)
 {
-    pc.nesp = pc.nesp_same = 0;
     if (pc.npair == 0) return PCM_OK;
     esp_flag_kernel<LA, LB><<<(pc.npair + 127) / 128, 128, 0, c->stream>>>(
         pc.npair, pc.sp.p, pc.ia.p, pc.ib.p, pc.spA.p, pc.spB.p, c->sh_bf.p, c->sh_atom.p, pc.Q.p, dP, c->nbf,
@@ -629,50 +628,75 @@ static int esp_class_stats(pcm_ctx *c)
     return PCM_OK;
 }
 
-// Density test and Hermite density coefficients of every class; in each class the
-// same-atom pairs come first, then the others, each in pair order.  One compaction
-// over the flags of all classes and one synchronisation for their counts.
-int esp_prepare_all(pcm_ctx *c, const double *dP)
+// Density test and Hermite density coefficients of the classes [k0, k1); in each class
+// the same-atom pairs come first, then the others, each in pair order.  One compaction
+// over the flags of these classes and one synchronisation for their counts.
+static int esp_prepare_classes(pcm_ctx *c, const double *dP, int k0, int k1)
 {
     EspBounds b;
     long long n = 0;
     for (int k = 0; k < 6; ++k) {
+        const int m = k >= k0 && k < k1 ? c->cls[k].npair : 0;
         b.at[2 * k] = (int)n;
-        b.at[2 * k + 1] = (int)n + c->cls[k].npair;
-        n += 2LL * c->cls[k].npair;
+        b.at[2 * k + 1] = (int)(n + m);
+        n += 2LL * m;
     }
     b.at[12] = (int)n;
-    if (n >= (1LL << 31)) {
-        set_last_error("too many primitive pairs");
-        return PCM_ERR_UNSUPPORTED;
-    }
-    PCM_TRY(c->flags8.alloc(std::max(1LL, n)));
-    PCM_TRY(c->idx32.alloc(std::max(1LL, n)));
-    unsigned char *f = c->flags8.p;
-    PCM_TRY((esp_flag_class<0, 0>(c, c->cls[0], dP, f + b.at[0])));
-    PCM_TRY((esp_flag_class<1, 0>(c, c->cls[1], dP, f + b.at[2])));
-    PCM_TRY((esp_flag_class<1, 1>(c, c->cls[2], dP, f + b.at[4])));
-    PCM_TRY((esp_flag_class<2, 0>(c, c->cls[3], dP, f + b.at[6])));
-    PCM_TRY((esp_flag_class<2, 1>(c, c->cls[4], dP, f + b.at[8])));
-    PCM_TRY((esp_flag_class<2, 2>(c, c->cls[5], dP, f + b.at[10])));
     if (n == 0) return PCM_OK;
+    PCM_TRY(c->flags8.alloc(n));
+    PCM_TRY(c->idx32.alloc(n));
+    unsigned char *f = c->flags8.p;
+    for (int k = k0; k < k1; ++k) {
+        unsigned char *fk = f + b.at[2 * k];
+        switch (k) {
+        case 0: PCM_TRY((esp_flag_class<0, 0>(c, c->cls[k], dP, fk))); break;
+        case 1: PCM_TRY((esp_flag_class<1, 0>(c, c->cls[k], dP, fk))); break;
+        case 2: PCM_TRY((esp_flag_class<1, 1>(c, c->cls[k], dP, fk))); break;
+        case 3: PCM_TRY((esp_flag_class<2, 0>(c, c->cls[k], dP, fk))); break;
+        case 4: PCM_TRY((esp_flag_class<2, 1>(c, c->cls[k], dP, fk))); break;
+        case 5: PCM_TRY((esp_flag_class<2, 2>(c, c->cls[k], dP, fk))); break;
+        }
+    }
     int first[13];
     PCM_TRY(compact_flags(c, f, n, c->idx32.p, nullptr, c->iscal.p + 16));
     esp_bounds_kernel<<<1, 32, 0, c->stream>>>(b, c->idx32.p, c->iscal.p + 16, c->iscal.p);
     PCM_LAUNCHED(c);
     PCM_CUDA(cudaMemcpyAsync(first, c->iscal.p, sizeof(first), cudaMemcpyDeviceToHost, c->stream));
     PCM_CUDA(cudaStreamSynchronize(c->stream));
-    for (int k = 0; k < 6; ++k) {
-        c->cls[k].nesp_same = first[2 * k + 1] - first[2 * k];
-        c->cls[k].nesp = first[2 * k + 2] - first[2 * k];
+    for (int k = k0; k < k1; ++k) {
+        PairClass &pc = c->cls[k];
+        pc.nesp_same = first[2 * k + 1] - first[2 * k];
+        pc.nesp = first[2 * k + 2] - first[2 * k];
+        const int *l = c->idx32.p + first[2 * k];
+        const int base = b.at[2 * k];
+        switch (k) {
+        case 0: PCM_TRY((esp_coef_class<0, 0>(c, pc, dP, l, base))); break;
+        case 1: PCM_TRY((esp_coef_class<1, 0>(c, pc, dP, l, base))); break;
+        case 2: PCM_TRY((esp_coef_class<1, 1>(c, pc, dP, l, base))); break;
+        case 3: PCM_TRY((esp_coef_class<2, 0>(c, pc, dP, l, base))); break;
+        case 4: PCM_TRY((esp_coef_class<2, 1>(c, pc, dP, l, base))); break;
+        case 5: PCM_TRY((esp_coef_class<2, 2>(c, pc, dP, l, base))); break;
+        }
     }
-    const int *l = c->idx32.p;
-    PCM_TRY((esp_coef_class<0, 0>(c, c->cls[0], dP, l + first[0], b.at[0])));
-    PCM_TRY((esp_coef_class<1, 0>(c, c->cls[1], dP, l + first[2], b.at[2])));
-    PCM_TRY((esp_coef_class<1, 1>(c, c->cls[2], dP, l + first[4], b.at[4])));
-    PCM_TRY((esp_coef_class<2, 0>(c, c->cls[3], dP, l + first[6], b.at[6])));
-    PCM_TRY((esp_coef_class<2, 1>(c, c->cls[4], dP, l + first[8], b.at[8])));
-    PCM_TRY((esp_coef_class<2, 2>(c, c->cls[5], dP, l + first[10], b.at[10])));
+    return PCM_OK;
+}
+
+// the same for every class: all classes at once while their flags can be numbered in 31
+// bits, else in groups that can
+int esp_prepare_all(pcm_ctx *c, const double *dP)
+{
+    for (auto &pc : c->cls) pc.nesp = pc.nesp_same = 0;
+    for (int k0 = 0; k0 < 6;) {
+        long long n = 2LL * c->cls[k0].npair;
+        if (n >= (1LL << 31)) {
+            set_last_error("too many primitive pairs");
+            return PCM_ERR_UNSUPPORTED;
+        }
+        int k1 = k0 + 1;
+        while (k1 < 6 && n + 2LL * c->cls[k1].npair < (1LL << 31)) n += 2LL * c->cls[k1++].npair;
+        PCM_TRY(esp_prepare_classes(c, dP, k0, k1));
+        k0 = k1;
+    }
     return PCM_OK;
 }
 
