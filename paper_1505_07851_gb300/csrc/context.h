@@ -63,6 +63,7 @@ struct DBuf {
         cudaError_t e = cudaMalloc((void **)&p, count * sizeof(T));
         if (e != cudaSuccess) {
             p = nullptr;
+            cudaGetLastError();   // reported here, not by the next launch
             set_last_error("cudaMalloc(%zu bytes): %s", count * sizeof(T), cudaGetErrorString(e));
             return e == cudaErrorMemoryAllocation ? PCM_ERR_OOM : PCM_ERR_CUDA;
         }

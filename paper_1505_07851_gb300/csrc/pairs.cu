@@ -414,12 +414,9 @@ static int screen_classes(pcm_ctx *c, int k0, int k1)
 int basis_build(pcm_ctx *c, int nshell, const int *shell_atom, const int *shell_l, const int *shell_nprim,
                 const double *exps, const double *coefs)
 {
-    // expand sp shells into an s and a p shell that share exponents
-    c->h_sh_atom.clear();
-    c->h_sh_l.clear();
-    c->h_sh_nprim.clear();
-    c->h_sh_off.clear();
-    c->h_sh_bf.clear();
+    // expand sp shells into an s and a p shell that share exponents; a basis that is
+    // refused here leaves the context's own as it was
+    std::vector<int> sh_atom, sh_l, sh_nprim, sh_off, sh_bf;
     std::vector<double> ex, co;
     int off = 0, coff = 0, bf = 0;
     for (int s = 0; s < nshell; ++s) {
@@ -440,11 +437,11 @@ int basis_build(pcm_ctx *c, int nshell, const int *shell_atom, const int *shell_
         const int nparts = (l == -1) ? 2 : 1;
         for (int part = 0; part < nparts; ++part) {
             const int ll = (l == -1) ? part : l;
-            c->h_sh_atom.push_back(shell_atom[s]);
-            c->h_sh_l.push_back(ll);
-            c->h_sh_nprim.push_back(n);
-            c->h_sh_off.push_back((int)ex.size());
-            c->h_sh_bf.push_back(bf);
+            sh_atom.push_back(shell_atom[s]);
+            sh_l.push_back(ll);
+            sh_nprim.push_back(n);
+            sh_off.push_back((int)ex.size());
+            sh_bf.push_back(bf);
             for (int i = 0; i < n; ++i) {
                 ex.push_back(exps[off + i]);
                 const double cf = coefs[coff + part * n + i];
@@ -459,8 +456,14 @@ int basis_build(pcm_ctx *c, int nshell, const int *shell_atom, const int *shell_
         off += n;
         coff += nparts * n;
     }
+    c->h_sh_atom.swap(sh_atom);
+    c->h_sh_l.swap(sh_l);
+    c->h_sh_nprim.swap(sh_nprim);
+    c->h_sh_off.swap(sh_off);
+    c->h_sh_bf.swap(sh_bf);
     c->nshell = (int)c->h_sh_l.size();
-    c->nbf = bf;
+    c->nbf = 0;                            // no basis until all of it is in place
+    c->fock_ord.on = false;
     const int ns = c->nshell;
     PCM_TRY(c->sh_atom.alloc(ns));
     PCM_TRY(c->sh_l.alloc(ns));
@@ -554,13 +557,16 @@ int basis_build(pcm_ctx *c, int nshell, const int *shell_atom, const int *shell_
         c->pl_nprim = c->h_sh_nprim;
         c->pair_layout_ok = true;
     }
-    if (c->opt.precision == PCM_FP64) return f64_prepare(c);
-    c->fock_ord.on = false;
-    if (!c->opt.fp32x2) return PCM_OK;
-    int first[7];
-    const float *x32[6];
-    for (int k = 0; k < 6; ++k) x32[k] = c->cls[k].Pxyz32.p;
-    return fock_order(c, kept_pairs(c, first), x32, c->fock_ord);
+    if (c->opt.precision == PCM_FP64) {
+        PCM_TRY(f64_prepare(c));
+    } else if (c->opt.fp32x2) {
+        int first[7];
+        const float *x32[6];
+        for (int k = 0; k < 6; ++k) x32[k] = c->cls[k].Pxyz32.p;
+        PCM_TRY(fock_order(c, kept_pairs(c, first), x32, c->fock_ord));
+    }
+    c->nbf = bf;
+    return PCM_OK;
 }
 
 }  // namespace pcm
