@@ -243,8 +243,8 @@ __host__ __device__ constexpr size_t p2m_smem(int L)
 // Raw sums of one class over a cell's ESP pairs: raw[cell][split][s][lm] (re, im)
 // = sum B_s b_l (x + iy)^m.  A batch of 32 pairs: the warps fill b in shared
 // memory (columns paired so that every warp has the same rows), then a thread
-// per (l, m) adds the pairs' terms in pair order.  FP64-bound: about 50 warp
-// instructions per pair for the columns and 13 (2 + 2 (L+1)^2) for the sums.
+// per (l, m) adds the pairs' terms in pair order.  FP64-bound: about 60 warp
+// instructions per pair for the columns and 16 (2 + 2 (L+1)^2) for the sums.
 template <int L>
 __global__ void __launch_bounds__(P2M_NT) mp_p2m_kernel(const int *__restrict__ beg,
                                                         const int *__restrict__ end, const int *__restrict__ pos,
