@@ -31,9 +31,13 @@ namespace pcm {
 
 constexpr int F64_LSUM[6] = {0, 1, 2, 2, 3, 4};
 constexpr int F64_SORT_POINTS = 1024;     // fewer points than this stay in library order
-// side of a cell (bohr).  2.5 / 3.0: Fock correction of 150 s/sp atoms 28.5 / 29.4 ms, of 300
-// 92.2 / 88.9, gradient of 150 83.0 / 90.3, of 180 s/p/d atoms 170 / 179 (2.0: 30.6, 104.8, 83.8, 173)
-constexpr double F64_CELL = 2.5;
+// side of a cell (bohr): expansions cost cells times points, direct interactions go by the
+// cells' volume, so larger molecules take larger cells.  2.5 / 3.0 / 3.6, Fock correction and
+// gradient: 200 s/sp atoms (8.4k points) 47.6 / 47.2 / 51.2 and 131 / 139 / 156 ms, 300 s/p/d
+// (11.8k) 132 / 130 / 143 and 365 / 388 / 452, 550 s/p/d (23.5k) 388 / 347 / 350 and 1001 / 970 /
+// 1071, 1000 s/p/d (43.5k) 1102 / 931 / 864 and 2696 / 2463 / 2552
+constexpr double F64_CELL = 2.5, F64_CELL_LARGE = 3.0;
+constexpr int F64_CELL_POINTS = 16000;    // from this many points on the larger one
 constexpr int F64_PTBITS = 6;             // cells per side of the points' grid
 constexpr int F64_RC_CLASSES = 16;        // up to this many exponent classes rho and cn are tabulated per (class, pair)
 // From this many pairs and points on the cells' expansions are used: setting them up costs
@@ -235,7 +239,7 @@ int f64_prepare(pcm_ctx *c)
 {
     F64Int &f = c->f64;
     const int M = c->M;
-    const F64Box box = f.box = cavity_box(c, F64_CELL);
+    const F64Box box = f.box = cavity_box(c, M < F64_CELL_POINTS ? F64_CELL : F64_CELL_LARGE);
     const F64Src src = kept_pairs(c, f.off);
     const int n = f.off[6];
     f.ntile = (M + 31) / 32;
