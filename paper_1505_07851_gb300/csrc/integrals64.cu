@@ -50,8 +50,8 @@ constexpr int F64_MP_PAIRS = 40000;
 constexpr int F64_MP_POINTS = 3500;
 constexpr int F64_MP_POINTS_D = 5000;
 // thread blocks that a launch aims at: many more than fit, so that blocks with few
-// expanded cells and blocks with many even out (300-atom Fock: 82.9 ms with 16 per
-// SM, 75.7 with 32, 73.4 with 64)
+// expanded cells and blocks with many even out (Fock correction of 300 s/sp atoms 100.8 ms
+// with 16 per SM, 94.7 with 32, 91.6 with 64; gradient of 180 s/p/d atoms 180, 173, 169)
 constexpr int F64_CTAS = 152 * 64;
 
 // scratch that a context keeps: the partial sums of a Fock launch (more than this only
